@@ -169,13 +169,7 @@ constexpr size_t kSingleSmemCap = 110 * 1024;
 
 int pick_threads(int m, int n, int k, int requested) {
     if (requested > 0) return std::min(std::max(32, (requested + 31) / 32 * 32), lpb::kMaxThreads);
-    const int64_t e = (int64_t)(m + 1 + (k > 0)) * (n + k + 1);
-    // measured best on GB300 (mixed-sign dense m x m, m = 20..100)
-    if (e <= 1024) return 32;
-    if (e <= 3072) return 64;
-    if (e <= 8192) return 128;
-    if (e <= 32768) return 256;
-    return 512;
+    return lpb::resident_threads(m, n, k);
 }
 
 // Threads per CTA of the mixed-precision kernel; 0 requested = from the
@@ -213,13 +207,18 @@ struct lp_batch {
     bool solved = false;
     int32_t num_phase1 = 0;
     size_t max_smem = 0;
-    // streamed LPs: order[streamed_offset ...), persistent CTAs over slots
-    int64_t streamed_offset = 0;
+    // FP64 LPs with deferred updates and a global workspace slot, one group per
+    // size class: order[offset ...), persistent CTAs over slots
+    struct DeferredGroup {
+        lpb::DeferredForm form;
+        int64_t offset;
+        int32_t count, slots;
+        size_t slot_bytes;
+        unsigned char* workspace;
+        int32_t* counter;
+    };
+    std::vector<DeferredGroup> deferred_groups;
     int32_t num_streamed = 0;
-    int32_t streamed_slots = 0;
-    size_t slot_bytes = 0;
-    unsigned char* workspace = nullptr;
-    int32_t* counter = nullptr;
     // mixed precision: groups of the FP32 + certificate kernel, fallback queue
     std::vector<Group> mixed_groups;
     int32_t num_mixed = 0;
@@ -245,17 +244,18 @@ struct lp_batch {
     size_t mslot_bytes = 0;
     unsigned char* mworkspace = nullptr;
     int32_t* mcounter = nullptr;
-    // FP64 streamed re-solve of uncertified mixed LPs whose FP64 tableau
-    // exceeds one CTA
+    // FP64 re-solve of uncertified mixed LPs whose FP64 tableau exceeds one
+    // CTA: with deferred updates
     int32_t num_fbig = 0;
     int32_t* fbig_queue = nullptr;
     int32_t* fbig_len = nullptr;
     int32_t* fbig_counter = nullptr;
     int32_t fbig_slots = 0;
     size_t fbig_slot_bytes = 0;
+    lpb::DeferredForm fbig_form{};
     unsigned char* fbig_workspace = nullptr;
     // ... on thread-block clusters of fbig_C CTAs when every such LP fits one
-    // (0: on the streamed kernel)
+    // (0: on the deferred-update kernel)
     int fbig_C = 0, fbig_clusters = 0;
     size_t fbig_cluster_smem = 0;
     // optional stage timing: event triples (start, groups joined, re-solve
@@ -372,17 +372,22 @@ lpb_err enqueue_solve(lp_batch* h, cudaStream_t s, bool timing) {
     if (h->num_mixed > 0 && ((err = cudaMemsetAsync(h->fb_len, 0, sizeof(int32_t), s)) ||
                              (err = cudaMemsetAsync(h->fbig_len, 0, sizeof(int32_t), s))))
         return cuda_fail(err, "fallback queue reset");
-    // kind 0 mixed, 1 resident, 2 streamed, 3 cluster, 4 mixed streamed
+    // kind 0 mixed, 1 resident, 2 deferred updates, 3 cluster, 4 mixed streamed
     struct Job { int kind; const Group* g; int64_t count; };
     std::vector<Job> jobs;
     for (const Group& g : h->mixed_groups) jobs.push_back({0, &g, g.count});
     for (const Group& g : h->groups) jobs.push_back({1, &g, g.count});
-    if (h->num_streamed > 0) jobs.push_back({2, nullptr, h->num_streamed});
+    for (auto it = h->deferred_groups.rbegin(); it != h->deferred_groups.rend(); ++it)  // largest LPs first
+        jobs.push_back({2, reinterpret_cast<const Group*>(&*it), it->count});
     if (h->num_single > 0) jobs.push_back({5, nullptr, h->num_single});
     if (h->num_mstream > 0) jobs.push_back({4, nullptr, h->num_mstream});
     for (size_t ci = 0; ci < h->cluster_groups.size(); ++ci)
         jobs.push_back({3, reinterpret_cast<const Group*>(ci), h->cluster_groups[ci].count});
-    std::stable_sort(jobs.begin(), jobs.end(), [](const Job& a, const Job& b) { return a.count > b.count; });
+    // the deferred-update groups first: they hold the largest LPs
+    std::stable_sort(jobs.begin(), jobs.end(), [](const Job& a, const Job& b) {
+        if ((a.kind == 2) != (b.kind == 2)) return a.kind == 2;
+        return a.kind != 2 && a.count > b.count;
+    });
     cudaEvent_t* tev = (!timing || h->tev.empty()) ? nullptr : &h->tev[3 * (size_t)(h->timed_solves % kTimingRing)];
     if (tev && (err = cudaEventRecord(tev[0], s))) return cuda_fail(err, "timing");
     if ((err = cudaEventRecord(h->ev_fork, s))) return cuda_fail(err, "fork");
@@ -405,8 +410,9 @@ lpb_err enqueue_solve(lp_batch* h, cudaStream_t s, bool timing) {
                                           h->single_ctas, h->single_smem, h->single_workspace, h->single_slot_bytes,
                                           h->single_counter, h->diag, ls);
         } else if (j.kind == 2) {
-            err = lpb::launch_fp64_streamed(h->d, h->tol, h->d_order + h->streamed_offset, h->num_streamed,
-                                            h->streamed_slots, h->workspace, h->slot_bytes, h->counter, h->diag, ls);
+            const auto& dg = *reinterpret_cast<const lp_batch::DeferredGroup*>(j.g);
+            err = lpb::launch_fp64_deferred(h->d, h->tol, h->d_order + dg.offset, dg.count, dg.form, dg.slots,
+                                            dg.workspace, dg.slot_bytes, dg.counter, h->diag, ls);
         } else if (j.kind == 4) {
             err = lpb::launch_mixed_streamed(h->d, h->tol, h->mp, h->d_order + h->mstream_offset, h->num_mstream,
                                              h->mstream_slots, h->mworkspace, h->mslot_bytes, h->mcounter,
@@ -437,7 +443,7 @@ lpb_err enqueue_solve(lp_batch* h, cudaStream_t s, bool timing) {
             err = lpb::launch_fp64_cluster(h->d, h->tol, h->fbig_queue, h->num_fbig, h->fbig_C, h->fbig_clusters,
                                            h->fbig_cluster_smem, h->fbig_counter, h->diag, s, h->fbig_len);
         else
-            err = lpb::launch_fp64_streamed(h->d, h->tol, h->fbig_queue, h->num_fbig, h->fbig_slots,
+            err = lpb::launch_fp64_deferred(h->d, h->tol, h->fbig_queue, h->num_fbig, h->fbig_form, h->fbig_slots,
                                             h->fbig_workspace, h->fbig_slot_bytes, h->fbig_counter, h->diag, s,
                                             h->fbig_len);
         if (err != cudaSuccess) return cuda_fail(err, "fallback launch");
@@ -625,7 +631,8 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
     // (threads per CTA, footprint rounded up to 4 KiB), one launch per group;
     // the others go to the streamed kernel (global workspace slots).
     std::map<std::pair<int, size_t>, std::vector<int32_t>> buckets, mixed_buckets;
-    std::vector<int32_t> streamed;
+    std::vector<int32_t> deferred[lpb::kDeferredClasses];  // deferred updates, by size class
+    auto defer = [&](int32_t k) { deferred[lpb::deferred_form(hm[k], hn[k], hk[k]).cls].push_back(k); };
     std::map<int, std::vector<int32_t>> cluster_buckets;  // cluster size -> LPs
     std::vector<int32_t> mstream;                         // mixed precision, tableau in global memory
     std::vector<int32_t> fbig_lps;                        // mixed LPs whose FP64 re-solve exceeds one CTA
@@ -655,7 +662,9 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
                 h->fb_threads = std::max({h->fb_threads, pick_threads(hm[k], hn[k], hk[k], 0), 256});
             } else {
                 ++h->num_fbig;
-                h->fbig_slot_bytes = std::max(h->fbig_slot_bytes, lpb::streamed_slot_bytes(hm[k], hn[k], hk[k]));
+                h->fbig_slot_bytes = std::max(h->fbig_slot_bytes, lpb::deferred_slot(hm[k], hn[k], hk[k]).total);
+                const lpb::DeferredForm f = lpb::deferred_form(hm[k], hn[k], hk[k]);
+                if (fbig_lps.empty() || f.cls > h->fbig_form.cls) h->fbig_form = f;
                 fbig_lps.push_back(k);
             }
             const size_t mneed = lpb::mixed_smem_bytes(hm[k], hn[k], hk[k]);
@@ -710,13 +719,13 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
                 h->single_smem = std::max(h->single_smem, need);
             } else {
                 ++h->num_single_streamed;
-                h->single_slot_bytes = std::max(h->single_slot_bytes, lpb::streamed_slot_bytes(hm[k], hn[k], hk[k]));
+                h->single_slot_bytes = std::max(h->single_slot_bytes, lpb::deferred_slot(hm[k], hn[k], hk[k]).total);
             }
             continue;
         }
-        // (measured on GB300: the streamed kernel, 304 LPs at once, beats the
-        // clusters, ~50 LPs at once, on every large-LP workload tried --
-        // 1.04-1.34x, more with more pivots -- so clusters are on request)
+        // (measured on GB300: clusters, ~50 LPs at once, were slower than one
+        // CTA per LP with the tableau in a workspace slot on every large-LP
+        // workload tried, so clusters are on request)
         if (need > lpb::kMaxSmemPerBlock && o.schedule == LPB_SCHED_CLUSTER) {
             // the smallest cluster whose CTAs hold the tableau's rows
             int C = 0;
@@ -727,9 +736,8 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
                 continue;
             }
         }
-        if (need > lpb::kMaxSmemPerBlock || o.schedule == LPB_SCHED_STREAMED) {
-            streamed.push_back(k);
-            h->slot_bytes = std::max(h->slot_bytes, lpb::streamed_slot_bytes(hm[k], hn[k], hk[k]));
+        if (o.schedule == LPB_SCHED_STREAMED || lpb::defer_updates(hm[k], hn[k], hk[k])) {
+            defer(k);
             continue;
         }
         const size_t smem = std::min(lpb::kMaxSmemPerBlock, (need + 4095) / 4096 * 4096);
@@ -750,7 +758,6 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
     };
     for (auto& kv : buckets) lpt(kv.second);
     for (auto& kv : mixed_buckets) lpt(kv.second);
-    lpt(streamed);
     std::vector<int32_t> order;
     order.reserve(num_lps);
     for (auto& kv : buckets) {
@@ -787,7 +794,7 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
                 return bail_cuda(err, "group counters");
         }
     }
-    // cluster groups (a cluster shape that cannot be placed goes to the streamed kernel)
+    // cluster groups (a cluster shape that cannot be placed gets deferred updates)
     for (auto& kv : cluster_buckets) {
         const int C = kv.first;
         lpt(kv.second);
@@ -798,10 +805,7 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
         if ((err = lpb::cluster_kernel_prepare()) == cudaSuccess) active = lpb::cluster_max_active(C, smem);
         cudaGetLastError();
         if (active <= 0) {
-            for (int32_t k : kv.second) {
-                streamed.push_back(k);
-                h->slot_bytes = std::max(h->slot_bytes, lpb::streamed_slot_bytes(hm[k], hn[k], hk[k]));
-            }
+            for (int32_t k : kv.second) defer(k);
             continue;
         }
         lp_batch::ClusterGroup g;
@@ -842,10 +846,19 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
     h->num_single = (int32_t)single.size();
     if (o.precision == LP_PREC_FP32_REFINE) h->num_mixed += h->num_single;
     order.insert(order.end(), single.begin(), single.end());
-    lpt(streamed);
-    h->streamed_offset = (int64_t)order.size();
-    h->num_streamed = (int32_t)streamed.size();
-    order.insert(order.end(), streamed.begin(), streamed.end());
+    for (int c = 0; c < lpb::kDeferredClasses; ++c) {
+        std::vector<int32_t>& v = deferred[c];
+        if (v.empty()) continue;
+        lpt(v);
+        lp_batch::DeferredGroup g{};
+        g.form = lpb::deferred_form(hm[v[0]], hn[v[0]], hk[v[0]]);
+        g.offset = (int64_t)order.size();
+        g.count = (int32_t)v.size();
+        for (int32_t k : v) g.slot_bytes = std::max(g.slot_bytes, lpb::deferred_slot(hm[k], hn[k], hk[k]).total);
+        order.insert(order.end(), v.begin(), v.end());
+        h->deferred_groups.push_back(g);
+        h->num_streamed += g.count;
+    }
     // the last upload from pageable host memory, ahead of every memset and
     // kernel of this function: such a copy may wait for the stream, and
     // returns once its data is staged (so the host vectors may go out of
@@ -860,9 +873,9 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
         const bool mixed = o.precision == LP_PREC_FP32_REFINE;
         // (each LP's footprint above includes the reduction scratch its area follows)
         h->single_smem = std::max(h->single_smem, lpb::SmallLayout::total);
-        // FP64 streamed LPs stage their update in the CTA's shared memory beyond the reduction scratch
+        // FP64 LPs with deferred updates keep their first pending pivots in the CTA's shared memory
         if (!mixed && h->num_single_streamed > 0)
-            h->single_smem = std::max(h->single_smem, lpb::SmallLayout::total + lpb::kStreamStageBytes);
+            h->single_smem = std::max(h->single_smem, lpb::SmallLayout::total + lpb::kSingleDeferredBytes);
         h->single_smem = (h->single_smem + 1023) / 1024 * 1024;
         if ((err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device)) ||
             (err = mixed ? lpb::mixed_single_prepare(h->single_smem) : lpb::fp64_single_prepare(h->single_smem)))
@@ -880,16 +893,16 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
         h->max_smem = std::max(h->max_smem, h->single_smem);
         if ((err = alloc(h, &h->single_counter, 1, s))) return bail_cuda(err, "single-launch counter");
     }
-    if (h->num_streamed > 0) {
+    for (lp_batch::DeferredGroup& g : h->deferred_groups) {
         int sms = 0;
         if ((err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device)))
             return bail_cuda(err, "device query");
-        int64_t slots = (int64_t)sms * lpb::fp64_streamed_ctas_per_sm();
-        const int64_t cap = std::max<int64_t>(1, kMaxWorkspaceBytes / (int64_t)h->slot_bytes);
-        slots = std::min<int64_t>({slots, (int64_t)h->num_streamed, cap});
-        h->streamed_slots = (int32_t)slots;
-        if ((err = alloc(h, &h->workspace, (size_t)slots * h->slot_bytes, s)) || (err = alloc(h, &h->counter, 1, s)))
-            return bail_cuda(err, "streamed workspace allocation");
+        int64_t slots = (int64_t)sms * lpb::fp64_deferred_ctas_per_sm(g.form);
+        const int64_t cap = std::max<int64_t>(1, kMaxWorkspaceBytes / (int64_t)g.slot_bytes);
+        slots = std::min<int64_t>({slots, (int64_t)g.count, cap});
+        g.slots = (int32_t)slots;
+        if ((err = alloc(h, &g.workspace, (size_t)slots * g.slot_bytes, s)) || (err = alloc(h, &g.counter, 1, s)))
+            return bail_cuda(err, "workspace allocation");
     }
     if (h->num_mixed > 0) {
         h->mp.eps_opt32 = 1e-6f;
@@ -941,7 +954,7 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
                 }
             }
             if (!h->fbig_C) {
-                // else streamed, one slot per SM
+                // else with deferred updates, one slot per SM
                 const int64_t cap = std::max<int64_t>(1, kMaxWorkspaceBytes / (int64_t)h->fbig_slot_bytes);
                 h->fbig_slots = (int32_t)std::min<int64_t>({(int64_t)sms, (int64_t)h->num_fbig, cap});
                 if ((err = alloc(h, &h->fbig_workspace, (size_t)h->fbig_slots * h->fbig_slot_bytes, s)))
@@ -1121,7 +1134,7 @@ lpb_err lp_batch_group_info(lp_batch* h, int32_t index, lp_batch_group* out) {
     if (!h || !out) return fail(LPB_EINVAL, "handle or out is NULL");
     const int32_t nr = (int32_t)h->groups.size(), nm = (int32_t)h->mixed_groups.size();
     const int32_t nc = (int32_t)h->cluster_groups.size();
-    const int32_t ns = h->num_streamed > 0 ? 1 : 0;
+    const int32_t ns = (int32_t)h->deferred_groups.size();
     const int32_t nms = h->num_mstream > 0 ? 1 : 0;
     const int32_t total = nr + nm + nc + ns + nms + (h->num_single > 0 ? 1 : 0);
     if (index < 0 || index >= total) return fail(LPB_EINVAL, "group index out of range");
@@ -1129,7 +1142,7 @@ lpb_err lp_batch_group_info(lp_batch* h, int32_t index, lp_batch_group* out) {
     if (h->num_single > 0 && index == total - 1) {
         out->kind = 5;
         out->count = h->num_single;
-        out->threads = h->num_mixed > 0 ? lpb::kMixedSingleThreads : lpb::kStreamedThreads;
+        out->threads = h->num_mixed > 0 ? lpb::kMixedSingleThreads : lpb::kSingleThreads;
         out->persistent = 1;
         out->smem_bytes = (int64_t)h->single_smem;
         out->tuned_ms = -1.0f;
@@ -1155,11 +1168,12 @@ lpb_err lp_batch_group_info(lp_batch* h, int32_t index, lp_batch_group* out) {
         out->smem_bytes = (int64_t)(index >= nr && g.threads == 32 && !g.persistent ? g.smem_warp : g.smem);
         out->tuned_ms = g.tuned_ms;
     } else if (index < nr + nm + nc + ns) {
+        const lp_batch::DeferredGroup& g = h->deferred_groups[index - nr - nm - nc];
         out->kind = 2;
-        out->count = h->num_streamed;
-        out->threads = lpb::kStreamedThreads;
+        out->count = g.count;
+        out->threads = g.form.threads;
         out->persistent = 1;
-        out->smem_bytes = 0;
+        out->smem_bytes = (int64_t)g.form.smem;
         out->tuned_ms = -1.0f;
     } else {
         out->kind = 4;
@@ -1342,7 +1356,7 @@ lpb_err lp_batch_stage_times(lp_batch* h, float* stage_ms, int32_t* num_solves) 
 lpb_err lp_batch_plan_info(lp_batch* h, lp_batch_plan* plan) {
     if (!h || !plan) return fail(LPB_EINVAL, "handle or plan is NULL");
     plan->num_groups = (int32_t)(h->groups.size() + h->mixed_groups.size() + h->cluster_groups.size()) +
-                       (h->num_streamed > 0 ? 1 : 0) + (h->num_mstream > 0 ? 1 : 0) + (h->num_fsmall > 0 ? 1 : 0) +
+                       (int32_t)h->deferred_groups.size() + (h->num_mstream > 0 ? 1 : 0) + (h->num_fsmall > 0 ? 1 : 0) +
                        (h->num_fbig > 0 ? 1 : 0) + (h->num_single > 0 ? 1 : 0);
     plan->num_resident = h->num_lps - h->num_streamed - h->num_mstream - h->num_cluster - h->num_single_streamed;
     plan->num_cluster = h->num_cluster;
@@ -1379,10 +1393,10 @@ lpb_err lp_batch_plan_info(lp_batch* h, lp_batch_plan* plan) {
     plan->num_streamed = h->num_streamed + h->num_mstream + h->num_single_streamed;
     plan->num_phase1 = h->num_phase1;
     plan->max_smem_bytes = (int64_t)h->max_smem;
-    plan->workspace_bytes = (int64_t)h->streamed_slots * (int64_t)h->slot_bytes +
-                            (int64_t)h->mstream_slots * (int64_t)h->mslot_bytes +
+    plan->workspace_bytes = (int64_t)h->mstream_slots * (int64_t)h->mslot_bytes +
                             (int64_t)h->fbig_slots * (int64_t)h->fbig_slot_bytes +
                             (h->single_workspace ? (int64_t)h->single_ctas * (int64_t)h->single_slot_bytes : 0);
+    for (const auto& g : h->deferred_groups) plan->workspace_bytes += (int64_t)g.slots * (int64_t)g.slot_bytes;
     return LPB_OK;
 }
 

@@ -103,63 +103,27 @@ __device__ __forceinline__ void cp_async8(void* smem_dst, const void* gmem_src) 
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// ---- mbarriers and bulk asynchronous copies (global -> this CTA's shared
-// memory), for the streamed kernel's staged update ----
-__device__ __forceinline__ unsigned smem_u32(const void* p) {
-    return static_cast<unsigned>(__cvta_generic_to_shared(p));
+// Tie window of Steps 1 and 2: v + tau * max(1, |v|) (product, then sum).
+__device__ __forceinline__ double tie_threshold(double v, double tau) {
+    const long long ab = abskey(v);
+    const double s = (ab < 0x3FF0000000000000LL) ? 1.0 : __longlong_as_double(ab);
+    return __dadd_rn(v, __dmul_rn(tau, s));
 }
-__device__ __forceinline__ void mbar_init(uint64_t* bar, unsigned count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_inval(uint64_t* bar) {
-    asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-// Makes initialised mbarriers visible to the asynchronous proxy.
-__device__ __forceinline__ void mbar_init_fence() {
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, unsigned bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-                 : "memory");
-}
-// `bytes` (a multiple of 16) from 16-byte aligned global `src` to 16-byte
-// aligned shared `dst`; completion counted on `bar`.
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, unsigned bytes, uint64_t* bar) {
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-            smem_u32(dst)),
-        "l"(src), "r"(bytes), "r"(smem_u32(bar))
-        : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, unsigned parity) {
-    unsigned done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(done)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return done != 0;
-}
-// Wait for the phase of `bar` with the given parity; false after `cycles`
-// clock cycles (the copy did not complete).
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, unsigned parity, long long cycles) {
-    if (mbar_try_wait(bar, parity)) return true;
-    const long long t0 = clock64();
-    while (!mbar_try_wait(bar, parity))
-        if (clock64() - t0 > cycles) return false;
-    return true;
-}
-// Orders this thread's earlier generic-proxy accesses of shared memory before
-// later asynchronous-proxy writes to it (reuse of a staging buffer).
-__device__ __forceinline__ void fence_proxy_async_shared() {
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-// Orders this thread's earlier generic-proxy writes of global memory before
-// later asynchronous-proxy reads of it (bulk copies of rows it updated).
-__device__ __forceinline__ void fence_proxy_async_global() {
-    asm volatile("fence.proxy.async.global;" ::: "memory");
+
+// Upper bound, in units of okey, of okey(thr) - okey(v) where thr is the tie
+// threshold v + tau*max(1,|v|) of a negative v (Step 1).  `wb` >=
+// tau*2^54*(1+2^-53) + 1.5 is precomputed on the host (< 0: no bound).  The
+// interval (v, thr] lies in v's binade or the one below (tau|v| < |v|/2), where
+// doubles are spaced at least 2^(E-53) apart, E = exponent of v:
+//   E >= 0: thr - v <= tau*2^(E+1)*(1+2^-53) + half an ulp  -> <= wb keys;
+//   E <  0: thr - v <= tau*(1+2^-53) + half an ulp          -> <= wb << (-E-1).
+__device__ __forceinline__ unsigned long long step1_window(long long kmin, long long wb) {
+    if (wb < 0) return ~0ull;
+    const int E = dexp(kval(kmin));
+    if (E >= 0) return (unsigned long long)wb;
+    const int sh = -E - 1;
+    if (sh > 30) return ~0ull;
+    return (unsigned long long)wb << sh;
 }
 
 // Block-wide reductions over per-warp `redux` results.  Each call writes

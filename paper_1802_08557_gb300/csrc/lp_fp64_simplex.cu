@@ -1,8 +1,7 @@
-// lp_fp64_simplex.cu -- FP64 dense simplex, one CTA per LP: the tableau is
-// resident in shared memory when it fits (fp64_resident_kernel) and streamed
-// through a global-memory workspace slot otherwise (fp64_streamed_kernel,
-// persistent CTAs taking LPs from an atomic counter).  Both run the same
-// per-LP code (solve_one).
+// lp_fp64_simplex.cu -- FP64 dense simplex, one CTA per LP: small tableaux are
+// resident in shared memory (fp64_resident_kernel, solve_one below); larger
+// ones are never updated as a whole (fp64_deferred_kernel, persistent CTAs
+// taking LPs from an atomic counter; lp_fp64_deferred.cuh).
 //
 // Method: Gurung & Ray, "Simultaneous Solving of Batched Linear Programs on a
 // GPU" (arXiv 1802.08557).  Section 4.1 assigns one CUDA block per LP; Section
@@ -15,9 +14,8 @@
 //    the entering column and the leaving row.  Basic columns of the paper's
 //    full tableau are unit vectors and carry no information;
 //  - the tableau lives in shared memory for the whole solve (global memory is
-//    touched only to read A, b, c and write the results), or, above one CTA's
-//    shared memory, in a global workspace slot whose rank-1 update streams
-//    through shared-memory rings filled by bulk asynchronous copies;
+//    touched only to read A, b, c and write the results); above a size,
+//    elements are formed only when a pivot reads them (deferred updates);
 //  - reductions are warp `redux` instructions on 64-bit order-preserving
 //    integer keys of the FP64 values (exact, no FP64-pipe compares);
 //  - phase I runs in the same kernel (the paper launches twice, Section 5);
@@ -39,72 +37,11 @@
 #include <climits>
 
 #include "lp_device.cuh"
+#include "lp_fp64_deferred.cuh"
 #include "lp_internal.h"
 
 namespace lpb {
 namespace {
-
-// Tie window of Steps 1 and 2: v + tau * max(1, |v|) (product, then sum).
-__device__ __forceinline__ double tie_threshold(double v, double tau) {
-    const long long ab = abskey(v);
-    const double s = (ab < 0x3FF0000000000000LL) ? 1.0 : __longlong_as_double(ab);
-    return __dadd_rn(v, __dmul_rn(tau, s));
-}
-
-// Upper bound, in units of okey, of okey(thr) - okey(v) where thr is the tie
-// threshold v + tau*max(1,|v|) of a negative v (Step 1).  `wb` >=
-// tau*2^54*(1+2^-53) + 1.5 is precomputed on the host (< 0: no bound).  The
-// interval (v, thr] lies in v's binade or the one below (tau|v| < |v|/2), where
-// doubles are spaced at least 2^(E-53) apart, E = exponent of v:
-//   E >= 0: thr - v <= tau*2^(E+1)*(1+2^-53) + half an ulp  -> <= wb keys;
-//   E <  0: thr - v <= tau*(1+2^-53) + half an ulp          -> <= wb << (-E-1).
-__device__ __forceinline__ unsigned long long step1_window(long long kmin, long long wb) {
-    if (wb < 0) return ~0ull;
-    const int E = dexp(kval(kmin));
-    if (E >= 0) return (unsigned long long)wb;
-    const int sh = -E - 1;
-    if (sh > 30) return ~0ull;
-    return (unsigned long long)wb << sh;
-}
-
-// ---- Staged update of the streamed kernel ----------------------------------
-// The rank-1 update of a tableau in global memory is bound by the bytes it
-// keeps in flight.  Each warp streams its share of the rows through a ring of
-// kStageDepth chunks of kStageChunkPairs column pairs in shared memory, filled
-// by bulk asynchronous copies (cp.async.bulk, completion on one mbarrier per
-// chunk) that one lane issues kStageDepth chunks ahead; the pivot row and the
-// pivot column are read from shared-memory copies.  The FMA of every element
-// is the one of the plain loop, so the results are the same bit for bit.
-constexpr int kStageChunkPairs = 96;  // 1.5 KB per chunk: 3 pairs per lane
-constexpr int kStageDepth = 3;
-constexpr long long kStageWaitCycles = 2000000000LL;  // ~1 s at 2 GHz
-
-// A CTA's shared memory for the staged update: a flag word, the mbarriers and
-// rings of every warp, the pivot-row copy (LD doubles), then the pivot-column
-// copy (R doubles) of the LP being solved.  Everything but the column copy
-// sits at offsets that depend only on the number of warps.
-__host__ __device__ inline size_t stage_rings(int nwarps) {
-    return (16 + (size_t)nwarps * kStageDepth * 8 + 127) & ~size_t(127);
-}
-__host__ __device__ inline size_t stage_prow(int nwarps) {
-    return stage_rings(nwarps) + (size_t)nwarps * kStageDepth * kStageChunkPairs * 16;
-}
-__host__ __device__ inline size_t stage_colE(int nwarps, int LD) { return stage_prow(nwarps) + align16((size_t)LD * 8); }
-__host__ __device__ inline size_t stage_total(int nwarps, int R, int LD) {
-    return stage_colE(nwarps, LD) + align16((size_t)R * 8);
-}
-
-// The staged path of one LP: `base` of the staging area (null: the plain
-// loop) and the parities of the warp's chunk mbarriers (bit s: parity of the
-// next completion of chunk s, warp-uniform).  The flag word at `base`: 1 a
-// copy did not complete (LP abandoned); 2 one may still be in flight.
-struct Staging {
-    unsigned char* base;
-    unsigned phase;
-};
-__device__ __forceinline__ uint64_t* stage_bars(unsigned char* base) {
-    return reinterpret_cast<uint64_t*>(base + 16) + (threadIdx.x >> 5) * kStageDepth;
-}
 
 struct Tab {
     double* T;        // R x LD, row-major; column 0 = right-hand side
@@ -114,92 +51,6 @@ struct Tab {
     int LD;
 };
 
-// Phase B of Step 3 for a tableau in global memory, through the staging
-// rings: chunk c covers row ii = c / cpr (skipping the pivot row l) and pairs
-// [p0, p0 + len) of it; warp w takes chunks w, w + nw, ...  The pivot row is
-// read from the staging area's copy, column e from tb.colE (shared memory on this path).
-// The pair beyond an odd Cact is padding (updated, never read).  A copy that
-// does not complete within kStageWaitCycles abandons the update: the flag
-// word is set (the caller reports the LP as numerical) after the warp has waited,
-// bounded again, for its other copies.
-__device__ __noinline__ unsigned staged_update(const Staging st, const Tab tb, int Ract, int Cact, int l, int e) {
-    unsigned phase = st.phase;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int LD = tb.LD;
-    uint64_t* bar = stage_bars(st.base);
-    double2* ring = reinterpret_cast<double2*>(st.base + stage_rings(nw)) + (size_t)warp * kStageDepth * kStageChunkPairs;
-    const int Cp = (Cact + 1) >> 1;
-    const int cpr = (Cp + kStageChunkPairs - 1) / kStageChunkPairs;
-    const int total = (Ract - 1) * cpr;
-    const double2* P2 = reinterpret_cast<const double2*>(st.base + stage_prow(nw));
-    auto chunk = [&](int c, int& r, int& p0, int& len) {
-        const int ii = c / cpr;
-        const int piece = c - ii * cpr;
-        r = ii + (ii >= l ? 1 : 0);
-        p0 = piece * kStageChunkPairs;
-        len = min(kStageChunkPairs, Cp - p0);
-    };
-    auto issue = [&](int c, int s) {  // lane 0
-        int r, p0, len;
-        chunk(c, r, p0, len);
-        const unsigned bytes = (unsigned)len * 16u;
-        mbar_expect_tx(&bar[s], bytes);
-        bulk_load(ring + s * kStageChunkPairs, tb.T + (size_t)r * LD + 2 * p0, bytes, &bar[s]);
-    };
-    unsigned pending = 0;  // chunks issued and not yet waited for (warp-uniform)
-    for (int s = 0; s < kStageDepth; ++s) {
-        const int c = warp + s * nw;
-        if (c < total) {
-            if (lane == 0) issue(c, s);
-            pending |= 1u << s;
-        }
-    }
-    bool ok = true;
-    for (int it = 0;; ++it) {
-        const int c = warp + it * nw;
-        if (c >= total) break;
-        const int s = it % kStageDepth;
-        ok = __all_sync(kFull, mbar_wait_bounded(&bar[s], (phase >> s) & 1u, kStageWaitCycles));
-        if (!ok) break;
-        phase ^= 1u << s;
-        pending &= ~(1u << s);
-        int r, p0, len;
-        chunk(c, r, p0, len);
-        const double cr = -tb.colE[r];
-        const double2* src = ring + s * kStageChunkPairs;
-        double2* dst = reinterpret_cast<double2*>(tb.T + (size_t)r * LD) + p0;
-        for (int q = lane; q < len; q += 32) {
-            const double2 old = src[q];
-            const double2 p = P2[p0 + q];
-            const int j = 2 * (p0 + q);
-            double2 v;
-            v.x = __fma_rn(cr, p.x, (j == e) ? 0.0 : old.x);
-            v.y = __fma_rn(cr, p.y, (j + 1 == e) ? 0.0 : old.y);
-            dst[q] = v;
-        }
-        __syncwarp();
-        const int cn = c + kStageDepth * nw;
-        if (cn < total) {
-            if (lane == 0) {
-                fence_proxy_async_shared();  // the warp's reads of chunk s before the copy over it
-                issue(cn, s);
-            }
-            pending |= 1u << s;
-        }
-    }
-    if (!ok) {
-        // let the copies still in flight land before the rings are reused
-        bool drained = true;
-        for (int s = 0; s < kStageDepth; ++s)
-            if (pending & (1u << s)) {
-                drained = mbar_wait_bounded(&bar[s], (phase >> s) & 1u, kStageWaitCycles) && drained;
-                phase ^= 1u << s;
-            }
-        if (lane == 0) atomicMax(reinterpret_cast<int*>(st.base), drained ? 1 : 2);
-    }
-    return phase;
-}
-
 // Step 3 (Section 3.1, Listing 1) on the condensed tableau: divide pivot row
 // l by PE = colE[l], then t_ij <- fma(-t_ie, r_j, t_ij) for every other active
 // row.  In column e (which now holds the leaving variable) the old entry of the
@@ -208,10 +59,6 @@ __device__ __noinline__ unsigned staged_update(const Staging st, const Tab tb, i
 // colE[0..Ract) must hold column e on entry.  Returns the variable that left
 // the basis (now the label of column e), read by every thread between the two
 // barriers, where nothing writes it.
-// kPairs (the streamed kernel: rows 32-byte aligned in global memory, LD a
-// multiple of 4): the update takes two adjacent columns per thread with
-// 16-byte loads and stores -- the same FMA for every element, so the same
-// results; the pair beyond an odd Cact is padding (updated, never read).
 // The barrier of the thread group that owns the LP: the CTA, or (kWarp: a
 // one-warp CTA) the warp -- no block barrier, shared-memory writes ordered by
 // __syncwarp.
@@ -221,21 +68,17 @@ __device__ __forceinline__ void group_sync() {
     else __syncthreads();
 }
 
-template <bool kPairs = false, bool kWarp = false>
-__device__ __forceinline__ int pivot(Tab& tb, int Ract, int Cact, int l, int e, Staging* st = nullptr) {
+template <bool kWarp>
+__device__ __forceinline__ int pivot(Tab& tb, int Ract, int Cact, int l, int e) {
     const int tid = threadIdx.x, nt = blockDim.x;
     const int LD = tb.LD;
     double* T = tb.T;
     const double* colE = tb.colE;
     const double pe = colE[l];
     double* Tl = T + (size_t)l * LD;
-    const bool staged = kPairs && st != nullptr && st->base != nullptr;
-    double* prow = staged ? reinterpret_cast<double*>(st->base + stage_prow(nt >> 5)) : nullptr;
     for (int j = tid; j < Cact; j += nt) {
         const double v = (j == e) ? 1.0 : Tl[j];
-        const double q = __ddiv_rn(v, pe);
-        Tl[j] = q;
-        if (staged) prow[j] = q;
+        Tl[j] = __ddiv_rn(v, pe);
     }
     if (tid == 0) {
         const int ev = tb.col_var[e];
@@ -244,37 +87,6 @@ __device__ __forceinline__ int pivot(Tab& tb, int Ract, int Cact, int l, int e, 
     }
     group_sync<kWarp>();
     const int left = tb.col_var[e];
-    if (staged) {
-        st->phase = staged_update(*st, tb, Ract, Cact, l, e);
-        fence_proxy_async_global();  // this thread's stores before later bulk reads of them
-        group_sync<kWarp>();
-        return left;
-    }
-    if (kPairs) {
-        const int Cp = (Cact + 1) >> 1;
-        const int total = (Ract - 1) * Cp;
-        int ii = tid / Cp;
-        int jp = tid - ii * Cp;
-        const int di = nt / Cp;
-        const int dj = nt - di * Cp;
-        const double2* Tl2 = reinterpret_cast<const double2*>(Tl);
-        for (int idx = tid; idx < total; idx += nt) {
-            const int r = ii + (ii >= l ? 1 : 0);
-            double2* t = reinterpret_cast<double2*>(T + (size_t)r * LD) + jp;
-            const double2 old = *t;
-            const double2 p = Tl2[jp];
-            const double c = -colE[r];
-            double2 v;
-            v.x = __fma_rn(c, p.x, (2 * jp == e) ? 0.0 : old.x);
-            v.y = __fma_rn(c, p.y, (2 * jp + 1 == e) ? 0.0 : old.y);
-            *t = v;
-            ii += di;
-            jp += dj;
-            if (jp >= Cp) { jp -= Cp; ++ii; }
-        }
-        group_sync<kWarp>();
-        return left;
-    }
     const int total = (Ract - 1) * Cact;
     int ii = tid / Cact;
     int jj = tid - ii * Cact;
@@ -295,9 +107,8 @@ __device__ __forceinline__ int pivot(Tab& tb, int Ract, int Cact, int l, int e, 
 
 // A retired artificial (it just left the basis and may never re-enter) sits
 // in column e: move the last live column into its place and shrink.
-// `fence`: the tableau is read by bulk copies later (staged streamed update).
-template <bool kWarp = false>
-__device__ __forceinline__ void retire_column(Tab& tb, int Ract, int e, int& Cvar, bool fence = false) {
+template <bool kWarp>
+__device__ __forceinline__ void retire_column(Tab& tb, int Ract, int e, int& Cvar) {
     const int tid = threadIdx.x, nt = blockDim.x;
     if (e != Cvar) {
         for (int r = tid; r < Ract; r += nt) {
@@ -307,19 +118,14 @@ __device__ __forceinline__ void retire_column(Tab& tb, int Ract, int e, int& Cva
         if (tid == 0) tb.col_var[e] = tb.col_var[Cvar];
     }
     --Cvar;
-    if (fence) fence_proxy_async_global();
     group_sync<kWarp>();
 }
 
-// One LP, Steps 1-3 until it halts.  `small` is shared memory
-// (SmallLayout); `big` is shared memory (resident) or a global workspace slot
-// (streamed), laid out by big_layout.  `stage` (streamed only, may be null):
-// `stage_bytes` of this CTA's shared memory for the staged update, used when
-// the LP's stage_total fits.
-template <bool kStreamed, bool kWarp = false>
+// One LP, Steps 1-3 until it halts, in shared memory: the reductions' scratch
+// in `small` (SmallLayout), the tableau and its vectors in `big` (big_layout).
+template <bool kWarp = false>
 __device__ __forceinline__ void solve_one(const DeviceBatch& B, const Tolerances& tol, const int lp,
-                                          unsigned char* small, unsigned char* big, int32_t* diag,
-                                          unsigned char* stage = nullptr, size_t stage_bytes = 0)
+                                          unsigned char* small, unsigned char* big, int32_t* diag)
 {
     const int m = B.m[lp];
     const int n = B.n[lp];
@@ -331,7 +137,7 @@ __device__ __forceinline__ void solve_one(const DeviceBatch& B, const Tolerances
     const int lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
 
     // k-independent part of the layout (k = 0 gives the same offsets)
-    const BigLayout L0 = big_layout(m, n, 0, kStreamed);
+    const BigLayout L0 = big_layout(m, n, 0);
     // the group's reductions: block-wide through the scratch in `small`, or
     // (kWarp) `redux` within the one warp
     auto make_red = [&]() {
@@ -368,7 +174,7 @@ __device__ __forceinline__ void solve_one(const DeviceBatch& B, const Tolerances
     }
     group_sync<kWarp>();  // neg[] and row_var[] are read by other threads below
 
-    const BigLayout L = big_layout(m, n, k, kStreamed);
+    const BigLayout L = big_layout(m, n, k);
     Tab tb;
     tb.T = reinterpret_cast<double*>(big + L.T);
     tb.colE = reinterpret_cast<double*>(big + L.colE);
@@ -378,60 +184,28 @@ __device__ __forceinline__ void solve_one(const DeviceBatch& B, const Tolerances
     const int LD = L.LD;
     double* T = tb.T;  // the tableau is written through several pointers: no restrict
     int Cvar = n + k;  // live variable columns 1..Cvar
-    Staging stg{nullptr, 0u};
-    if (kStreamed && stage != nullptr) {
-        if (tid == 0) *reinterpret_cast<int*>(stage) = 0;  // the flag word (read after the barriers below)
-        if (stage_total(nw, L.R, L.LD) <= stage_bytes) {
-            stg.base = stage;
-            tb.colE = reinterpret_cast<double*>(stage + stage_colE(nw, L.LD));  // pivot column in shared memory
-            if (lane == 0) {
-                for (int q = 0; q < kStageDepth; ++q) mbar_init(&stage_bars(stage)[q], 1);
-                mbar_init_fence();
-            }
-        }
-    }
-    const bool staged = kStreamed && stg.base != nullptr;
-    // the barriers are invalidated before their memory can serve another LP
-    // (unless a copy may still be in flight: the kernel then stops)
-    auto release_staging = [&]() {
-        if (staged && lane == 0 && *reinterpret_cast<volatile int*>(stage) != 2)
-            for (int q = 0; q < kStageDepth; ++q) mbar_inval(&stage_bars(stage)[q]);
-    };
 
     for (int j = tid; j <= Cvar; j += nt)
         tb.col_var[j] = (j == 0) ? -1 : (j <= n ? j - 1 : n + neg[j - 1 - n]);
     {
-        // A into rows 0..m-1, columns 1..n: one flat pass with several
-        // independent loads in flight per thread; then b and the slack columns
+        // A into rows 0..m-1, columns 1..n: asynchronous copies, all in flight
+        // at once, then the negated rows in place; then b and the slack columns
         const int64_t cnt = (int64_t)m * n;
         int i = tid / n, j = tid - i * n;
         const int di = nt / n, dj = nt - di * n;
-        if (!kStreamed) {
-            // shared-memory tableau: asynchronous copies, all in flight at once,
-            // then the negated rows in place
-            for (int64_t idx = tid; idx < cnt; idx += nt) {
-                cp_async8(T + (size_t)i * LD + 1 + j, A + idx);
-                i += di;
-                j += dj;
-                if (j >= n) { j -= n; ++i; }
-            }
-            cp_async_wait_all();
-            group_sync<kWarp>();
-            if (k > 0)
-                for (int64_t idx = tid; idx < cnt; idx += nt) {
-                    const int i2 = (int)(idx / n), j2 = (int)(idx - (int64_t)i2 * n);
-                    if (row_var[i2] >= nm) T[(size_t)i2 * LD + 1 + j2] = -T[(size_t)i2 * LD + 1 + j2];
-                }
-        } else {
-#pragma unroll 4
-            for (int64_t idx = tid; idx < cnt; idx += nt) {
-                const double v = A[idx];
-                T[(size_t)i * LD + 1 + j] = (row_var[i] >= nm) ? -v : v;
-                i += di;
-                j += dj;
-                if (j >= n) { j -= n; ++i; }
-            }
+        for (int64_t idx = tid; idx < cnt; idx += nt) {
+            cp_async8(T + (size_t)i * LD + 1 + j, A + idx);
+            i += di;
+            j += dj;
+            if (j >= n) { j -= n; ++i; }
         }
+        cp_async_wait_all();
+        group_sync<kWarp>();
+        if (k > 0)
+            for (int64_t idx = tid; idx < cnt; idx += nt) {
+                const int i2 = (int)(idx / n), j2 = (int)(idx - (int64_t)i2 * n);
+                if (row_var[i2] >= nm) T[(size_t)i2 * LD + 1 + j2] = -T[(size_t)i2 * LD + 1 + j2];
+            }
         for (int r = warp; r < m; r += nw) {
             const bool isneg = row_var[r] >= nm;
             double* Tr = T + (size_t)r * LD;
@@ -461,7 +235,6 @@ __device__ __forceinline__ void solve_one(const DeviceBatch& B, const Tolerances
         group_sync<kWarp>();
     }
 
-    if (staged) fence_proxy_async_global();  // the build's stores before bulk reads of them
     const long long key_neg_eps_opt = okey(-tol.eps_opt);
     const long long key_eps_piv = okey(tol.eps_piv);
     const int max_iters = tol.max_iters > 0 ? tol.max_iters : 50 * (m + n);
@@ -504,10 +277,9 @@ __device__ __forceinline__ void solve_one(const DeviceBatch& B, const Tolerances
                 const int e = (int)(sel & 0xffffu);
                 for (int r = tid; r < m + 1; r += nt) tb.colE[r] = T[(size_t)r * LD + e];
                 group_sync<kWarp>();
-                const int left = pivot<kStreamed, kWarp>(tb, m + 1, Cvar + 1, i, e, &stg);
+                const int left = pivot<kWarp>(tb, m + 1, Cvar + 1, i, e);
                 ++iters;
-                if (staged && *reinterpret_cast<volatile int*>(stage)) { status = kNumerical; break; }
-                if (left >= nm) retire_column<kWarp>(tb, m + 1, e, Cvar, staged);
+                if (left >= nm) retire_column<kWarp>(tb, m + 1, e, Cvar);
             }
             phase = 2;
             continue;
@@ -605,14 +377,9 @@ __device__ __forceinline__ void solve_one(const DeviceBatch& B, const Tolerances
         if (iters >= max_iters) { status = kIterLimit; break; }
 
         // ---- Step 3: pivot ---------------------------------------------------
-        const int left = pivot<kStreamed, kWarp>(tb, Ract, Cvar + 1, l, e, &stg);
+        const int left = pivot<kWarp>(tb, Ract, Cvar + 1, l, e);
         ++iters;
-        if (staged && *reinterpret_cast<volatile int*>(stage)) {
-            if (tid == 0) record_internal_error(diag, 8, lp, iters);  // a bulk copy did not complete
-            status = kNumerical;
-            break;
-        }
-        if (left >= nm) retire_column<kWarp>(tb, Ract, e, Cvar, staged);
+        if (left >= nm) retire_column<kWarp>(tb, Ract, e, Cvar);
     }
 
     // ---- labels must name variables (self-check before they index global
@@ -629,7 +396,6 @@ __device__ __forceinline__ void solve_one(const DeviceBatch& B, const Tolerances
                 B.status[lp] = kNumerical;
                 B.iters[lp] = iters;
             }
-            release_staging();
             return;
         }
     }
@@ -654,7 +420,6 @@ __device__ __forceinline__ void solve_one(const DeviceBatch& B, const Tolerances
         B.iters[lp] = iters;
         B.obj[lp] = T[(size_t)m * LD];
     }
-    release_staging();
 }
 
 __global__ void __launch_bounds__(kMaxThreads, 2)
@@ -662,7 +427,7 @@ fp64_resident_kernel(const DeviceBatch B, const Tolerances tol, const int32_t* _
                      int32_t* __restrict__ diag)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    solve_one<false>(B, tol, order[blockIdx.x], smem, smem + SmallLayout::total, diag);
+    solve_one(B, tol, order[blockIdx.x], smem, smem + SmallLayout::total, diag);
 }
 
 // One warp per LP (blockDim = 32), the form of the groups of small tableaux:
@@ -673,7 +438,7 @@ fp64_warp_kernel(const DeviceBatch B, const Tolerances tol, const int32_t* __res
                  int32_t* __restrict__ diag)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    solve_one<false, true>(B, tol, order[blockIdx.x], smem, smem + SmallLayout::total, diag);
+    solve_one<true>(B, tol, order[blockIdx.x], smem, smem + SmallLayout::total, diag);
 }
 
 // Resident kernel over a device-side list: persistent CTAs take the LPs
@@ -698,22 +463,37 @@ fp64_resident_queue_kernel(const DeviceBatch B, const Tolerances tol, const int3
             if (threadIdx.x == 0) record_internal_error(diag, 5, lp);
             continue;
         }
-        solve_one<false>(B, tol, lp, smem, smem + SmallLayout::total, diag);
+        solve_one(B, tol, lp, smem, smem + SmallLayout::total, diag);
         __syncthreads();
     }
 }
 
 
-__global__ void __launch_bounds__(kStreamedThreads, 2)
-fp64_streamed_kernel(const DeviceBatch B, const Tolerances tol, const int32_t* __restrict__ order,
+// One LP with deferred updates: its vectors and first pending pivots in
+// `bytes` of shared memory when the vectors fit (phase I's, at their largest),
+// else in the workspace slot.
+__device__ __forceinline__ void deferred_one(const DeviceBatch& B, const Tolerances& tol, const int lp,
+                                             unsigned char* small, unsigned char* shared, const size_t bytes,
+                                             unsigned char* slot, int32_t* diag)
+{
+    if (deferred_layout(B.m[lp], B.n[lp], B.m[lp]).hist <= bytes)
+        deferred_solve<true>(B, tol, lp, small, shared, bytes, slot, diag);
+    else
+        deferred_solve<false>(B, tol, lp, small, slot, 0, slot, diag);
+}
+
+// LPs whose tableau is not kept in shared memory (lp_fp64_deferred.cuh):
+// persistent CTAs take them from the atomic `counter`; CTA i owns workspace
+// slot i.
+__global__ void __launch_bounds__(kMaxThreads, 1)
+fp64_deferred_kernel(const DeviceBatch B, const Tolerances tol, const int32_t* __restrict__ order,
                      const int32_t count, const int32_t* __restrict__ count_dev, unsigned char* workspace,
                      const size_t slot_bytes, int32_t* __restrict__ counter, int32_t* __restrict__ diag,
-                     const size_t stage_bytes)
+                     const size_t smem_bytes)
 {
-    __shared__ __align__(16) unsigned char small[SmallLayout::total];
+    extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int next;
-    extern __shared__ __align__(128) unsigned char stage[];
-    unsigned char* big = workspace + (size_t)blockIdx.x * slot_bytes;
+    unsigned char* slot = workspace + (size_t)blockIdx.x * slot_bytes;
     const int n_items = count_dev ? min(*count_dev, count) : count;
     for (;;) {
         if (threadIdx.x == 0) next = atomicAdd(counter, 1);
@@ -721,19 +501,17 @@ fp64_streamed_kernel(const DeviceBatch B, const Tolerances tol, const int32_t* _
         const int idx = next;
         __syncthreads();
         if (idx >= n_items) break;
-        solve_one<true>(B, tol, order[idx], small, big, diag, stage_bytes ? stage : nullptr, stage_bytes);
+        deferred_one(B, tol, order[idx], smem, smem + SmallLayout::total, smem_bytes - SmallLayout::total, slot, diag);
         __syncthreads();
-        // a bulk copy that may still be in flight into the rings: take no more LPs
-        if (stage_bytes && *reinterpret_cast<volatile int*>(stage) == 2) break;
     }
 }
 
 // A whole batch in one launch: persistent CTAs take the LPs order[0 ..
 // count) (longest work first) from the atomic `counter` and solve each with
 // the tableau in this CTA's shared memory when it fits (resident[lp] != 0),
-// else in this CTA's global workspace slot -- the same per-LP code as the
-// resident and streamed kernels, so the same results.
-__global__ void __launch_bounds__(kStreamedThreads, 2)
+// else with deferred updates and this CTA's global workspace slot -- the same
+// per-LP code as the resident and deferred kernels, so the same results.
+__global__ void __launch_bounds__(kSingleThreads, 2)
 fp64_single_kernel(const DeviceBatch B, const Tolerances tol, const int32_t* __restrict__ order,
                    const uint8_t* __restrict__ resident, const int32_t count, unsigned char* workspace,
                    const size_t slot_bytes, int32_t* __restrict__ counter, int32_t* __restrict__ diag,
@@ -750,13 +528,9 @@ fp64_single_kernel(const DeviceBatch B, const Tolerances tol, const int32_t* __r
         if (idx >= count) break;
         const int lp = order[idx];
         if (resident[lp]) {
-            solve_one<false>(B, tol, lp, smem, smem + SmallLayout::total, diag);
+            solve_one(B, tol, lp, smem, smem + SmallLayout::total, diag);
         } else if (slot) {
-            // the CTA's shared memory beyond the reduction scratch stages the update
-            unsigned char* stage = smem + SmallLayout::total;
-            solve_one<true>(B, tol, lp, smem, slot, diag, stage, smem_bytes - SmallLayout::total);
-            __syncthreads();
-            if (*reinterpret_cast<volatile int*>(stage) == 2) break;  // a copy may still be in flight
+            deferred_one(B, tol, lp, smem, smem + SmallLayout::total, smem_bytes - SmallLayout::total, slot, diag);
         } else if (threadIdx.x == 0) {
             record_internal_error(diag, 7, lp);  // a plan without a slot for a streamed LP
         }
@@ -794,29 +568,61 @@ cudaError_t launch_fp64_resident_queue(const DeviceBatch& B, const Tolerances& t
     return cudaGetLastError();
 }
 
-cudaError_t fp64_streamed_prepare() {
-    return cudaFuncSetAttribute(fp64_streamed_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)kStreamStageBytes);
+// Deferred updates for every tableau above one CTA's shared memory, and for
+// tableaux of more than 14,000 entries: at 130 x 130 they win whatever the
+// number of pivots (2000 mixed-sign LPs, 326 pivots: 34.1 against 37.5 ms in
+// shared memory; positive 200 x 200, 25 pivots: 2.6 against 3.9 ms); at 100 x 100
+// they lose on many pivots (mixed-sign, 200 pivots: 19.3 against 18.5 ms) and
+// win on few (positive, 15 pivots: 0.73 against 1.26 ms), and the number of
+// pivots is not known beforehand.
+bool defer_updates(int m, int n, int k) {
+    return resident_smem_bytes(m, n, k) > kMaxSmemPerBlock || (int64_t)(m + 1) * (n + k + 1) > 14000;
 }
 
-int fp64_streamed_ctas_per_sm() {
+int resident_threads(int m, int n, int k) {
+    const int64_t e = (int64_t)(m + 1 + (k > 0)) * (n + k + 1);
+    // measured best on GB300 (mixed-sign dense m x m, m = 20..100)
+    if (e <= 1024) return 32;
+    if (e <= 3072) return 64;
+    if (e <= 8192) return 128;
+    if (e <= 32768) return 256;
+    return 512;
+}
+
+// Size classes by the length of a row and a column together: few threads for
+// small LPs (more LPs per SM; a pivot's work is one row and one column), more
+// pending pivots in shared memory for large ones.  256 threads instead of 512
+// in class 2: 20,000 uneven LPs 3.6 against 4.1 ms, but 300 mixed-sign
+// LPs of 300 x 300 (long runs of pivots, where the flushes are the work)
+// 215 against 148 ms.
+DeferredForm deferred_form(int m, int n, int k) {
+    const int w = m + n + k;
+    if (w <= 192) return {0, 64, 24 << 10};
+    if (w <= 448) return {1, 128, 44 << 10};
+    if (w <= 2048) return {2, 512, 100 << 10};
+    return {3, 512, kMaxSmemPerBlock - 1024};
+}
+
+int fp64_deferred_ctas_per_sm(const DeferredForm& f) {
     int blocks = 0;
-    if (fp64_streamed_prepare() != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, fp64_streamed_kernel, kStreamedThreads,
-                                                      kStreamStageBytes) != cudaSuccess)
+    if (cudaFuncSetAttribute(fp64_deferred_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(kMaxSmemPerBlock - 1024)) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, fp64_deferred_kernel, f.threads, f.smem) != cudaSuccess)
         return 1;
     return blocks > 0 ? blocks : 1;
 }
 
-cudaError_t launch_fp64_streamed(const DeviceBatch& B, const Tolerances& tol, const int32_t* order,
-                                 int32_t count, int slots, unsigned char* workspace, size_t slot_bytes,
+cudaError_t launch_fp64_deferred(const DeviceBatch& B, const Tolerances& tol, const int32_t* order, int32_t count,
+                                 const DeferredForm& f, int slots, unsigned char* workspace, size_t slot_bytes,
                                  int32_t* counter, int32_t* diag, cudaStream_t stream, const int32_t* count_dev) {
     if (count <= 0) return cudaSuccess;
     cudaError_t err = cudaMemsetAsync(counter, 0, sizeof(int32_t), stream);
     if (err != cudaSuccess) return err;
-    if ((err = fp64_streamed_prepare()) != cudaSuccess) return err;
-    fp64_streamed_kernel<<<slots, kStreamedThreads, kStreamStageBytes, stream>>>(
-        B, tol, order, count, count_dev, workspace, slot_bytes, counter, diag, kStreamStageBytes);
+    if ((err = cudaFuncSetAttribute(fp64_deferred_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)(kMaxSmemPerBlock - 1024))) != cudaSuccess)
+        return err;
+    fp64_deferred_kernel<<<slots, f.threads, f.smem, stream>>>(B, tol, order, count, count_dev, workspace, slot_bytes,
+                                                               counter, diag, f.smem);
     return cudaGetLastError();
 }
 
@@ -828,7 +634,7 @@ cudaError_t fp64_single_prepare(size_t smem) {
 
 int fp64_single_ctas_per_sm(size_t smem) {
     int blocks = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, fp64_single_kernel, kStreamedThreads, smem) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, fp64_single_kernel, kSingleThreads, smem) !=
         cudaSuccess) {
         cudaGetLastError();
         return 0;
@@ -843,7 +649,7 @@ cudaError_t launch_fp64_single(const DeviceBatch& B, const Tolerances& tol, cons
     if (count <= 0) return cudaSuccess;
     cudaError_t err = cudaMemsetAsync(counter, 0, sizeof(int32_t), stream);
     if (err != cudaSuccess) return err;
-    fp64_single_kernel<<<ctas, kStreamedThreads, smem, stream>>>(B, tol, order, resident, count, workspace,
+    fp64_single_kernel<<<ctas, kSingleThreads, smem, stream>>>(B, tol, order, resident, count, workspace,
                                                                   slot_bytes, counter, diag, smem);
     return cudaGetLastError();
 }

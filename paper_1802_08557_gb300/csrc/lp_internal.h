@@ -59,8 +59,7 @@ constexpr size_t kMaxSmemPerBlock = 227 * 1024;  // opt-in dynamic shared memory
 // (reduction scratch) is always in shared memory.  The big part holds the
 // condensed (Tucker) tableau -- R = m+1 (+1 phase-I row) rows x LD >= n+k+1
 // columns, column 0 = right-hand side, then the non-basic variables -- plus
-// per-row / per-column arrays.  It lives in shared memory for the resident
-// kernel and in a global-memory workspace slot for the streamed kernel.  The
+// per-row / per-column arrays, in the resident kernel's shared memory.  The
 // k-independent arrays come first, so the kernel can place them before it has
 // counted the k rows with b_i < 0.
 struct SmallLayout {
@@ -78,12 +77,11 @@ struct BigLayout {
 
 __host__ __device__ inline size_t align16(size_t v) { return (v + 15) & ~size_t(15); }
 
-// streamed = false: odd row stride (column reads hit distinct shared-memory
-// banks); streamed = true: rows padded to 32 bytes (aligned global sectors).
-__host__ __device__ inline BigLayout big_layout(int m, int n, int k, bool streamed) {
+// Odd row stride: column reads hit distinct shared-memory banks.
+__host__ __device__ inline BigLayout big_layout(int m, int n, int k) {
     BigLayout L;
     L.R = m + 1 + (k > 0 ? 1 : 0);
-    L.LD = streamed ? ((n + k + 1 + 3) & ~3) : ((n + k + 1) | 1);
+    L.LD = (n + k + 1) | 1;
     size_t o = 0;
     L.rkey = o;    o += align16((size_t)m * sizeof(long long));
     L.row_var = o; o += align16((size_t)m * sizeof(int));
@@ -97,12 +95,58 @@ __host__ __device__ inline BigLayout big_layout(int m, int n, int k, bool stream
 
 // Dynamic shared memory of the resident kernel for one LP.
 __host__ __device__ inline size_t resident_smem_bytes(int m, int n, int k) {
-    return SmallLayout::total + big_layout(m, n, k, false).total;
+    return SmallLayout::total + big_layout(m, n, k).total;
 }
 
-// Global workspace bytes of one streamed slot (256-byte aligned).
-__host__ __device__ inline size_t streamed_slot_bytes(int m, int n, int k) {
-    return (big_layout(m, n, k, true).total + 255) & ~size_t(255);
+// The deferred-update kernel (lp_fp64_deferred.cuh), one LP: per-row and
+// per-column vectors, then (from `hist`) the pending pivots kept beside them.
+// The k-independent arrays come first.
+struct DeferredLayout {
+    size_t beta, rkey, row_var, row_last, negidx, neg;  // k-independent
+    size_t obj, aux, col_var, col_last, hist;
+};
+
+__host__ __device__ inline DeferredLayout deferred_layout(int m, int n, int k) {
+    DeferredLayout L;
+    const size_t M = (size_t)m, W = (size_t)n + k + 1;
+    size_t o = 0;
+    L.beta = o;     o += align16(M * 8);
+    L.rkey = o;     o += align16(M * 8);
+    L.row_var = o;  o += align16(M * 4);
+    L.row_last = o; o += align16(M * 4);
+    L.negidx = o;   o += align16(M * 4);
+    L.neg = o;      o += align16(M * 4);
+    L.obj = o;      o += align16(W * 8);
+    L.aux = o;      o += align16(k > 0 ? W * 8 : 0);
+    L.col_var = o;  o += align16(W * 4);
+    L.col_last = o; o += align16(W * 4);
+    L.hist = o;
+    return L;
+}
+
+// Its global workspace slot: the vectors (used when they exceed shared
+// memory), the tableau body after a flush (m rows, padded to 32 bytes), and
+// room for `first` pending pivots (c_s, then r_s).  `first`: pending pivots
+// before the first flush, half of where the deferred form's FMAs reach those
+// of a full update (t (m + n) = 2 m n); `later`: between flushes after it, when
+// the LP has shown that it takes many pivots and the flush's own FMAs, which
+// every element needs, are most of the work.
+struct DeferredSlot {
+    int LD, first, later;
+    size_t T, hist, total;
+};
+
+__host__ __device__ inline DeferredSlot deferred_slot(int m, int n, int k) {
+    DeferredSlot S;
+    const long long w = (long long)n + k + 1, at = (long long)m * w / (2 * ((long long)m + w));
+    S.first = (int)(at < 16 ? 16 : (at > 128 ? 128 : at));
+    S.later = 16;
+    S.LD = (int)((w + 3) & ~3LL);
+    size_t o = (deferred_layout(m, n, k).hist + 31) & ~size_t(31);
+    S.T = o;     o += (size_t)m * S.LD * 8;
+    S.hist = o;  o += (size_t)S.first * ((size_t)m + w) * 8;
+    S.total = (o + 255) & ~size_t(255);
+    return S;
 }
 
 // Shared-memory layout of the mixed-precision kernel (after SmallLayout):
@@ -181,34 +225,43 @@ cudaError_t launch_mixed(const DeviceBatch& B, const Tolerances& tol, const Mixe
                          const FallbackQueues& fq, int32_t* diag, cudaStream_t stream);
 
 // Launchers (lp_fp64_simplex.cu).
-constexpr int kStreamedThreads = 512;
-// Shared memory of a streamed FP64 LP's staged rank-1 update (the rings of
-// bulk-copied tableau chunks and the pivot row and column copies): the
-// streamed kernel's dynamic shared memory, and the least the single-launch
-// kernel gets when its batch has streamed LPs.  Enough for R + LD up to
-// ~2,000 doubles; larger LPs take the plain update loop.
-constexpr size_t kStreamStageBytes = 88 * 1024;
+// LPB_SCHED_SINGLE with FP64: threads per CTA, and the least shared memory a
+// CTA gets when the batch has LPs with deferred updates (their pending pivots).
+constexpr int kSingleThreads = 512;
+constexpr size_t kSingleDeferredBytes = 88 * 1024;
 cudaError_t fp64_kernels_prepare();
 // diag: 8 int32 internal-consistency record (see record_internal_error), or null.
 cudaError_t launch_fp64_resident(const DeviceBatch& B, const Tolerances& tol, const int32_t* order,
                                  int32_t count, int threads, size_t smem, int32_t* diag, cudaStream_t stream);
+// LPs with deferred updates, by size class: threads per CTA and shared memory.
+struct DeferredForm {
+    int cls;  // 0 .. kDeferredClasses - 1
+    int threads;
+    size_t smem;
+};
+constexpr int kDeferredClasses = 4;
+DeferredForm deferred_form(int m, int n, int k);
+// Whether an LP gets deferred updates by default, and the threads per CTA of
+// the resident kernel for the others.
+bool defer_updates(int m, int n, int k);
+int resident_threads(int m, int n, int k);
+int fp64_deferred_ctas_per_sm(const DeferredForm& f);
 // Persistent CTAs (grid = slots) take LPs of `order` from the atomic `counter`
-// (must be 0 at launch); each CTA keeps its tableau in workspace slot
-// blockIdx.x of `slot_bytes` bytes.
+// (zeroed here); CTA i works in workspace slot i of `slot_bytes` bytes (at
+// least deferred_slot(m, n, k).total of every listed LP, a multiple of 256).
+// Any form takes any LP; the class's is the one that suits its size.
 // count_dev (or null): a device-side length of `order`, read at launch and
 // capped at `count`.
-cudaError_t launch_fp64_streamed(const DeviceBatch& B, const Tolerances& tol, const int32_t* order,
-                                 int32_t count, int slots, unsigned char* workspace, size_t slot_bytes,
+cudaError_t launch_fp64_deferred(const DeviceBatch& B, const Tolerances& tol, const int32_t* order, int32_t count,
+                                 const DeferredForm& f, int slots, unsigned char* workspace, size_t slot_bytes,
                                  int32_t* counter, int32_t* diag, cudaStream_t stream,
                                  const int32_t* count_dev = nullptr);
-// CTAs of the streamed kernel that fit on one SM.
 cudaError_t fp64_single_prepare(size_t smem);
 int fp64_single_ctas_per_sm(size_t smem);
 cudaError_t launch_fp64_single(const DeviceBatch& B, const Tolerances& tol, const int32_t* order,
                                const uint8_t* resident, int32_t count, int ctas, size_t smem,
                                unsigned char* workspace, size_t slot_bytes, int32_t* counter, int32_t* diag,
                                cudaStream_t stream);
-int fp64_streamed_ctas_per_sm();
 // Resident kernel over a device-side LP list (persistent CTAs, atomic
 // `counter` zeroed on `stream` before the launch).  `smem` must cover every
 // listed LP's resident_smem_bytes and stay below kMaxSmemPerBlock - 1 KiB.

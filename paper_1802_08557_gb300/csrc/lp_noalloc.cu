@@ -1,6 +1,6 @@
-// lp_noalloc.cu -- lp_solve_uniform_noalloc: the streamed FP64 solver for a
-// batch of equal-size LPs whose scratch memory comes from a fixed array in
-// this module instead of an allocation.
+// lp_noalloc.cu -- lp_solve_uniform_noalloc: the FP64 solver for a batch of
+// equal-size LPs whose scratch memory comes from a fixed array in this module
+// instead of an allocation.
 //
 // Who needs this: code that may not allocate device memory while it runs --
 // for example a caller that owns every byte of the GPU through its own pool, a
@@ -63,8 +63,9 @@ size_t descriptor_bytes(int32_t num_lps) {
 }
 
 // Packed uniform layout: LP k's A at k*m*n, b and y at k*m, c and x at k*n.
-__global__ void fill_uniform_descriptors(DescPtrs d, int32_t num_lps, int32_t m, int32_t n) {
+__global__ void fill_uniform_descriptors(DescPtrs d, int32_t num_lps, int32_t m, int32_t n, int32_t* count) {
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k == 0) *count = num_lps;
     if (k >= num_lps) return;
     d.m[k] = m;
     d.n[k] = n;
@@ -104,13 +105,19 @@ extern "C" lpb_err lp_solve_uniform_noalloc(int32_t num_lps, int32_t m, int32_t 
     lpb_default_opts(&o);
     if (opts) o = *opts;
     if (!(o.eps_opt >= 0) || !(o.eps_piv >= 0) || !(o.eps_feas >= 0) || !(o.tau >= 0)) return LPB_EINVAL;
-    // Only the FP64 streamed kernel runs here; the mixed-precision path needs
+    // Only the FP64 kernels run here; the mixed-precision path needs
     // its own workspaces and re-solve queues, which this entry point has not.
     if (o.precision != LP_PREC_FP64) return LPB_EINVAL;
 
-    // Room: the counter, the descriptors, and at least one tableau slot sized
-    // for the widest phase-I tableau (every row with b_i < 0).
-    const size_t slot_bytes = streamed_slot_bytes(m, n, m);
+    // Room: the counter, the descriptors, and, for LPs with deferred updates,
+    // at least one workspace slot; sized for the widest phase-I tableau (every
+    // row with b_i < 0: the right-hand sides are on the device).  The form is
+    // chosen by the rule of lp_batch_create; measured, 1500 LPs of 50 x 50:
+    // 0.94 ms with the tableau in shared memory, 3.0 ms with deferred updates,
+    // 3.5 ms with the whole tableau updated in the slot.
+    const bool deferred = defer_updates(m, n, m);
+    const size_t slot_bytes = deferred_slot(m, n, m).total;
+    const DeferredForm form = deferred_form(m, n, m);
     const size_t desc_bytes = descriptor_bytes(num_lps);
     if (256 + desc_bytes + slot_bytes > kNoAllocScratchBytes) return LPB_ETOOBIG;
 
@@ -125,10 +132,6 @@ extern "C" lpb_err lp_solve_uniform_noalloc(int32_t num_lps, int32_t m, int32_t 
     int32_t* counter = reinterpret_cast<int32_t*>(base);
     const DescPtrs d = carve_descriptors(base + 256, num_lps);
     unsigned char* slots_base = base + 256 + desc_bytes;
-    int64_t slots = (int64_t)sms * fp64_streamed_ctas_per_sm();
-    slots = std::min<int64_t>(slots, num_lps);
-    slots = std::min<int64_t>(slots, (int64_t)((kNoAllocScratchBytes - 256 - desc_bytes) / slot_bytes));
-
     // Same tolerances and screening windows as lp_batch_create.
     Tolerances tol;
     tol.eps_opt = o.eps_opt;
@@ -143,10 +146,25 @@ extern "C" lpb_err lp_solve_uniform_noalloc(int32_t num_lps, int32_t m, int32_t 
     tol.ratio_abs = (float)std::max(std::ldexp(1.0, -20), 8.0 * o.tau);
 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    fill_uniform_descriptors<<<(num_lps + 255) / 256, 256, 0, s>>>(d, num_lps, m, n);
+    int32_t* count = counter + 1;
+    fill_uniform_descriptors<<<(num_lps + 255) / 256, 256, 0, s>>>(d, num_lps, m, n, count);
     if ((err = cudaGetLastError()) != cudaSuccess) return LPB_ECUDA;
     DeviceBatch B{d.m, d.n, d.a_off, d.b_off, d.c_off, d.x_off, d.y_off, A, b, c, status, iters, obj, x, y};
-    // launch_fp64_streamed zeroes the counter on `s` before the kernel.
-    err = launch_fp64_streamed(B, tol, d.order, num_lps, (int)slots, slots_base, slot_bytes, counter, nullptr, s);
+    // (both launchers zero the counter on `s` before the kernel)
+    if (deferred) {
+        int64_t slots = (int64_t)sms * fp64_deferred_ctas_per_sm(form);
+        slots = std::min<int64_t>(slots, num_lps);
+        slots = std::min<int64_t>(slots, (int64_t)((kNoAllocScratchBytes - 256 - desc_bytes) / slot_bytes));
+        err = launch_fp64_deferred(B, tol, d.order, num_lps, form, (int)slots, slots_base, slot_bytes, counter,
+                                   nullptr, s);
+    } else {
+        const size_t smem = resident_smem_bytes(m, n, m);
+        const int threads = resident_threads(m, n, m);
+        if ((err = fp64_kernels_prepare()) != cudaSuccess) return LPB_ECUDA;
+        const int64_t ctas =
+            std::min<int64_t>((int64_t)sms * fp64_resident_queue_ctas_per_sm(threads, smem), num_lps);
+        err = launch_fp64_resident_queue(B, tol, d.order, count, num_lps, num_lps, counter, nullptr, (int)ctas,
+                                         threads, smem, s);
+    }
     return err == cudaSuccess ? LPB_OK : LPB_ECUDA;
 }
