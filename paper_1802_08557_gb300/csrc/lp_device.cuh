@@ -110,6 +110,28 @@ __device__ __forceinline__ double tie_threshold(double v, double tau) {
     return __dadd_rn(v, __dmul_rn(tau, s));
 }
 
+// u / pe rounded to nearest, given y = 1 / pe rounded to nearest (one
+// reciprocal per pivot row instead of one inside every divide: 5 FP64
+// instructions per quotient, all on the FP64 pipe that bounds the kernel).
+// P. Markstein, IBM J. Res. Dev. 34 (1990): with y the rounded reciprocal and q
+// within one ulp of u / pe, fma(fma(-pe, q, u), y, q) is the rounded
+// quotient.  u y is within 1.5 ulp, so one such step brings it within one ulp
+// and a second one rounds it.  Exponents within 400 of zero keep every term
+// normal; others take the divide.  A zero u gives its signed zero: in the
+// divide a zero numerator leaves the fast path for the whole warp, and a
+// row can hold many.
+__device__ __forceinline__ double quotient(double u, double pe, double y) {
+    const int eu = dexp(u), ep = dexp(pe);
+    const bool zero = abskey(u) == 0 && ep <= 400;
+    const double v = zero ? 1.0 : u;
+    double q = __dmul_rn(v, y);
+    q = __fma_rn(__fma_rn(-pe, q, v), y, q);
+    q = __fma_rn(__fma_rn(-pe, q, v), y, q);
+    if (!(zero || (eu >= -400 && eu <= 400)) || ep < -400 || ep > 400) q = __ddiv_rn(u, pe);
+    const int sign = (__double2hiint(u) ^ __double2hiint(pe)) & INT_MIN;
+    return zero ? __hiloint2double(sign, 0) : q;
+}
+
 // Upper bound, in units of okey, of okey(thr) - okey(v) where thr is the tie
 // threshold v + tau*max(1,|v|) of a negative v (Step 1).  `wb` >=
 // tau*2^54*(1+2^-53) + 1.5 is precomputed on the host (< 0: no bound).  The

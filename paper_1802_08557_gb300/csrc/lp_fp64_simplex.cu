@@ -469,27 +469,30 @@ fp64_resident_queue_kernel(const DeviceBatch B, const Tolerances tol, const int3
 }
 
 
-// One LP with deferred updates: its vectors and first pending pivots in
-// `bytes` of shared memory when the vectors fit (phase I's, at their largest),
-// else in the workspace slot.
-__device__ __forceinline__ void deferred_one(const DeviceBatch& B, const Tolerances& tol, const int lp,
-                                             unsigned char* small, unsigned char* shared, const size_t bytes,
-                                             unsigned char* slot, int32_t* diag)
+// One LP of any size with deferred updates: its vectors and first pending
+// pivots in `bytes` of shared memory when the vectors fit (phase I's, at their
+// largest), else in the workspace slot.
+__device__ __forceinline__ void deferred_large(const DeviceBatch& B, const Tolerances& tol, const int lp,
+                                               unsigned char* small, unsigned char* shared, const size_t bytes,
+                                               unsigned char* slot, int32_t* diag)
 {
+    DeferBlock g(small);
     if (deferred_layout(B.m[lp], B.n[lp], B.m[lp]).hist <= bytes)
-        deferred_solve<true>(B, tol, lp, small, shared, bytes, slot, diag);
+        deferred_solve_large(g, B, tol, lp, shared, bytes, slot, diag);
     else
-        deferred_solve<false>(B, tol, lp, small, slot, 0, slot, diag);
+        deferred_solve_large(g, B, tol, lp, slot, 0, slot, diag);
 }
 
 // LPs whose tableau is not kept in shared memory (lp_fp64_deferred.cuh):
 // persistent CTAs take them from the atomic `counter`; CTA i owns workspace
-// slot i.
-__global__ void __launch_bounds__(kMaxThreads, 1)
-fp64_deferred_kernel(const DeviceBatch B, const Tolerances tol, const int32_t* __restrict__ order,
-                     const int32_t count, const int32_t* __restrict__ count_dev, unsigned char* workspace,
-                     const size_t slot_bytes, int32_t* __restrict__ counter, int32_t* __restrict__ diag,
-                     const size_t smem_bytes)
+// slot i.  One warp per LP, one CTA per LP, and one CTA per LP of any size.
+enum DeferredKind { kDeferOneWarp, kDeferCta, kDeferLarge };
+template <DeferredKind kKind>
+__device__ __forceinline__ void deferred_queue(const DeviceBatch& B, const Tolerances& tol,
+                                               const int32_t* __restrict__ order, const int32_t count,
+                                               const int32_t* __restrict__ count_dev, unsigned char* workspace,
+                                               const size_t slot_bytes, int32_t* __restrict__ counter,
+                                               int32_t* __restrict__ diag, const size_t smem_bytes)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int next;
@@ -501,9 +504,45 @@ fp64_deferred_kernel(const DeviceBatch B, const Tolerances tol, const int32_t* _
         const int idx = next;
         __syncthreads();
         if (idx >= n_items) break;
-        deferred_one(B, tol, order[idx], smem, smem + SmallLayout::total, smem_bytes - SmallLayout::total, slot, diag);
+        const int lp = order[idx];
+        if constexpr (kKind == kDeferOneWarp) {
+            DeferWarp g;
+            deferred_solve(g, B, tol, lp, smem, smem_bytes, slot, diag);
+        } else if constexpr (kKind == kDeferCta) {
+            DeferBlock g(smem);
+            deferred_solve(g, B, tol, lp, smem + SmallLayout::total, smem_bytes - SmallLayout::total, slot, diag);
+        } else {
+            deferred_large(B, tol, lp, smem, smem + SmallLayout::total, smem_bytes - SmallLayout::total, slot, diag);
+        }
         __syncthreads();
     }
+}
+
+__global__ void __maxnreg__(80)
+fp64_deferred_warp_kernel(const DeviceBatch B, const Tolerances tol, const int32_t* __restrict__ order,
+                          const int32_t count, const int32_t* __restrict__ count_dev, unsigned char* workspace,
+                          const size_t slot_bytes, int32_t* __restrict__ counter, int32_t* __restrict__ diag,
+                          const size_t smem_bytes)
+{
+    deferred_queue<kDeferOneWarp>(B, tol, order, count, count_dev, workspace, slot_bytes, counter, diag, smem_bytes);
+}
+
+__global__ void __maxnreg__(80)
+fp64_deferred_kernel(const DeviceBatch B, const Tolerances tol, const int32_t* __restrict__ order,
+                     const int32_t count, const int32_t* __restrict__ count_dev, unsigned char* workspace,
+                     const size_t slot_bytes, int32_t* __restrict__ counter, int32_t* __restrict__ diag,
+                     const size_t smem_bytes)
+{
+    deferred_queue<kDeferCta>(B, tol, order, count, count_dev, workspace, slot_bytes, counter, diag, smem_bytes);
+}
+
+__global__ void __launch_bounds__(kMaxThreads, 2)
+fp64_deferred_large_kernel(const DeviceBatch B, const Tolerances tol, const int32_t* __restrict__ order,
+                           const int32_t count, const int32_t* __restrict__ count_dev, unsigned char* workspace,
+                           const size_t slot_bytes, int32_t* __restrict__ counter, int32_t* __restrict__ diag,
+                           const size_t smem_bytes)
+{
+    deferred_queue<kDeferLarge>(B, tol, order, count, count_dev, workspace, slot_bytes, counter, diag, smem_bytes);
 }
 
 // A whole batch in one launch: persistent CTAs take the LPs order[0 ..
@@ -530,7 +569,7 @@ fp64_single_kernel(const DeviceBatch B, const Tolerances tol, const int32_t* __r
         if (resident[lp]) {
             solve_one(B, tol, lp, smem, smem + SmallLayout::total, diag);
         } else if (slot) {
-            deferred_one(B, tol, lp, smem, smem + SmallLayout::total, smem_bytes - SmallLayout::total, slot, diag);
+            deferred_large(B, tol, lp, smem, smem + SmallLayout::total, smem_bytes - SmallLayout::total, slot, diag);
         } else if (threadIdx.x == 0) {
             record_internal_error(diag, 7, lp);  // a plan without a slot for a streamed LP
         }
@@ -568,15 +607,19 @@ cudaError_t launch_fp64_resident_queue(const DeviceBatch& B, const Tolerances& t
     return cudaGetLastError();
 }
 
-// Deferred updates for every tableau above one CTA's shared memory, and for
-// tableaux of more than 14,000 entries: at 130 x 130 they win whatever the
-// number of pivots (2000 mixed-sign LPs, 326 pivots: 34.1 against 37.5 ms in
-// shared memory; positive 200 x 200, 25 pivots: 2.6 against 3.9 ms); at 100 x 100
-// they lose on many pivots (mixed-sign, 200 pivots: 19.3 against 18.5 ms) and
-// win on few (positive, 15 pivots: 0.73 against 1.26 ms), and the number of
-// pivots is not known beforehand.
-bool defer_updates(int m, int n, int k) {
-    return resident_smem_bytes(m, n, k) > kMaxSmemPerBlock || (int64_t)(m + 1) * (n + k + 1) > 14000;
+// Deferred updates for every tableau above one CTA's shared memory, and below
+// that by size.  The number of pivots decides, and is not known beforehand; a
+// packing LP (no negative entry in A) takes few.  Measured, positive LPs,
+// deferred against resident, ms: 45 x 45 0.38 / 0.44, 40 x 60 0.41 / 0.53, 130 x 60
+// 0.99 / 1.19, 130 x 130 1.04 / 2.02, but 30 x 70 0.54 / 0.50, 16 x 130 0.97 / 0.56
+// (few elements per pivot row or column: the pivot's fixed cost counts) and
+// 20 x 20 0.22 / 0.20.  Other LPs, mixed signs: 130 x 130 (326 pivots) 34.7 / 37.5,
+// 100 x 100 (200 pivots) 20.3 / 18.5, 70 x 70 11.5 / 8.1.
+bool defer_updates(int m, int n, int k, bool nonneg) {
+    if (resident_smem_bytes(m, n, k) > kMaxSmemPerBlock) return true;
+    const int64_t e = (int64_t)(m + 1) * (n + k + 1);
+    if (nonneg && e > kDeferNonneg && m >= 32 && n >= 32) return true;
+    return e > 14000;
 }
 
 int resident_threads(int m, int n, int k) {
@@ -589,25 +632,34 @@ int resident_threads(int m, int n, int k) {
     return 512;
 }
 
-// Size classes by the length of a row and a column together: few threads for
-// small LPs (more LPs per SM; a pivot's work is one row and one column), more
-// pending pivots in shared memory for large ones.  256 threads instead of 512
-// in class 2: 20,000 uneven LPs 3.6 against 4.1 ms, but 300 mixed-sign
-// LPs of 300 x 300 (long runs of pivots, where the flushes are the work)
-// 215 against 148 ms.
-DeferredForm deferred_form(int m, int n, int k) {
-    const int w = m + n + k;
-    if (w <= 192) return {0, 64, 24 << 10};
-    if (w <= 448) return {1, 128, 44 << 10};
-    if (w <= 2048) return {2, 512, 100 << 10};
-    return {3, 512, kMaxSmemPerBlock - 1024};
+// Size classes by the longer of a row and a column, d: a thread for each up to
+// 256 (a warp's FP64 instruction holds its quarter of the SM's FP64 pipe for 64
+// clocks, so one LP needs its elements spread over warps), 9 KB of shared memory
+// per warp, 24 warps per SM at 80 registers.  Above, several per thread: 256
+// threads and three CTAs per SM suit short runs of pivots (20,000 uneven packing
+// LPs 2.7 against 3.2 ms with 512), 512 threads the flushes of long ones (300
+// mixed-sign 300 x 300 LPs 179 against 238 ms).
+DeferredForm deferred_form(int m, int n, int k, bool nonneg) {
+    const int d = m > n + k + 1 ? m : n + k + 1;
+    for (int c = 0; c < 4; ++c)
+        if (d <= (32 << c)) return {c, 32 << c, (size_t)(9 << 10) << c};
+    if (d <= 1024) return nonneg ? DeferredForm{4, 256, 74 << 10} : DeferredForm{5, 512, 100 << 10};
+    return {6, kMaxThreads, kMaxSmemPerBlock - 1024};
 }
+
+namespace {
+using DeferredKernel = void (*)(const DeviceBatch, const Tolerances, const int32_t*, const int32_t, const int32_t*,
+                                unsigned char*, const size_t, int32_t*, int32_t*, const size_t);
+DeferredKernel deferred_kernel(const DeferredForm& f) {
+    return f.cls == 0 ? fp64_deferred_warp_kernel : (f.cls < 4 ? fp64_deferred_kernel : fp64_deferred_large_kernel);
+}
+}  // namespace
 
 int fp64_deferred_ctas_per_sm(const DeferredForm& f) {
     int blocks = 0;
-    if (cudaFuncSetAttribute(fp64_deferred_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (cudaFuncSetAttribute(deferred_kernel(f), cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)(kMaxSmemPerBlock - 1024)) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, fp64_deferred_kernel, f.threads, f.smem) != cudaSuccess)
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, deferred_kernel(f), f.threads, f.smem) != cudaSuccess)
         return 1;
     return blocks > 0 ? blocks : 1;
 }
@@ -618,11 +670,11 @@ cudaError_t launch_fp64_deferred(const DeviceBatch& B, const Tolerances& tol, co
     if (count <= 0) return cudaSuccess;
     cudaError_t err = cudaMemsetAsync(counter, 0, sizeof(int32_t), stream);
     if (err != cudaSuccess) return err;
-    if ((err = cudaFuncSetAttribute(fp64_deferred_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if ((err = cudaFuncSetAttribute(deferred_kernel(f), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)(kMaxSmemPerBlock - 1024))) != cudaSuccess)
         return err;
-    fp64_deferred_kernel<<<slots, f.threads, f.smem, stream>>>(B, tol, order, count, count_dev, workspace, slot_bytes,
-                                                               counter, diag, f.smem);
+    deferred_kernel(f)<<<slots, f.threads, f.smem, stream>>>(B, tol, order, count, count_dev, workspace, slot_bytes,
+                                                             counter, diag, f.smem);
     return cudaGetLastError();
 }
 

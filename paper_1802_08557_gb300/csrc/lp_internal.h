@@ -98,11 +98,11 @@ __host__ __device__ inline size_t resident_smem_bytes(int m, int n, int k) {
     return SmallLayout::total + big_layout(m, n, k).total;
 }
 
-// The deferred-update kernel (lp_fp64_deferred.cuh), one LP: per-row and
-// per-column vectors, then (from `hist`) the pending pivots kept beside them.
+// deferred_solve_large (lp_fp64_deferred.cuh): per-row and per-column vectors,
+// then (from `hist`) the pending pivots kept beside them.
 // The k-independent arrays come first.
 struct DeferredLayout {
-    size_t beta, rkey, row_var, row_last, negidx, neg;  // k-independent
+    size_t recip, beta, code, row_var, row_last, negidx, neg;  // k-independent
     size_t obj, aux, col_var, col_last, hist;
 };
 
@@ -110,8 +110,9 @@ __host__ __device__ inline DeferredLayout deferred_layout(int m, int n, int k) {
     DeferredLayout L;
     const size_t M = (size_t)m, W = (size_t)n + k + 1;
     size_t o = 0;
+    L.recip = o;    o += 16;
     L.beta = o;     o += align16(M * 8);
-    L.rkey = o;     o += align16(M * 8);
+    L.code = o;     o += align16(M * 4);
     L.row_var = o;  o += align16(M * 4);
     L.row_last = o; o += align16(M * 4);
     L.negidx = o;   o += align16(M * 4);
@@ -119,6 +120,25 @@ __host__ __device__ inline DeferredLayout deferred_layout(int m, int n, int k) {
     L.obj = o;      o += align16(W * 8);
     L.aux = o;      o += align16(k > 0 ? W * 8 : 0);
     L.col_var = o;  o += align16(W * 4);
+    L.col_last = o; o += align16(W * 4);
+    L.hist = o;
+    return L;
+}
+
+// deferred_solve: an owner's messages (4 doubles, 4 ints), the negated rows
+// (bits, list) and the restart points; the rest is in registers.
+struct DeferredRegLayout {
+    size_t box, negbits, neg, row_last;  // k-independent
+    size_t col_last, hist;
+};
+__host__ __device__ inline DeferredRegLayout deferred_reg_layout(int m, int n, int k) {
+    DeferredRegLayout L;
+    const size_t M = (size_t)m, W = (size_t)n + k + 1;
+    size_t o = 0;
+    L.box = o;      o += 48;
+    L.negbits = o;  o += align16((M + 31) / 32 * 4);
+    L.neg = o;      o += align16(M * 4);
+    L.row_last = o; o += align16(M * 4);
     L.col_last = o; o += align16(W * 4);
     L.hist = o;
     return L;
@@ -239,17 +259,22 @@ struct DeferredForm {
     int threads;
     size_t smem;
 };
-constexpr int kDeferredClasses = 4;
-DeferredForm deferred_form(int m, int n, int k);
+constexpr int kDeferredClasses = 7;
+DeferredForm deferred_form(int m, int n, int k, bool nonneg);
 // Whether an LP gets deferred updates by default, and the threads per CTA of
-// the resident kernel for the others.
-bool defer_updates(int m, int n, int k);
+// the resident kernel for the others.  nonneg: no negative entry was seen in A;
+// a packing LP takes few pivots.
+bool defer_updates(int m, int n, int k, bool nonneg);
+constexpr int64_t kDeferNonneg = 2000;  // least tableau entries of such an LP's deferred updates
+__host__ __device__ inline bool sign_matters(int m, int n) {
+    return (int64_t)(m + 1) * (n + 1) > kDeferNonneg && m >= 32 && n >= 32;
+}
 int resident_threads(int m, int n, int k);
 int fp64_deferred_ctas_per_sm(const DeferredForm& f);
 // Persistent CTAs (grid = slots) take LPs of `order` from the atomic `counter`
 // (zeroed here); CTA i works in workspace slot i of `slot_bytes` bytes (at
 // least deferred_slot(m, n, k).total of every listed LP, a multiple of 256).
-// Any form takes any LP; the class's is the one that suits its size.
+// A form takes the LPs of its class and of the classes below.
 // count_dev (or null): a device-side length of `order`, read at launch and
 // capped at `count`.
 cudaError_t launch_fp64_deferred(const DeviceBatch& B, const Tolerances& tol, const int32_t* order, int32_t count,
@@ -381,7 +406,12 @@ cudaError_t launch_hyperbox(const double* L, const double* lo, const double* hi,
 // non-finite entries, each of which is set to 0.
 cudaError_t launch_input_check(double* A, int64_t a_len, double* b, int64_t b_len, double* c, int64_t c_len,
                                unsigned long long* bad, cudaStream_t stream);
-// k[lp] = the number of rows of LP lp with b_i < 0 (rows that get an artificial).
-cudaError_t launch_count_negative_rhs(const DeviceBatch& B, int32_t num_lps, int32_t* k, cudaStream_t stream);
+// info[lp] = the number of rows of LP lp with b_i < 0 (rows that get an
+// artificial), plus kPlanSigned unless a sample of A has no negative entry,
+// plus kPlanSameA if A is the previous LP's (kPlanSigned is then that LP's).
+// The sign is looked for with want_sign, and only where sign_matters.
+constexpr int32_t kPlanSigned = 1 << 30, kPlanSameA = 1 << 29;
+cudaError_t launch_plan_info(const DeviceBatch& B, int32_t num_lps, bool want_sign, int32_t* info,
+                             cudaStream_t stream);
 
 }  // namespace lpb

@@ -115,9 +115,9 @@ extern "C" lpb_err lp_solve_uniform_noalloc(int32_t num_lps, int32_t m, int32_t 
     // chosen by the rule of lp_batch_create; measured, 1500 LPs of 50 x 50:
     // 0.94 ms with the tableau in shared memory, 3.0 ms with deferred updates,
     // 3.5 ms with the whole tableau updated in the slot.
-    const bool deferred = defer_updates(m, n, m);
+    const bool deferred = defer_updates(m, n, m, false);
     const size_t slot_bytes = deferred_slot(m, n, m).total;
-    const DeferredForm form = deferred_form(m, n, m);
+    const DeferredForm form = deferred_form(m, n, m, false);
     const size_t desc_bytes = descriptor_bytes(num_lps);
     if (256 + desc_bytes + slot_bytes > kNoAllocScratchBytes) return LPB_ETOOBIG;
 
