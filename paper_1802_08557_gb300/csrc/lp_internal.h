@@ -414,4 +414,14 @@ constexpr int32_t kPlanSigned = 1 << 30, kPlanSameA = 1 << 29;
 cudaError_t launch_plan_info(const DeviceBatch& B, int32_t num_lps, bool want_sign, int32_t* info,
                              cudaStream_t stream);
 
+// Up to five arrays copied device to device in one launch (lp_batch_results);
+// sizes multiples of 4 bytes, addresses 4-byte aligned.
+struct CopyList {
+    void* dst[5];
+    const void* src[5];
+    size_t bytes[5];
+    int count;
+};
+cudaError_t launch_copy_list(const CopyList& list, cudaStream_t stream);
+
 }  // namespace lpb

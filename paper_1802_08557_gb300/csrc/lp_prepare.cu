@@ -62,6 +62,27 @@ __global__ void plan_info_kernel(const DeviceBatch B, int32_t num_lps, bool want
     if (lane == 0) info[lp] = cnt | flags;
 }
 
+// Array blockIdx.y of the list, in 16-byte pieces where both ends allow it.
+// Bound by the launch for small batches (five separate copies were most of a
+// 5 x 5 batch's results), by HBM for large ones.
+__global__ void __launch_bounds__(256) copy_list_kernel(const __grid_constant__ CopyList list) {
+    const int a = blockIdx.y;
+    const size_t stride = (size_t)gridDim.x * blockDim.x, t0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const size_t bytes = list.bytes[a];
+    size_t done = 0;
+    if (((reinterpret_cast<uintptr_t>(list.dst[a]) | reinterpret_cast<uintptr_t>(list.src[a])) & 15u) == 0) {
+        const uint4* src = static_cast<const uint4*>(list.src[a]);
+        uint4* dst = static_cast<uint4*>(list.dst[a]);
+        const size_t n = bytes / 16;
+#pragma unroll 4
+        for (size_t i = t0; i < n; i += stride) dst[i] = src[i];
+        done = n * 4;
+    }
+    const uint32_t* src = static_cast<const uint32_t*>(list.src[a]);
+    uint32_t* dst = static_cast<uint32_t*>(list.dst[a]);
+    for (size_t i = done + t0; i < bytes / 4; i += stride) dst[i] = src[i];
+}
+
 int grid_for(int64_t len, int threads) {
     int64_t g = (len + threads * 4 - 1) / (threads * 4);
     if (g < 1) g = 1;
@@ -87,6 +108,16 @@ cudaError_t launch_plan_info(const DeviceBatch& B, int32_t num_lps, bool want_si
     const int t = 256;
     const int64_t threads = (int64_t)num_lps * 32;
     plan_info_kernel<<<(unsigned)((threads + t - 1) / t), t, 0, stream>>>(B, num_lps, want_sign, info);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_copy_list(const CopyList& list, cudaStream_t stream) {
+    size_t most = 0;
+    for (int i = 0; i < list.count; ++i) most = list.bytes[i] > most ? list.bytes[i] : most;
+    // four 16-byte pieces per thread, at most two waves of CTAs
+    const size_t blocks = (most + 16383) / 16384;
+    copy_list_kernel<<<dim3((unsigned)(blocks < 1 ? 1 : (blocks > 1216 ? 1216 : blocks)), list.count), 256, 0, stream>>>(
+        list);
     return cudaGetLastError();
 }
 
