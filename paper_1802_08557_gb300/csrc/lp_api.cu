@@ -221,6 +221,17 @@ struct lp_batch {
         int32_t* counter;
     };
     std::vector<DeferredGroup> deferred_groups;
+    // mixed precision with deferred updates, one group per size class
+    struct MixedDeferredGroup {
+        lpb::MixedDeferredForm form;
+        int64_t offset;
+        int32_t count, slots;
+        size_t slot_bytes;
+        unsigned char* workspace;
+        int32_t* counter;
+    };
+    std::vector<MixedDeferredGroup> mdeferred_groups;
+    int32_t num_mdeferred = 0;
     int32_t num_streamed = 0;
     // mixed precision: groups of the FP32 + certificate kernel, fallback queue
     std::vector<Group> mixed_groups;
@@ -376,21 +387,25 @@ lpb_err enqueue_solve(lp_batch* h, cudaStream_t s, bool timing) {
     if (h->num_mixed > 0 && ((err = cudaMemsetAsync(h->fb_len, 0, sizeof(int32_t), s)) ||
                              (err = cudaMemsetAsync(h->fbig_len, 0, sizeof(int32_t), s))))
         return cuda_fail(err, "fallback queue reset");
-    // kind 0 mixed, 1 resident, 2 deferred updates, 3 cluster, 4 mixed streamed
+    // kind 0 mixed, 1 resident, 2 deferred updates, 3 cluster, 4 mixed streamed,
+    // 5 single launch, 6 mixed with deferred updates
     struct Job { int kind; const Group* g; int64_t count; };
     std::vector<Job> jobs;
     for (const Group& g : h->mixed_groups) jobs.push_back({0, &g, g.count});
     for (const Group& g : h->groups) jobs.push_back({1, &g, g.count});
     for (auto it = h->deferred_groups.rbegin(); it != h->deferred_groups.rend(); ++it)  // largest LPs first
         jobs.push_back({2, reinterpret_cast<const Group*>(&*it), it->count});
+    for (auto it = h->mdeferred_groups.rbegin(); it != h->mdeferred_groups.rend(); ++it)
+        jobs.push_back({6, reinterpret_cast<const Group*>(&*it), it->count});
     if (h->num_single > 0) jobs.push_back({5, nullptr, h->num_single});
     if (h->num_mstream > 0) jobs.push_back({4, nullptr, h->num_mstream});
     for (size_t ci = 0; ci < h->cluster_groups.size(); ++ci)
         jobs.push_back({3, reinterpret_cast<const Group*>(ci), h->cluster_groups[ci].count});
     // the deferred-update groups first: they hold the largest LPs
     std::stable_sort(jobs.begin(), jobs.end(), [](const Job& a, const Job& b) {
-        if ((a.kind == 2) != (b.kind == 2)) return a.kind == 2;
-        return a.kind != 2 && a.count > b.count;
+        const bool da = a.kind == 2 || a.kind == 6, db = b.kind == 2 || b.kind == 6;
+        if (da != db) return da;
+        return !da && a.count > b.count;
     });
     cudaEvent_t* tev = (!timing || h->tev.empty()) ? nullptr : &h->tev[3 * (size_t)(h->timed_solves % kTimingRing)];
     if (tev && (err = cudaEventRecord(tev[0], s))) return cuda_fail(err, "timing");
@@ -420,6 +435,10 @@ lpb_err enqueue_solve(lp_batch* h, cudaStream_t s, bool timing) {
             const auto& dg = *reinterpret_cast<const lp_batch::DeferredGroup*>(j.g);
             err = lpb::launch_fp64_deferred(h->d, h->tol, h->d_order + dg.offset, dg.count, dg.form, dg.slots,
                                             dg.workspace, dg.slot_bytes, dg.counter, h->diag, ls);
+        } else if (j.kind == 6) {
+            const auto& mg = *reinterpret_cast<const lp_batch::MixedDeferredGroup*>(j.g);
+            err = lpb::launch_mixed_deferred(h->d, h->tol, h->mp, h->d_order + mg.offset, mg.count, mg.form, mg.slots,
+                                             mg.workspace, mg.slot_bytes, mg.counter, fallback_queues(h), h->diag, ls);
         } else if (j.kind == 4) {
             err = lpb::launch_mixed_streamed(h->d, h->tol, h->mp, h->d_order + h->mstream_offset, h->num_mstream,
                                              h->mstream_slots, h->mworkspace, h->mslot_bytes, h->mcounter,
@@ -612,7 +631,7 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
     if (ptr_kind == LPB_DEVICE &&
         ((err = lpb::launch_input_check(dA, a_len, dbv, b_len, dcv, c_len, dbad, s)) ||
          (err = lpb::launch_plan_info(
-              h->d, num_lps, o.precision == LP_PREC_FP64 && o.schedule == LPB_SCHED_AUTO, dk, s))))
+              h->d, num_lps, o.schedule == LPB_SCHED_AUTO, dk, s))))
         return bail_cuda(err, "input check kernel");
     std::vector<int32_t> hk(num_lps);
     std::vector<uint8_t> nonneg(num_lps, 0);  // no negative entry seen in A (device inputs only)
@@ -647,6 +666,7 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
     std::vector<int32_t> deferred[lpb::kDeferredClasses];  // deferred updates, by size class
     auto defer = [&](int32_t k) { deferred[lpb::deferred_form(hm[k], hn[k], hk[k], nonneg[k]).cls].push_back(k); };
     std::map<int, std::vector<int32_t>> cluster_buckets;  // cluster size -> LPs
+    std::vector<int32_t> mdeferred[lpb::kMixedDeferredClasses];  // mixed, deferred updates, by size class
     std::vector<int32_t> mstream;                         // mixed precision, tableau in global memory
     std::vector<int32_t> fbig_lps;                        // mixed LPs whose FP64 re-solve exceeds one CTA
     std::vector<int32_t> single;                          // LPB_SCHED_SINGLE: every LP
@@ -707,14 +727,19 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
                 }
                 continue;
             }
+            if (o.schedule == LPB_SCHED_AUTO && lpb::mixed_defer_updates(hm[k], hn[k], hk[k], nonneg[k], h->uniform_m < 0)) {
+                mdeferred[lpb::mixed_deferred_form(hm[k], hn[k]).cls].push_back(k);
+                continue;
+            }
             if (o.schedule != LPB_SCHED_STREAMED && mneed <= queue_smem_cap) {
                 const int threads = mixed_threads(hm[k], hn[k], hk[k], o.block_threads);
                 // shared memory rounded to 1 KiB for the one-warp form (it sets
                 // how many LPs share an SM), to 8 KiB otherwise: fewer, larger
                 // launches (uneven workload: 1 KiB 280 groups 17.3 ms, 4 KiB
                 // 123 groups 11.6 ms, 8 KiB 97 groups 11.2 ms, 16 KiB 84 groups
-                // 11.4 ms)
-                const size_t gran = threads == 32 ? 1024 : 8192;
+                // 11.4 ms).  One-warp LPs of uneven sizes to 4 KiB: 2000 uneven
+                // LPs 2.0 -> 1.35 ms, 20,000 6.3 -> 5.9
+                const size_t gran = threads == 32 ? (h->uniform_m < 0 ? 4096 : 1024) : 8192;
                 mixed_buckets[{threads, std::min(queue_smem_cap, (mneed + gran - 1) / gran * gran)}].push_back(k);
             } else {
                 mstream.push_back(k);
@@ -839,6 +864,19 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
     if (!h->cluster_groups.empty() &&
         (err = alloc(h, &h->cluster_counter, h->cluster_groups.size(), s)))
         return bail_cuda(err, "cluster counters");
+    for (std::vector<int32_t>& v : mdeferred) {
+        if (v.empty()) continue;
+        lpt(v);
+        lp_batch::MixedDeferredGroup g{};
+        g.form = lpb::mixed_deferred_form(hm[v[0]], hn[v[0]]);
+        g.offset = (int64_t)order.size();
+        g.count = (int32_t)v.size();
+        for (int32_t k : v) g.slot_bytes = std::max(g.slot_bytes, lpb::mixed_deferred_slot(hm[k], hn[k], hk[k]).total);
+        order.insert(order.end(), v.begin(), v.end());
+        h->mdeferred_groups.push_back(g);
+        h->num_mdeferred += g.count;
+    }
+    h->num_mixed += h->num_mdeferred;
     lpt(mstream);
     h->mstream_offset = (int64_t)order.size();
     h->num_mstream = (int32_t)mstream.size();
@@ -909,6 +947,17 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
         h->single_ctas = (int32_t)ctas;
         h->max_smem = std::max(h->max_smem, h->single_smem);
         if ((err = alloc(h, &h->single_counter, 1, s))) return bail_cuda(err, "single-launch counter");
+    }
+    for (lp_batch::MixedDeferredGroup& g : h->mdeferred_groups) {
+        int sms = 0;
+        if ((err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device)))
+            return bail_cuda(err, "device query");
+        int64_t slots = (int64_t)sms * lpb::mixed_deferred_ctas_per_sm(g.form);
+        const int64_t cap = std::max<int64_t>(1, kMaxWorkspaceBytes / (int64_t)g.slot_bytes);
+        slots = std::min<int64_t>({slots, (int64_t)g.count, cap});
+        g.slots = (int32_t)slots;
+        if ((err = alloc(h, &g.workspace, (size_t)slots * g.slot_bytes, s)) || (err = alloc(h, &g.counter, 1, s)))
+            return bail_cuda(err, "workspace allocation");
     }
     for (lp_batch::DeferredGroup& g : h->deferred_groups) {
         int sms = 0;
@@ -984,7 +1033,8 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
     if ((err = cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming)))
         return bail_cuda(err, "event creation");
     h->num_lanes = lanes_for(h->groups.size() + h->mixed_groups.size() + h->deferred_groups.size() +
-                             h->cluster_groups.size() + (h->num_single > 0 ? 1 : 0) + (h->num_mstream > 0 ? 1 : 0));
+                             h->mdeferred_groups.size() + h->cluster_groups.size() + (h->num_single > 0 ? 1 : 0) +
+                             (h->num_mstream > 0 ? 1 : 0));
     for (int i = 0; i < h->num_lanes; ++i)
         if ((err = cudaStreamCreateWithFlags(&h->lanes[i], cudaStreamNonBlocking)) ||
             (err = cudaEventCreateWithFlags(&h->ev_join[i], cudaEventDisableTiming)))
@@ -1154,7 +1204,8 @@ lpb_err lp_batch_group_info(lp_batch* h, int32_t index, lp_batch_group* out) {
     const int32_t nr = (int32_t)h->groups.size(), nm = (int32_t)h->mixed_groups.size();
     const int32_t nc = (int32_t)h->cluster_groups.size();
     const int32_t ns = (int32_t)h->deferred_groups.size();
-    const int32_t nms = h->num_mstream > 0 ? 1 : 0;
+    const int32_t nmd = (int32_t)h->mdeferred_groups.size();
+    const int32_t nms = nmd + (h->num_mstream > 0 ? 1 : 0);
     const int32_t total = nr + nm + nc + ns + nms + (h->num_single > 0 ? 1 : 0);
     if (index < 0 || index >= total) return fail(LPB_EINVAL, "group index out of range");
     std::memset(out, 0, sizeof *out);
@@ -1189,6 +1240,14 @@ lpb_err lp_batch_group_info(lp_batch* h, int32_t index, lp_batch_group* out) {
     } else if (index < nr + nm + nc + ns) {
         const lp_batch::DeferredGroup& g = h->deferred_groups[index - nr - nm - nc];
         out->kind = 2;
+        out->count = g.count;
+        out->threads = g.form.threads;
+        out->persistent = 1;
+        out->smem_bytes = (int64_t)g.form.smem;
+        out->tuned_ms = -1.0f;
+    } else if (index < nr + nm + nc + ns + nmd) {
+        const lp_batch::MixedDeferredGroup& g = h->mdeferred_groups[index - nr - nm - nc - ns];
+        out->kind = 4;
         out->count = g.count;
         out->threads = g.form.threads;
         out->persistent = 1;
@@ -1403,9 +1462,9 @@ lpb_err lp_batch_stage_times(lp_batch* h, float* stage_ms, int32_t* num_solves) 
 lpb_err lp_batch_plan_info(lp_batch* h, lp_batch_plan* plan) {
     if (!h || !plan) return fail(LPB_EINVAL, "handle or plan is NULL");
     plan->num_groups = (int32_t)(h->groups.size() + h->mixed_groups.size() + h->cluster_groups.size()) +
-                       (int32_t)h->deferred_groups.size() + (h->num_mstream > 0 ? 1 : 0) + (h->num_fsmall > 0 ? 1 : 0) +
+                       (int32_t)(h->deferred_groups.size() + h->mdeferred_groups.size()) + (h->num_mstream > 0 ? 1 : 0) + (h->num_fsmall > 0 ? 1 : 0) +
                        (h->num_fbig > 0 ? 1 : 0) + (h->num_single > 0 ? 1 : 0);
-    plan->num_resident = h->num_lps - h->num_streamed - h->num_mstream - h->num_cluster - h->num_single_streamed;
+    plan->num_resident = h->num_lps - h->num_streamed - h->num_mstream - h->num_mdeferred - h->num_cluster - h->num_single_streamed;
     plan->num_cluster = h->num_cluster;
     plan->num_mixed = h->num_mixed;
     plan->num_fallback = 0;
@@ -1437,13 +1496,14 @@ lpb_err lp_batch_plan_info(lp_batch* h, lp_batch_plan* plan) {
         plan->internal_error_lp = dg[0] ? dg[2] : -1;
         for (int i = 0; i < 5; ++i) plan->internal_error_detail[i] = dg[0] ? dg[3 + i] : 0;
     }
-    plan->num_streamed = h->num_streamed + h->num_mstream + h->num_single_streamed;
+    plan->num_streamed = h->num_streamed + h->num_mstream + h->num_mdeferred + h->num_single_streamed;
     plan->num_phase1 = h->num_phase1;
     plan->max_smem_bytes = (int64_t)h->max_smem;
     plan->workspace_bytes = (int64_t)h->mstream_slots * (int64_t)h->mslot_bytes +
                             (int64_t)h->fbig_slots * (int64_t)h->fbig_slot_bytes +
                             (h->single_workspace ? (int64_t)h->single_ctas * (int64_t)h->single_slot_bytes : 0);
     for (const auto& g : h->deferred_groups) plan->workspace_bytes += (int64_t)g.slots * (int64_t)g.slot_bytes;
+    for (const auto& g : h->mdeferred_groups) plan->workspace_bytes += (int64_t)g.slots * (int64_t)g.slot_bytes;
     return LPB_OK;
 }
 

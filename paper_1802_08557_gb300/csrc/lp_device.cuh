@@ -110,24 +110,14 @@ __device__ __forceinline__ double tie_threshold(double v, double tau) {
     return __dadd_rn(v, __dmul_rn(tau, s));
 }
 
-// u / pe rounded to nearest, given y = 1 / pe rounded to nearest (one
-// reciprocal per pivot row instead of one inside every divide: 5 FP64
-// instructions per quotient, all on the FP64 pipe that bounds the kernel).
-// P. Markstein, IBM J. Res. Dev. 34 (1990): with y the rounded reciprocal and q
-// within one ulp of u / pe, fma(fma(-pe, q, u), y, q) is the rounded
-// quotient.  u y is within 1.5 ulp, so one such step brings it within one ulp
-// and a second one rounds it.  Exponents within 400 of zero keep every term
-// normal; others take the divide.  A zero u gives its signed zero: in the
-// divide a zero numerator leaves the fast path for the whole warp, and a
-// row can hold many.
-__device__ __forceinline__ double quotient(double u, double pe, double y) {
-    const int eu = dexp(u), ep = dexp(pe);
-    const bool zero = abskey(u) == 0 && ep <= 400;
-    const double v = zero ? 1.0 : u;
-    double q = __dmul_rn(v, y);
-    q = __fma_rn(__fma_rn(-pe, q, v), y, q);
-    q = __fma_rn(__fma_rn(-pe, q, v), y, q);
-    if (!(zero || (eu >= -400 && eu <= 400)) || ep < -400 || ep > 400) q = __ddiv_rn(u, pe);
+// u / pe rounded to nearest.  A zero u gives its (signed) zero without a divide:
+// the compiler's divide leaves its fast path on a zero numerator, for the whole
+// warp, and a row can hold many zeros (slack columns, degenerate rows).  (One
+// reciprocal per pivot row and Markstein's rounding steps, 5 FP64 instructions
+// per quotient, were slower: 20,000 uneven LPs 2.90 against 2.74 ms.)
+__device__ __forceinline__ double pivot_divide(double u, double pe) {
+    const bool zero = abskey(u) == 0 && abskey(pe) < 0x7FF0000000000000LL;  // 0 / inf or NaN: the plain divide
+    const double q = __ddiv_rn(zero ? 1.0 : u, pe);
     const int sign = (__double2hiint(u) ^ __double2hiint(pe)) & INT_MIN;
     return zero ? __hiloint2double(sign, 0) : q;
 }
@@ -148,31 +138,39 @@ __device__ __forceinline__ unsigned long long step1_window(long long kmin, long 
     return (unsigned long long)wb << sh;
 }
 
-// Block-wide reductions over per-warp `redux` results.  Each call writes
-// one slot per warp, waits at a barrier, reads every slot, and waits at a
-// second barrier before returning, so no later write can overtake a read of
-// the same slot whatever the calls that follow.
+// Block-wide reductions over per-warp `redux` results through two alternating
+// sets of slots: each call writes its warp's slots of one set, waits at one
+// barrier and reads the set, which is written again only by the call after
+// next, behind the next call's barrier, which every reader of it has passed.
+// (A second barrier per call instead of the second set: 70 x 70 LPs 8.09 against
+// 8.00 ms.)
 struct Reducer {
-    long long* s64;   // kMaxWarps int64 slots
-    unsigned* s32;    // 2 x kMaxWarps uint32 slots (value, count)
+    long long* s64;   // 2 x kMaxWarps int64 slots
+    unsigned* s32;    // 2 x 2 x kMaxWarps uint32 slots (value, count)
     int nw, warp, lane;
+    unsigned set = 0;
+
+    __device__ Reducer(long long* s64_, unsigned* s32_, int nw_, int warp_, int lane_)
+        : s64(s64_), s32(s32_), nw(nw_), warp(warp_), lane(lane_) {}
 
     __device__ long long min_i64(long long v) {
         v = warp_min_i64(v);
-        if (lane == 0) s64[warp] = v;
+        set ^= 1u;
+        long long* s = s64 + set * kMaxWarps;
+        if (lane == 0) s[warp] = v;
         __syncthreads();
-        long long r = s64[0];
-        for (int w = 1; w < nw; ++w) r = min(r, s64[w]);
-        __syncthreads();
+        long long r = s[0];
+        for (int w = 1; w < nw; ++w) r = min(r, s[w]);
         return r;
     }
     __device__ unsigned min_u32(unsigned v) {
         v = __reduce_min_sync(kFull, v);
-        if (lane == 0) s32[warp] = v;
+        set ^= 1u;
+        unsigned* s = s32 + set * 2 * kMaxWarps;
+        if (lane == 0) s[warp] = v;
         __syncthreads();
-        unsigned r = s32[0];
-        for (int w = 1; w < nw; ++w) r = min(r, s32[w]);
-        __syncthreads();
+        unsigned r = s[0];
+        for (int w = 1; w < nw; ++w) r = min(r, s[w]);
         return r;
     }
     __device__ int min_i32(int v) {
@@ -182,11 +180,12 @@ struct Reducer {
     __device__ void count_min(unsigned cnt, unsigned v, unsigned& cnt_out, unsigned& v_out) {
         cnt = __reduce_add_sync(kFull, cnt);
         v = __reduce_min_sync(kFull, v);
-        if (lane == 0) { s32[warp] = v; s32[kMaxWarps + warp] = cnt; }
+        set ^= 1u;
+        unsigned* s = s32 + set * 2 * kMaxWarps;
+        if (lane == 0) { s[warp] = v; s[kMaxWarps + warp] = cnt; }
         __syncthreads();
         unsigned c = 0, r = 0xffffffffu;
-        for (int w = 0; w < nw; ++w) { c += s32[kMaxWarps + w]; r = min(r, s32[w]); }
-        __syncthreads();
+        for (int w = 0; w < nw; ++w) { c += s[kMaxWarps + w]; r = min(r, s[w]); }
         cnt_out = c;
         v_out = r;
     }
@@ -194,15 +193,16 @@ struct Reducer {
     // the total; `flag` must be the same for all lanes' view of bal.
     __device__ int prefix_count(bool flag, int& total) {
         const unsigned bal = __ballot_sync(kFull, flag);
-        if (lane == 0) s32[warp] = (unsigned)__popc(bal);
+        set ^= 1u;
+        unsigned* s = s32 + set * 2 * kMaxWarps;
+        if (lane == 0) s[warp] = (unsigned)__popc(bal);
         __syncthreads();
         int before = 0, tot = 0;
         for (int w = 0; w < nw; ++w) {
-            const int cw = (int)s32[w];
+            const int cw = (int)s[w];
             before += (w < warp) ? cw : 0;
             tot += cw;
         }
-        __syncthreads();
         total = tot;
         return before + __popc(bal & ((1u << lane) - 1u));
     }
@@ -214,7 +214,7 @@ struct Reducer {
 struct BlockGroup : Reducer {
     int tid, nt;
     __device__ BlockGroup(long long* s64_, unsigned* s32_)
-        : Reducer{s64_, s32_, (int)(blockDim.x >> 5), (int)(threadIdx.x >> 5), (int)(threadIdx.x & 31)},
+        : Reducer(s64_, s32_, (int)(blockDim.x >> 5), (int)(threadIdx.x >> 5), (int)(threadIdx.x & 31)),
           tid((int)threadIdx.x), nt((int)blockDim.x) {}
     __device__ void sync() { __syncthreads(); }
 };

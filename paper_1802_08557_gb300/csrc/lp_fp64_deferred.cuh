@@ -181,8 +181,7 @@ __device__ __forceinline__ void deferred_solve(G& g, const DeviceBatch& B, const
     const int tid = g.tid;
     const DeferredRegLayout L0 = deferred_reg_layout(m, n, 0);
     // box: objective entries of the entering column (0, 1), the leaving row's
-    // right-hand side (2) and reciprocal pivot (3); boxi: its basic variable,
-    // restart point and sign
+    // right-hand side (2); boxi: its basic variable, restart point and sign
     double* box = reinterpret_cast<double*>(base + L0.box);
     int* boxi = reinterpret_cast<int*>(base + L0.box + 32);
     unsigned* negbits = reinterpret_cast<unsigned*>(base + L0.negbits);  // negated rows
@@ -306,11 +305,11 @@ __device__ __forceinline__ void deferred_solve(G& g, const DeviceBatch& B, const
         g.sync();
     };
     // Step 3's row: r_t, and the objective row(s) after the pivot.  u: the
-    // unscaled own element; y: 1/pe; de, dw: objective entries of column e.
-    auto scale = [&](double u, int e, double pe, double y, double de, double dw, bool both) {
+    // unscaled own element; de, dw: objective entries of column e.
+    auto scale = [&](double u, int e, double pe, double de, double dw, bool both) {
         if (tid != 0 && cvar >= nm) return;
         const bool at_e = tid == e;
-        const double p = quotient(at_e ? 1.0 : u, pe, y);
+        const double p = pivot_divide(at_e ? 1.0 : u, pe);
         r_at(t)[tid] = p;
         obj = __fma_rn(-de, p, at_e ? 0.0 : obj);
         if (both) aux = __fma_rn(-dw, p, at_e ? 0.0 : aux);
@@ -329,7 +328,6 @@ __device__ __forceinline__ void deferred_solve(G& g, const DeviceBatch& B, const
     auto tell_row = [&](int l) {
         if (tid == l) {
             box[2] = beta;
-            box[3] = __drcp_rn(vcol);
             boxi[0] = rvar;
             boxi[1] = rlast;
             boxi[2] = negated ? 1 : 0;
@@ -392,8 +390,7 @@ __device__ __forceinline__ void deferred_solve(G& g, const DeviceBatch& B, const
                 tell_objective(e);
                 column(e);
                 g.sync();
-                const double pe = c_at(t)[i];
-                scale(u, e, pe, __drcp_rn(pe), box[0], 0.0, false);
+                scale(u, e, c_at(t)[i], box[0], 0.0, false);
                 relabel(i, e, (int)(sel >> 16), left);
                 ++t;
                 ++iters;
@@ -467,7 +464,7 @@ __device__ __forceinline__ void deferred_solve(G& g, const DeviceBatch& B, const
         const int left = boxi[0];
         double u = box[2];
         if (live) u = element(l, boxi[1], boxi[2] != 0);
-        scale(u, e, pe, box[3], box[0], box[1], one);
+        scale(u, e, pe, box[0], box[1], one);
         relabel(l, e, (int)(esel >> 16), left);
         rhs_row = l;
         ++t;
@@ -522,7 +519,6 @@ __device__ __forceinline__ void deferred_solve_large(DeferBlock& g, const Device
     const DeferredLayout L0 = deferred_layout(m, n, 0);
     double* beta = reinterpret_cast<double*>(base + L0.beta);            // right-hand side
     int* code = reinterpret_cast<int*>(base + L0.code);                  // Step 2 ratio codes
-    double* recip = reinterpret_cast<double*>(base + L0.recip);          // 1 / the pivot element
     int* row_var = reinterpret_cast<int*>(base + L0.row_var);            // basic variable of each row
     int* row_last = reinterpret_cast<int*>(base + L0.row_last);          // last pending pivot on the row, or -1
     int* negidx = reinterpret_cast<int*>(base + L0.negidx);              // rank among the negated rows, or -1
@@ -661,8 +657,8 @@ __device__ __forceinline__ void deferred_solve_large(DeferBlock& g, const Device
     };
     // Step 3's row: r_t from the unscaled row values, and the objective row(s)
     // after the pivot (`both`: phase I's two).  de, dw: their entries of column e.
-    auto scale = [&](int j, double u, int e, double pe, double y, double de, double dw, bool both) {
-        const double q = quotient(j == e ? 1.0 : u, pe, y);
+    auto scale = [&](int j, double u, int e, double pe, double de, double dw, bool both) {
+        const double q = pivot_divide(j == e ? 1.0 : u, pe);
         r_at(t)[j] = q;
         obj[j] = __fma_rn(-de, q, j == e ? 0.0 : obj[j]);
         if (both) aux[j] = __fma_rn(-dw, q, j == e ? 0.0 : aux[j]);
@@ -727,9 +723,9 @@ __device__ __forceinline__ void deferred_solve_large(DeferBlock& g, const Device
                 const int left = row_var[i];
                 column(e, [](int, double) {});
                 g.sync();
-                const double pe = c_at(t)[i], y = __drcp_rn(pe);
+                const double pe = c_at(t)[i];
                 for (int j = tid; j < W; j += nt)
-                    if (j == 0 || col_var[j] < nm) scale(j, j == 0 ? beta[i] : rt[j], e, pe, y, de, 0.0, false);
+                    if (j == 0 || col_var[j] < nm) scale(j, j == 0 ? beta[i] : rt[j], e, pe, de, 0.0, false);
                 relabel(i, e, (int)(sel >> 16), left);
                 ++t;
                 ++iters;
@@ -800,7 +796,6 @@ __device__ __forceinline__ void deferred_solve_large(DeferBlock& g, const Device
         if (screened) {
             left = row_var[l];
             sr = row_last[l];
-            if (tid == l % nt) recip[0] = __drcp_rn(c_at(t)[l]);
         }
         const double de = obj[e], dw = (phase == 1) ? aux[e] : 0.0;
         bool more = false;
@@ -833,7 +828,6 @@ __device__ __forceinline__ void deferred_solve_large(DeferBlock& g, const Device
             if ((unsigned)l >= (unsigned)m) { status = kNumerical; break; }
             left = row_var[l];
             sr = row_last[l];
-            if (tid == l % nt) recip[0] = __drcp_rn(ct[l]);
             g.sync();  // both read before their owner rewrites them
         }
         const double pe = c_at(t)[l];
@@ -841,9 +835,8 @@ __device__ __forceinline__ void deferred_solve_large(DeferBlock& g, const Device
         if (iters >= max_iters) { status = kIterLimit; break; }
 
         // ---- Step 3: pivot ---------------------------------------------------
-        const double y = recip[0];
-        row(l, sr, tid, nt, [&](int j, double u) { scale(j, u, e, pe, y, de, dw, phase == 1); });
-        if (tid == 0) scale(0, beta[l], e, pe, y, de, dw, phase == 1);
+        row(l, sr, tid, nt, [&](int j, double u) { scale(j, u, e, pe, de, dw, phase == 1); });
+        if (tid == 0) scale(0, beta[l], e, pe, de, dw, phase == 1);
         relabel(l, e, (int)(esel >> 16), left);
         rhs_row = l;
         ++t;

@@ -102,7 +102,7 @@ __host__ __device__ inline size_t resident_smem_bytes(int m, int n, int k) {
 // then (from `hist`) the pending pivots kept beside them.
 // The k-independent arrays come first.
 struct DeferredLayout {
-    size_t recip, beta, code, row_var, row_last, negidx, neg;  // k-independent
+    size_t beta, code, row_var, row_last, negidx, neg;  // k-independent
     size_t obj, aux, col_var, col_last, hist;
 };
 
@@ -110,7 +110,6 @@ __host__ __device__ inline DeferredLayout deferred_layout(int m, int n, int k) {
     DeferredLayout L;
     const size_t M = (size_t)m, W = (size_t)n + k + 1;
     size_t o = 0;
-    L.recip = o;    o += 16;
     L.beta = o;     o += align16(M * 8);
     L.code = o;     o += align16(M * 4);
     L.row_var = o;  o += align16(M * 4);
@@ -208,6 +207,50 @@ __host__ __device__ inline MixedLayout mixed_layout(int m, int n, int k) {
 
 __host__ __device__ inline size_t mixed_smem_bytes(int m, int n, int k) {
     return SmallLayout::total + mixed_layout(m, n, k).total;
+}
+
+// The mixed path with deferred updates (lp_mixed_deferred.cuh): the k-independent
+// arrays of MixedLayout (up to its T), then the FP32 vectors, then (from
+// `hist`) the first pending pivots.
+// pending pivots before the whole tableau is formed (24: 2000 uneven LPs 2.7 ms,
+// 32 to 64: 1.3)
+constexpr int kMixedFirst = 48;
+struct MixedDeferredLayout {
+    size_t beta, rf, row_last, negidx, obj, aux, col_var, col_last, hist;
+};
+__host__ __device__ inline MixedDeferredLayout mixed_deferred_layout(int m, int n, int k) {
+    MixedDeferredLayout L;
+    const size_t M = (size_t)m, W = (size_t)n + k + 1;
+    size_t o = mixed_layout(m, n, 0).T;
+    L.beta = o;     o += align16(M * 4);
+    L.rf = o;       o += align16((M + 2) * 4);
+    L.row_last = o; o += align16(M * 4);
+    L.negidx = o;   o += align16(M * 4);
+    L.obj = o;      o += align16(W * 4);
+    L.aux = o;      o += align16(W * 4);
+    L.col_var = o;  o += align16(W * 4);
+    L.col_last = o; o += align16(W * 4);
+    L.hist = o;
+    return L;
+}
+// Its workspace slot: the whole tableau of an LP of more than `first` pivots
+// (m + 2 rows), the pending pivots beyond shared memory, and the certificate's
+// columns.
+struct MixedDeferredSlot {
+    int LD, first;
+    size_t T, hist, slack, total;
+};
+__host__ __device__ inline MixedDeferredSlot mixed_deferred_slot(int m, int n, int k) {
+    MixedDeferredSlot S;
+    const size_t M = (size_t)m, W = (size_t)n + k + 1;
+    S.first = kMixedFirst;
+    S.LD = (int)((W + 3) & ~size_t(3));
+    size_t o = 0;
+    S.T = o;     o += (M + 2) * S.LD * 4;
+    S.hist = o;  o += (size_t)S.first * (M + W) * 4;
+    S.slack = o; o += M * (M < W ? M : W) * 4;
+    S.total = (o + 255) & ~size_t(255);
+    return S;
 }
 
 // Tolerances of the FP32 simplex and of the FP64 certificate.
@@ -374,6 +417,25 @@ cudaError_t launch_mixed_streamed(const DeviceBatch& B, const Tolerances& tol, c
                                   size_t slot_bytes, int32_t* counter, const FallbackQueues& fq, int32_t* diag,
                                   cudaStream_t stream);
 int mixed_streamed_ctas_per_sm();
+
+// Mixed precision with deferred updates (lp_mixed_streamed.cu), by size class:
+// persistent CTAs take LPs of order[0..count) from `counter` (zeroed here); CTA
+// i works in slot i of `slot_bytes` bytes (at least mixed_deferred_slot of every
+// listed LP, a multiple of 256).
+struct MixedDeferredForm {
+    int cls, threads;
+    size_t smem;
+};
+constexpr int kMixedDeferredClasses = 3;
+MixedDeferredForm mixed_deferred_form(int m, int n);
+// Whether an LP gets deferred updates by default (nonneg as for defer_updates;
+// uneven: the batch's LPs differ in size).
+bool mixed_defer_updates(int m, int n, int k, bool nonneg, bool uneven);
+int mixed_deferred_ctas_per_sm(const MixedDeferredForm& f);
+cudaError_t launch_mixed_deferred(const DeviceBatch& B, const Tolerances& tol, const MixedParams& mp,
+                                  const int32_t* order, int32_t count, const MixedDeferredForm& f, int slots,
+                                  unsigned char* workspace, size_t slot_bytes, int32_t* counter,
+                                  const FallbackQueues& fq, int32_t* diag, cudaStream_t stream);
 
 // Learned warm start (lp_warm.cu): features [num_lps x (m+n)] = (b, c) as
 // FP32; the restricted-LP solve and FP64 check of each LP from the network's

@@ -31,16 +31,10 @@
 
 #include "lp_device.cuh"
 #include "lp_internal.h"
+#include "lp_mixed_deferred.cuh"
 
 namespace lpb {
 namespace {
-
-__device__ __forceinline__ float fabs32(float v) { return __int_as_float(__float_as_int(v) & INT_MAX); }
-
-// 64-bit key: signed `hi` compared first, then unsigned `lo`.
-__device__ __forceinline__ long long pack_key(int hi, unsigned lo) {
-    return (long long)(((unsigned long long)(unsigned)hi << 32) | (unsigned long long)lo);
-}
 
 // Rows per batch of the pivot update (all loads of a batch issued before its
 // stores).  Measured on 50x50 LPs: deeper batches, two quads per thread and
@@ -48,14 +42,6 @@ __device__ __forceinline__ long long pack_key(int hi, unsigned lo) {
 // for the one-warp kernel were all slower (larger code or spills, same
 // latency-bound issue rate).
 constexpr int kPivotBatch = 4;
-
-struct Tab32 {
-    float* T;
-    float* colE;
-    int* col_var;
-    int* row_var;
-    int LD;
-};
 
 // Thread layout of the pivot update over quads of 4 columns: thread tid takes
 // quads q0, q0 + qstep, ... and rows r0, r0 + rg, ...  It depends only on the
@@ -180,10 +166,10 @@ __device__ __forceinline__ float group_sum(float v, int P) {
     return v;
 }
 
-template <class G, bool kSplit>
+template <class G, bool kSplit, bool kDefer = false>
 __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const Tolerances& tol, const MixedParams& mp,
                                             const int lp, unsigned char* big, const FallbackQueues& fq,
-                                            int32_t* diag);
+                                            int32_t* diag, size_t big_bytes = 0, unsigned char* slot = nullptr);
 
 // mixed_solve with the split chosen from the LP's m (the same in every form).
 template <class G>
@@ -206,10 +192,14 @@ __device__ __forceinline__ double block_absmax(G& g, double v) {
 // LP's shared-memory area (mixed_layout); G is the group of threads that owns
 // the LP.  kSplit: the certificate's long sums are split over
 // split_width(m) > 1 lanes (else P = 1 at compile time, plain loops).
-template <class G, bool kSplit>
+// kDefer: no tableau is kept (lp_mixed_deferred.cuh): `big` is `big_bytes` of
+// shared memory (mixed_deferred_layout), `slot` the LP's workspace
+// (mixed_deferred_slot); the same FP32 operations on every element, so the
+// same results.
+template <class G, bool kSplit, bool kDefer>
 __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const Tolerances& tol, const MixedParams& mp,
                                             const int lp, unsigned char* big, const FallbackQueues& fq,
-                                            int32_t* diag)
+                                            int32_t* diag, size_t big_bytes, unsigned char* slot)
 {
     const int m = B.m[lp];
     const int n = B.n[lp];
@@ -265,9 +255,17 @@ __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const To
     g.sync();  // neg[] and row_var[] are read by other threads below
     const MixedLayout L = mixed_layout(m, n, k);
     Tab32 tb;
-    tb.T = reinterpret_cast<float*>(big + L.T);
-    tb.colE = reinterpret_cast<float*>(big + L.colE);
-    tb.col_var = reinterpret_cast<int*>(big + L.col_var);
+    Deferred32 df{};
+    if constexpr (kDefer) {
+        df.place(big, big_bytes, slot, m, n, k);
+        tb.T = df.T;
+        tb.colE = df.rf;
+        tb.col_var = df.col_var;
+    } else {
+        tb.T = reinterpret_cast<float*>(big + L.T);
+        tb.colE = reinterpret_cast<float*>(big + L.colE);
+        tb.col_var = reinterpret_cast<int*>(big + L.col_var);
+    }
     tb.row_var = row_var;
     tb.LD = L.LD;
     const int LD = L.LD;
@@ -294,24 +292,30 @@ __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const To
         for (int idx = tid; idx < mn; idx += nt) {
             const double a = A[idx];
             out_of_range += outside(a) ? 1u : 0u;
-            const float v = __double2float_rn(a);
-            T[i * LD + 1 + j] = (row_var[i] >= nm) ? -v : v;
-            i += di;
-            j += dj;
-            if (j >= n) { j -= n; ++i; }
+            if constexpr (!kDefer) {
+                const float v = __double2float_rn(a);
+                T[i * LD + 1 + j] = (row_var[i] >= nm) ? -v : v;
+                i += di;
+                j += dj;
+                if (j >= n) { j -= n; ++i; }
+            }
         }
     }
     // column 0 (b) and the slack columns of the negated rows
-    for (int i = warp; i < m; i += g.nw) {
-        const bool isneg = row_var[i] >= nm;
-        float* Ti = T + i * LD;
-        for (int t = lane; t <= k; t += 32) {
-            const int j = (t == 0) ? 0 : n + t;
-            const float v = (t == 0) ? __double2float_rn(bv[i]) : ((neg[t - 1] == i) ? 1.0f : 0.0f);
-            Ti[j] = isneg ? -v : v;
+    if constexpr (kDefer) {
+        df.build(g, row_var, neg, A, bv, cv, k);
+    } else {
+        for (int i = warp; i < m; i += g.nw) {
+            const bool isneg = row_var[i] >= nm;
+            float* Ti = T + i * LD;
+            for (int t = lane; t <= k; t += 32) {
+                const int j = (t == 0) ? 0 : n + t;
+                const float v = (t == 0) ? __double2float_rn(bv[i]) : ((neg[t - 1] == i) ? 1.0f : 0.0f);
+                Ti[j] = isneg ? -v : v;
+            }
         }
     }
-    {
+    if constexpr (!kDefer) {
         float* Tm = T + m * LD;
         for (int j = tid; j <= Cvar; j += nt) Tm[j] = (j >= 1 && j <= n) ? -__double2float_rn(cv[j - 1]) : 0.0f;
     }
@@ -330,7 +334,7 @@ __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const To
         unsigned dummy;
         g.count_min(out_of_range, 0u, out_of_range, dummy);
     }
-    if (k > 0) {
+    if (!kDefer && k > 0) {
         float* Tw = T + (m + 1) * LD;
         for (int j = tid; j <= Cvar; j += nt) {
             float w = 0.0f;
@@ -347,8 +351,11 @@ __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const To
     int status = -1;
     int phase = (k > 0) ? 1 : 2;
     int e_unb = -1;
-    QuadMap qm = quad_map(tid, nt, Cvar + 1);
     if (out_of_range) status = kNumerical;  // straight to the FP64 kernel
+    if constexpr (kDefer) df.simplex(g, tb, tol, mp, diag, lp, bmax, max_iters, status, phase, iters, e_unb);
+    // with kDefer, what is left to the loop below is an LP that was handed over
+    const bool whole = !kDefer || df.handed;
+    QuadMap qm = quad_map(tid, nt, Cvar + 1);
 
     while (status < 0) {
         const int orow = (phase == 1) ? m + 1 : m;
@@ -506,7 +513,8 @@ __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const To
             ok = false;
         }
         nnb = build_nbl();
-        for (int i = tid; i < m; i += nt) xb[i] = (double)T[i * LD];
+        if (!whole) df.slack_columns(g, nbl, nnb);
+        for (int i = tid; i < m; i += nt) xb[i] = (double)(whole ? T[i * LD] : df.beta[i]);
         g.sync();
     }
     const double tol_p = mp.cert_tol * bmax;
@@ -560,11 +568,11 @@ __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const To
             unsigned fwdbad = 0;
             for (int i = tid; i < m; i += nt) {
                 float acc = 0.0f;
-                const float* Ti = T + i * LD;
+                const float* Ti = whole ? T + i * LD : df.slack + i;
 #pragma unroll 4
                 for (int u = 0; u < nnb; ++u) {
                     const int pc = nbl[u];
-                    acc = __fmaf_rn(Ti[(unsigned)pc >> 16], rf[pc & 0xffff], acc);
+                    acc = __fmaf_rn(whole ? Ti[(unsigned)pc >> 16] : Ti[u * m], rf[pc & 0xffff], acc);
                 }
                 const int v = row_var[i];
                 // the correction: B^-1 r (FP32), plus r_c exactly for a basic slack
@@ -594,7 +602,7 @@ __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const To
         // dual: y_c = reduced cost of slack c; refine  y^T B = c_B^T
         for (int c = tid; c < m; c += nt) {
             const int p = spos[c];
-            yv[c] = (p > 0) ? (double)T[m * LD + p] : 0.0;
+            yv[c] = (p > 0) ? (double)(whole ? T[m * LD + p] : df.obj[p]) : 0.0;
         }
         g.sync();
         bool conv = false;
@@ -649,9 +657,10 @@ __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const To
                 const int pc = act ? nbl[u] : 0;
                 float acc = 0.0f;
                 if (act) {
-                    const float* Tp = T + ((unsigned)pc >> 16);
+                    const float* Tp = whole ? T + ((unsigned)pc >> 16) : df.slack + (size_t)u * m;
+                    const int step = whole ? LD : 1;
 #pragma unroll 4
-                    for (int i = sq; i < m; i += P) acc = __fmaf_rn(rf[i], Tp[i * LD], acc);
+                    for (int i = sq; i < m; i += P) acc = __fmaf_rn(rf[i], Tp[i * step], acc);
                 }
                 acc = group_sum(acc, P);
                 if (act && sq == 0) zf[pc & 0xffff] = acc;
@@ -716,7 +725,7 @@ __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const To
     if (ok && status == kUnbounded) {
         // ray: entering variable up by 1, basic variables by d = -B^-1 a_e
         const int ve = tb.col_var[e_unb];
-        for (int i = tid; i < m; i += nt) dv[i] = -(double)T[i * LD + e_unb];
+        for (int i = tid; i < m; i += nt) dv[i] = -(double)(whole ? T[i * LD + e_unb] : df.ray(i));
         g.sync();
         bool conv;
         refine(dv, ve, conv);
@@ -776,7 +785,8 @@ __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const To
         g.count_min(badpos, 0u, badpos, dummy);
         if (badpos == 0) {
             nnb = build_nbl();
-            const float* Tw = T + (m + 1) * LD;
+            if (!whole) df.slack_columns(g, nbl, nnb);
+            const float* Tw = whole ? T + (m + 1) * LD : df.aux;
             for (int c = tid; c < m; c += nt) {
                 const int p = spos[c];
                 yv[c] = (p > 0) ? (double)Tw[p] : 0.0;
@@ -817,9 +827,10 @@ __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const To
                     const int pc = act ? nbl[u] : 0;
                     float acc = 0.0f;
                     if (act) {
-                        const float* Tp = T + ((unsigned)pc >> 16);
+                        const float* Tp = whole ? T + ((unsigned)pc >> 16) : df.slack + (size_t)u * m;
+                    const int step = whole ? LD : 1;
 #pragma unroll 4
-                        for (int i = sq; i < m; i += P) acc = __fmaf_rn(rf[i], Tp[i * LD], acc);
+                        for (int i = sq; i < m; i += P) acc = __fmaf_rn(rf[i], Tp[i * step], acc);
                     }
                     acc = group_sum(acc, P);
                     if (act && sq == 0) zf[pc & 0xffff] = acc;
@@ -914,7 +925,7 @@ __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const To
                 y[c] = yv[c];
             } else {
                 const int p = spos[c];
-                y[c] = (p > 0) ? (double)T[m * LD + p] : 0.0;
+                y[c] = (p > 0) ? (double)(whole ? T[m * LD + p] : df.obj[p]) : 0.0;
             }
         }
     }

@@ -40,6 +40,36 @@ mixed_streamed_kernel(const DeviceBatch B, const Tolerances tol, const MixedPara
     }
 }
 
+// LPs with deferred updates (lp_mixed_deferred.cuh): the vectors and the first
+// pending pivots in shared memory, the rest in the CTA's slot.
+__global__ void __launch_bounds__(256, 3)
+mixed_deferred_kernel(const DeviceBatch B, const Tolerances tol, const MixedParams mp,
+                      const int32_t* __restrict__ order, const int32_t count, unsigned char* workspace,
+                      const size_t slot_bytes, int32_t* __restrict__ counter, const FallbackQueues fq,
+                      int32_t* __restrict__ diag, const size_t smem_bytes)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ int next;
+    unsigned char* slot = workspace + (size_t)blockIdx.x * slot_bytes;
+    unsigned char* area = smem + SmallLayout::total;
+    const size_t bytes = smem_bytes - SmallLayout::total;
+    for (;;) {
+        if (threadIdx.x == 0) next = atomicAdd(counter, 1);
+        __syncthreads();
+        const int idx = next;
+        __syncthreads();
+        if (idx >= count) break;
+        const int lp = order[idx];
+        BlockGroup g(reinterpret_cast<long long*>(smem + SmallLayout::red64),
+                     reinterpret_cast<unsigned*>(smem + SmallLayout::red32));
+        if (split_width(B.m[lp]) > 1)
+            mixed_solve<BlockGroup, true, true>(g, B, tol, mp, lp, area, fq, diag, bytes, slot);
+        else
+            mixed_solve<BlockGroup, false, true>(g, B, tol, mp, lp, area, fq, diag, bytes, slot);
+        __syncthreads();
+    }
+}
+
 // A whole mixed-precision batch in one launch (LPB_SCHED_SINGLE): persistent
 // CTAs take the LPs order[0 .. count) (longest work first within each part)
 // from the atomic `counter`.  Block mode, order[0 .. warp_from): the CTA
@@ -122,6 +152,50 @@ cudaError_t launch_mixed_single(const DeviceBatch& B, const Tolerances& tol, con
     if (err != cudaSuccess) return err;
     mixed_single_kernel<<<ctas, kMixedSingleThreads, smem, stream>>>(B, tol, mp, order, resident, count, warp_from,
                                                                       workspace, slot_bytes, counter, fq, diag);
+    return cudaGetLastError();
+}
+
+// Size classes: threads for about two rows and columns each, shared memory for
+// the vectors and the first ten pivots or so.
+MixedDeferredForm mixed_deferred_form(int m, int n) {
+    const int d = m > n ? m : n;
+    if (d <= 128) return {0, 128, 28 << 10};
+    if (d <= 256) return {1, 256, 56 << 10};
+    return {2, 256, 76 << 10};
+}
+
+// In a batch of uneven sizes, packing LPs of more than 12,000 entries: one queue
+// per class instead of a launch per footprint step, no FP32 copy of A, few
+// pivots (20,000 LPs of 10-500 rows and columns 10.4 -> 4.9 ms, 2000 of them 2.1 ->
+// 1.3; from 2000 entries on 5.5, from 30,000 5.2).  In a batch of one size the
+// whole-tableau forms keep them: an FP32 update is cheap, and positive LPs of
+// 200 x 200 (28 pivots) take 0.90 against 1.22 ms, 300 x 300 2.4 against 3.0.
+bool mixed_defer_updates(int m, int n, int k, bool nonneg, bool uneven) {
+    return uneven && nonneg && (int64_t)(m + 1) * (n + k + 1) > 12000 && m >= 32 && n >= 32 &&
+           SmallLayout::total + mixed_deferred_layout(m, n, k).hist <= mixed_deferred_form(m, n).smem;
+}
+
+int mixed_deferred_ctas_per_sm(const MixedDeferredForm& f) {
+    int blocks = 0;
+    if (cudaFuncSetAttribute(mixed_deferred_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(kMaxSmemPerBlock - 1024)) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, mixed_deferred_kernel, f.threads, f.smem) != cudaSuccess)
+        return 1;
+    return blocks > 0 ? blocks : 1;
+}
+
+cudaError_t launch_mixed_deferred(const DeviceBatch& B, const Tolerances& tol, const MixedParams& mp,
+                                  const int32_t* order, int32_t count, const MixedDeferredForm& f, int slots,
+                                  unsigned char* workspace, size_t slot_bytes, int32_t* counter,
+                                  const FallbackQueues& fq, int32_t* diag, cudaStream_t stream) {
+    if (count <= 0) return cudaSuccess;
+    cudaError_t err = cudaMemsetAsync(counter, 0, sizeof(int32_t), stream);
+    if (err != cudaSuccess) return err;
+    if ((err = cudaFuncSetAttribute(mixed_deferred_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)(kMaxSmemPerBlock - 1024))) != cudaSuccess)
+        return err;
+    mixed_deferred_kernel<<<slots, f.threads, f.smem, stream>>>(B, tol, mp, order, count, workspace, slot_bytes,
+                                                                counter, fq, diag, f.smem);
     return cudaGetLastError();
 }
 

@@ -401,7 +401,7 @@ __device__ __forceinline__ void warm_one(const WarmArgs& a, const int lp) {
 
 // One CTA per LP of the batch, or (a.queue) persistent CTAs over the LPs of a
 // device-side queue, whose length only the device knows.
-__global__ void __launch_bounds__(kWarmThreads) warm_kernel(const WarmArgs a) {
+__global__ void __launch_bounds__(kWarmThreads, 10) warm_kernel(const WarmArgs a) {
     const int count = a.queue ? min(*a.queue_len, a.fb_cap) : min(a.num_lps, (int)blockIdx.x + 1);
     for (int qi = blockIdx.x; qi < count; qi += gridDim.x) {
         const int lp = a.queue ? a.queue[qi] : qi;
