@@ -138,39 +138,33 @@ __device__ __forceinline__ unsigned long long step1_window(long long kmin, long 
     return (unsigned long long)wb << sh;
 }
 
-// Block-wide reductions over per-warp `redux` results through two alternating
-// sets of slots: each call writes its warp's slots of one set, waits at one
-// barrier and reads the set, which is written again only by the call after
-// next, behind the next call's barrier, which every reader of it has passed.
-// (A second barrier per call instead of the second set: 70 x 70 LPs 8.09 against
-// 8.00 ms.)
+// Block-wide reductions over per-warp `redux` results.  Each call writes
+// one slot per warp, waits at a barrier, reads every slot, and waits at a
+// second barrier before returning, so no later write can overtake a read of
+// the same slot whatever the calls that follow.  (Two alternating sets of slots
+// and one barrier: the fewer barriers gave 1% at most, and the set's addressing
+// cost the warm kernel, whose issue slots are 76% busy, 5%.)
 struct Reducer {
-    long long* s64;   // 2 x kMaxWarps int64 slots
-    unsigned* s32;    // 2 x 2 x kMaxWarps uint32 slots (value, count)
+    long long* s64;   // kMaxWarps int64 slots
+    unsigned* s32;    // 2 x kMaxWarps uint32 slots (value, count)
     int nw, warp, lane;
-    unsigned set = 0;
-
-    __device__ Reducer(long long* s64_, unsigned* s32_, int nw_, int warp_, int lane_)
-        : s64(s64_), s32(s32_), nw(nw_), warp(warp_), lane(lane_) {}
 
     __device__ long long min_i64(long long v) {
         v = warp_min_i64(v);
-        set ^= 1u;
-        long long* s = s64 + set * kMaxWarps;
-        if (lane == 0) s[warp] = v;
+        if (lane == 0) s64[warp] = v;
         __syncthreads();
-        long long r = s[0];
-        for (int w = 1; w < nw; ++w) r = min(r, s[w]);
+        long long r = s64[0];
+        for (int w = 1; w < nw; ++w) r = min(r, s64[w]);
+        __syncthreads();
         return r;
     }
     __device__ unsigned min_u32(unsigned v) {
         v = __reduce_min_sync(kFull, v);
-        set ^= 1u;
-        unsigned* s = s32 + set * 2 * kMaxWarps;
-        if (lane == 0) s[warp] = v;
+        if (lane == 0) s32[warp] = v;
         __syncthreads();
-        unsigned r = s[0];
-        for (int w = 1; w < nw; ++w) r = min(r, s[w]);
+        unsigned r = s32[0];
+        for (int w = 1; w < nw; ++w) r = min(r, s32[w]);
+        __syncthreads();
         return r;
     }
     __device__ int min_i32(int v) {
@@ -180,12 +174,11 @@ struct Reducer {
     __device__ void count_min(unsigned cnt, unsigned v, unsigned& cnt_out, unsigned& v_out) {
         cnt = __reduce_add_sync(kFull, cnt);
         v = __reduce_min_sync(kFull, v);
-        set ^= 1u;
-        unsigned* s = s32 + set * 2 * kMaxWarps;
-        if (lane == 0) { s[warp] = v; s[kMaxWarps + warp] = cnt; }
+        if (lane == 0) { s32[warp] = v; s32[kMaxWarps + warp] = cnt; }
         __syncthreads();
         unsigned c = 0, r = 0xffffffffu;
-        for (int w = 0; w < nw; ++w) { c += s[kMaxWarps + w]; r = min(r, s[w]); }
+        for (int w = 0; w < nw; ++w) { c += s32[kMaxWarps + w]; r = min(r, s32[w]); }
+        __syncthreads();
         cnt_out = c;
         v_out = r;
     }
@@ -193,16 +186,15 @@ struct Reducer {
     // the total; `flag` must be the same for all lanes' view of bal.
     __device__ int prefix_count(bool flag, int& total) {
         const unsigned bal = __ballot_sync(kFull, flag);
-        set ^= 1u;
-        unsigned* s = s32 + set * 2 * kMaxWarps;
-        if (lane == 0) s[warp] = (unsigned)__popc(bal);
+        if (lane == 0) s32[warp] = (unsigned)__popc(bal);
         __syncthreads();
         int before = 0, tot = 0;
         for (int w = 0; w < nw; ++w) {
-            const int cw = (int)s[w];
+            const int cw = (int)s32[w];
             before += (w < warp) ? cw : 0;
             tot += cw;
         }
+        __syncthreads();
         total = tot;
         return before + __popc(bal & ((1u << lane) - 1u));
     }
@@ -214,7 +206,7 @@ struct Reducer {
 struct BlockGroup : Reducer {
     int tid, nt;
     __device__ BlockGroup(long long* s64_, unsigned* s32_)
-        : Reducer(s64_, s32_, (int)(blockDim.x >> 5), (int)(threadIdx.x >> 5), (int)(threadIdx.x & 31)),
+        : Reducer{s64_, s32_, (int)(blockDim.x >> 5), (int)(threadIdx.x >> 5), (int)(threadIdx.x & 31)},
           tid((int)threadIdx.x), nt((int)blockDim.x) {}
     __device__ void sync() { __syncthreads(); }
 };
