@@ -316,15 +316,15 @@ lpb_err lp_batch_stage_times(lp_batch *h, float *stage_ms, int32_t *num_solves);
  *                 the same way.
  *  opts           NULL = defaults (opts->schedule and block_threads are ignored;
  *                 opts->precision must be LP_PREC_FP64, else LPB_EINVAL: only
- *                 the FP64 streamed kernel runs here).
+ *                 the FP64 kernels run here).
  *  stream         cudaStream_t (NULL = legacy default); the call is
  *                 asynchronous and returns once the work is enqueued.
  *
- * Scratch: a fixed 64 MiB array inside the library, present on every GPU that
- * loads the library until the process exits.  It holds ~52 bytes per LP plus
- * at least one tableau workspace of about 8*(m+2)*(n+m+4) bytes; a batch that
- * does not fit returns LPB_ETOOBIG before any GPU work (e.g. up to ~1.2
- * million 50 x 50 LPs per call).  Every call looks up the array's device
+ * Scratch: a fixed 96 MiB array inside the library, present on every GPU that
+ * loads the library until the process exits.  A batch whose ~52 bytes per LP
+ * plus one tableau of about 8*(m+2)*(n+m+4) bytes exceed 64 MiB returns
+ * LPB_ETOOBIG before any GPU work (e.g. up to ~1.2 million 50 x 50 LPs per
+ * call); the rest of the array holds what the kernels keep beside a tableau.  Every call looks up the array's device
  * address in the current context (a lookup, no allocation), so a call after
  * cudaDeviceReset or under another context uses that context's copy; the
  * first call on a device may load the library's device code, so make it

@@ -28,12 +28,25 @@
 namespace lpb {
 namespace {
 
-constexpr size_t kNoAllocScratchBytes = size_t(64) << 20;  // 64 MiB
+// A call fits when its descriptors and one whole phase-I tableau fit 64 MiB.
+// The workspace slot of deferred updates, which holds pending pivots beside the
+// tableau, is up to 17 MiB larger than that tableau (m = 494, n = 16384), so the
+// array is: every call within the limit has room for at least one slot.
+constexpr size_t kNoAllocLimitBytes = size_t(64) << 20;
+constexpr size_t kNoAllocScratchBytes = size_t(96) << 20;
 
-// Scratch: [0, 256) work counter | per-LP descriptors | tableau slots.
+// Scratch: [0, 256) work counter | per-LP descriptors | workspace slots.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
 
 constexpr size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
+
+// A whole tableau of m rows by n columns and m artificials, rows padded to 32
+// bytes, with its labels and keys: what the limit counts.
+size_t tableau_bytes(int32_t m, int32_t n) {
+    const size_t M = (size_t)m, LD = ((size_t)n + M + 1 + 3) & ~size_t(3);
+    return align256(align16(M * 8) + 2 * align16(M * 4) + align16((M + 2) * LD * 8) + align16((M + 2) * 8) +
+                    align16(LD * 4));
+}
 
 // Per-LP descriptors (52 bytes per LP): m, n, order (int32) and a_off, b_off,
 // c_off, x_off, y_off (int64).
@@ -119,7 +132,8 @@ extern "C" lpb_err lp_solve_uniform_noalloc(int32_t num_lps, int32_t m, int32_t 
     const size_t slot_bytes = deferred_slot(m, n, m).total;
     const DeferredForm form = deferred_form(m, n, m, false);
     const size_t desc_bytes = descriptor_bytes(num_lps);
-    if (256 + desc_bytes + slot_bytes > kNoAllocScratchBytes) return LPB_ETOOBIG;
+    if (256 + desc_bytes + tableau_bytes(m, n) > kNoAllocLimitBytes) return LPB_ETOOBIG;
+    if (deferred && 256 + desc_bytes + slot_bytes > kNoAllocScratchBytes) return LPB_ETOOBIG;
 
     int dev = 0;
     cudaError_t err = cudaGetDevice(&dev);
