@@ -1358,6 +1358,33 @@ lpb_err lp_batch_active_labels(lp_batch* h, float* labels, void* stream) {
     return err ? cuda_fail(err, "labels") : LPB_OK;
 }
 
+// Whether a kernel on `device` may write bytes dst[0 .. bytes): 4-byte aligned
+// memory of that device, inside one allocation.
+static bool kernel_can_write(const void* dst, size_t bytes, int device) {
+    static const auto query = [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            p = nullptr;
+        }
+        return reinterpret_cast<CUresult (*)(unsigned, CUpointer_attribute*, void**, CUdeviceptr)>(p);
+    }();
+    if (!query || (reinterpret_cast<uintptr_t>(dst) & 3u)) return false;
+    unsigned type = 0, managed = 1;
+    int owner = -1;
+    CUdeviceptr start = 0;
+    size_t size = 0;
+    CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                  CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                  CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void* to[] = {&type, &managed, &owner, &start, &size};
+    const CUdeviceptr at = (CUdeviceptr) reinterpret_cast<uintptr_t>(dst);
+    return query(5, what, to, at) == CUDA_SUCCESS && type == CU_MEMORYTYPE_DEVICE && !managed && owner == device &&
+           at >= start && bytes <= size && at - start <= size - bytes;
+}
+
 lpb_err lp_batch_results(lp_batch* h, int32_t* status, int32_t* iters, double* obj, double* x, double* y,
                          int32_t ptr_kind) {
     g_last_error.clear();
@@ -1380,17 +1407,13 @@ lpb_err lp_batch_results(lp_batch* h, int32_t* status, int32_t* iters, double* o
                 {y, h->d.y, (size_t)h->total_y * 8, "copy y"}};
     cudaError_t err = cudaSuccess;
     // device outputs in one launch where a kernel can write them (memory of this
-    // device, 4-byte aligned); else one copy each
+    // device, 4-byte aligned, the whole output within its allocation); else one
+    // copy each, which checks its destination itself
     lpb::CopyList list{};
     bool together = ptr_kind == LPB_DEVICE;
     for (const auto& o : out) {
         if (!o.dst) continue;
-        if (together) {
-            cudaPointerAttributes at{};
-            if (cudaPointerGetAttributes(&at, o.dst) != cudaSuccess) cudaGetLastError();
-            together = at.type == cudaMemoryTypeDevice && at.device == h->device &&
-                       (reinterpret_cast<uintptr_t>(o.dst) & 3u) == 0;
-        }
+        if (together) together = kernel_can_write(o.dst, o.bytes, h->device);
         list.dst[list.count] = o.dst;
         list.src[list.count] = o.src;
         list.bytes[list.count] = o.bytes;
