@@ -10,7 +10,12 @@
 //    completion counted on an mbarrier), `stages` tiles in flight per CTA.
 //    Thread t then owns LP t of the tile: obj = fma over i = 0..dim-1 in index
 //    order, h_i chosen by a 32-bit integer sign test (no FP64 compare), the shared
-//    box read from shared memory (a broadcast).  x, when asked for, is written
+//    box read from shared memory (a broadcast).  A thread reads 4 coordinates per
+//    step in 16-byte loads where dim allows it (2, or 1): with 8-byte loads the
+//    rows of a warp, 8 dim bytes apart, met in the same banks for an even dim
+//    (16-way for 16, 32, 48, 64).  2^22 LPs, one box, us, 8-byte loads and tiles of
+//    128 before: dim 16 277 -> 123, dim 28 241 -> 209, dim 32 531 -> 247; 2^21 of
+//    dim 64 689 -> 315.  x, when asked for, is written
 //    by a flat pass over the tile (coalesced stores).  Tiles that are not
 //    whole (the last one) or arrays that are not 16-byte aligned are loaded
 //    with plain loads instead.
@@ -116,7 +121,12 @@ __device__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
     return true;
 }
 
-template <bool kBoxPerLp>
+// The bit of the lane that tells apart the lanes of a quarter warp whose rows
+// (8 dim bytes apart, dim a multiple of 4) start in the same bank.
+__device__ __forceinline__ int swap_shift(int dim) { return dim % 16 == 0 ? 0 : (dim % 8 == 0 ? 1 : 2); }
+
+// kWidth: coordinates per step, a divisor of dim (1, 2 or 4).
+template <bool kBoxPerLp, int kWidth>
 __global__ void __launch_bounds__(128) hyperbox_tile_kernel(const HbArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem);        // one per stage
@@ -203,10 +213,47 @@ __global__ void __launch_bounds__(128) hyperbox_tile_kernel(const HbArgs a) {
             const double* lo = kBoxPerLp ? Ls + tile_elems + (size_t)tid * dim : box;
             const double* hi = kBoxPerLp ? Ls + 2 * tile_elems + (size_t)tid * dim : box + dim;
             double acc = 0.0;
+            auto step = [&](double li, double lv, double hv) { acc = __fma_rn(li, is_negative(li) ? lv : hv, acc); };
+            if (kWidth == 4) {
+                // lanes that would meet in a bank read the two halves of their four
+                // coordinates in opposite order
+                const int first = ((tid >> swap_shift(dim)) & 1) * 2, second = 2 - first;
+                for (int i = 0; i < dim; i += 4) {
+                    const double2 p = *reinterpret_cast<const double2*>(l + i + first);
+                    const double2 q = *reinterpret_cast<const double2*>(l + i + second);
+                    double2 lo0, lo1, hi0, hi1;
+                    if (kBoxPerLp) {
+                        const double2 a0 = *reinterpret_cast<const double2*>(lo + i + first);
+                        const double2 a1 = *reinterpret_cast<const double2*>(lo + i + second);
+                        const double2 b0 = *reinterpret_cast<const double2*>(hi + i + first);
+                        const double2 b1 = *reinterpret_cast<const double2*>(hi + i + second);
+                        lo0 = first ? a1 : a0, lo1 = first ? a0 : a1;
+                        hi0 = first ? b1 : b0, hi1 = first ? b0 : b1;
+                    } else {
+                        lo0 = *reinterpret_cast<const double2*>(lo + i), lo1 = *reinterpret_cast<const double2*>(lo + i + 2);
+                        hi0 = *reinterpret_cast<const double2*>(hi + i), hi1 = *reinterpret_cast<const double2*>(hi + i + 2);
+                    }
+                    const double2 l0 = first ? q : p, l1 = first ? p : q;
+                    step(l0.x, lo0.x, hi0.x);
+                    step(l0.y, lo0.y, hi0.y);
+                    step(l1.x, lo1.x, hi1.x);
+                    step(l1.y, lo1.y, hi1.y);
+                }
+            } else if (kWidth == 2) {
+#pragma unroll 2
+                for (int i = 0; i < dim; i += 2) {
+                    const double2 l2 = *reinterpret_cast<const double2*>(l + i);
+                    const double2 lo2 = *reinterpret_cast<const double2*>(lo + i);
+                    const double2 hi2 = *reinterpret_cast<const double2*>(hi + i);
+                    step(l2.x, lo2.x, hi2.x);
+                    step(l2.y, lo2.y, hi2.y);
+                }
+            } else {
 #pragma unroll 4
-            for (int i = 0; i < dim; ++i) {
-                const double li = l[i];
-                acc = __fma_rn(li, is_negative(li) ? lo[i] : hi[i], acc);
+                for (int i = 0; i < dim; ++i) {
+                    const double li = l[i];
+                    acc = __fma_rn(li, is_negative(li) ? lo[i] : hi[i], acc);
+                }
             }
             a.obj[lp0 + tid] = acc;
         }
@@ -296,16 +343,27 @@ cudaError_t launch_hyperbox(const double* L, const double* lo, const double* hi,
         return cudaGetLastError();
     }
     const int arrays = box_per_lp ? 3 : 1;
-    a.tile_lps = (dim * arrays <= 96) ? 128 : 64;
+    // Rows of more than 12 doubles (8 with a box each): one warp per CTA and two
+    // stages, as many CTAs as fit, so that the FP64 pipe and the copies of an SM
+    // never wait for one CTA's barrier.  2^22 LPs of dim 28, one box: 209 us against
+    // 211, 217 and 235 with tiles of 64, 96 and 128, 219 with three stages; 2^20 with
+    // a box and x each 164, 193 (64 and 128), 252 (three stages).  Short rows: tiles
+    // of 128, where a tile's fixed cost counts (dim 2: 27 us against 31 with tiles of
+    // 32; dim 5 with boxes and x, 2 M LPs: 54 against 56), and up to 40 KB in flight
+    // per CTA (dim 12: 95 us with three stages, 99 with four, 100 with two).
+    const bool short_rows = dim <= (box_per_lp ? 8 : 12);
+    a.tile_lps = short_rows ? 128 : 32;
     a.stage_bytes = (int)((size_t)a.tile_lps * dim * 8 * arrays);
-    a.stages = std::max(2, std::min(4, (48 << 10) / a.stage_bytes));
+    a.stages = short_rows ? std::max(2, std::min(4, (40 << 10) / a.stage_bytes)) : 2;
     a.stage_offset = ((64 + 2 * dim * 8 + 127) / 128) * 128;  // mbarriers, shared box, then the stages
     const size_t smem = (size_t)a.stage_offset + (size_t)a.stages * a.stage_bytes;
     a.num_tiles = (num_lps + a.tile_lps - 1) / a.tile_lps;
     auto aligned = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
     const bool bulk = aligned(L) && (!box_per_lp || (aligned(lo) && aligned(hi)));
     a.num_full_tiles = bulk ? num_lps / a.tile_lps : 0;
-    auto kernel = box_per_lp ? hyperbox_tile_kernel<true> : hyperbox_tile_kernel<false>;
+    auto kernel = dim % 4 == 0   ? (box_per_lp ? hyperbox_tile_kernel<true, 4> : hyperbox_tile_kernel<false, 4>)
+                  : dim % 2 == 0 ? (box_per_lp ? hyperbox_tile_kernel<true, 2> : hyperbox_tile_kernel<false, 2>)
+                                 : (box_per_lp ? hyperbox_tile_kernel<true, 1> : hyperbox_tile_kernel<false, 1>);
     if ((err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return err;
     int per_sm = 0;
     if ((err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, a.tile_lps, smem))) return err;
