@@ -19,7 +19,7 @@
 //    by a flat pass over the tile (coalesced stores).  Tiles that are not
 //    whole (the last one) or arrays that are not 16-byte aligned are loaded
 //    with plain loads instead.
-//  - larger dim: one warp per LP, lanes over i, a fixed xor-tree sum.
+//  - larger dim: a warp's lanes over i, a fixed xor-tree sum, up to 8 LPs per warp.
 // Bound: the FP64 pipe (one FMA per 8 bytes of l) for one shared box and no x;
 // HBM bandwidth when every LP has its own box or x is written.
 //
@@ -287,26 +287,65 @@ __global__ void __launch_bounds__(128) hyperbox_tile_kernel(const HbArgs a) {
             if (pending & (1u << s)) mbar_wait(&bar[s], (phase >> s) & 1u);
 }
 
-template <bool kBoxPerLp>
-__global__ void __launch_bounds__(256) hyperbox_warp_kernel(const HbArgs a) {
+// kLps LPs per warp.  The xor-tree sum of one LP by itself is 5 adds of the whole
+// warp, as much FP64 pipe as 160 coordinates; for 8 LPs together each step halves
+// the LPs that a lane still carries: 4 + 2 + 1 + 1 + 1 adds, the same sums; and 8
+// rows' loads are in flight.  One LP per warp against 8, one box, us: 400,000 of
+// dim 65 231 -> 112, of dim 160 311 -> 161; 4 LPs and a box each, 150,000 of dim
+// 100: 103 -> 71.  80 registers, three CTAs per SM (64 spill).
+template <bool kBoxPerLp, int kLps>
+__global__ void __launch_bounds__(256, 3) hyperbox_warp_kernel(const HbArgs a) {
     const int lane = threadIdx.x & 31;
     const int dim = a.dim;
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t k = w0; k < a.num_lps; k += nw) {
+    for (int64_t k = w0 * kLps; k < a.num_lps; k += nw * kLps) {
+        const int last = (int)(a.num_lps - 1 - k < kLps - 1 ? a.num_lps - 1 - k : kLps - 1);
         const int64_t base = k * dim;
-        const double* l = a.L + base;
-        const double* lo = kBoxPerLp ? a.lo + base : a.lo;
-        const double* hi = kBoxPerLp ? a.hi + base : a.hi;
-        double acc = 0.0;
-        for (int i = lane; i < dim; i += 32) {
-            const double li = l[i];
-            const double h = is_negative(li) ? lo[i] : hi[i];
-            acc = __fma_rn(li, h, acc);
-            if (a.x) a.x[base + i] = h;
+        double acc[kLps];
+#pragma unroll
+        for (int q = 0; q < kLps; ++q) acc[q] = 0.0;
+        const double *L = a.L + base + lane, *lo = a.lo + lane, *hi = a.hi + lane;
+        if (kBoxPerLp) lo += base, hi += base;
+        double* x = a.x ? a.x + base + lane : nullptr;
+#pragma unroll 1
+        for (int i = lane; i < dim; i += 32, L += 32, lo += 32, hi += 32) {
+            double li[kLps], l0[kLps], h0[kLps];
+            int at = 0;
+#pragma unroll
+            for (int q = 0; q < kLps; ++q) {
+                li[q] = L[at];
+                l0[q] = (kBoxPerLp || q == 0) ? lo[at] : l0[0];
+                h0[q] = (kBoxPerLp || q == 0) ? hi[at] : h0[0];
+                if (q < last) at += dim;  // past the last LP: its row again, not stored
+            }
+            at = 0;
+#pragma unroll
+            for (int q = 0; q < kLps; ++q) {
+                l0[q] = is_negative(li[q]) ? l0[q] : h0[q];
+                acc[q] = __fma_rn(li[q], l0[q], acc[q]);
+            }
+            if (x) {
+#pragma unroll
+                for (int q = 0; q < kLps; ++q, at += dim)
+                    if (q <= last) x[at] = l0[q];
+                x += 32;
+            }
         }
-        for (int o = 16; o > 0; o >>= 1) acc = __dadd_rn(acc, __shfl_xor_sync(kFullMask, acc, o));
-        if (lane == 0) a.obj[k] = acc;
+        int o = 16, lp = 0;
+#pragma unroll
+        for (int w = kLps / 2; w > 0; w >>= 1, o >>= 1) {
+            const bool up = (lane & o) != 0;
+#pragma unroll
+            for (int q = 0; q < w; ++q) {
+                const double keep = up ? acc[q + w] : acc[q], give = up ? acc[q] : acc[q + w];
+                acc[q] = __dadd_rn(keep, __shfl_xor_sync(kFullMask, give, o));
+            }
+            if (up) lp += w;
+        }
+#pragma unroll
+        for (; o > 0; o >>= 1) acc[0] = __dadd_rn(acc[0], __shfl_xor_sync(kFullMask, acc[0], o));
+        if ((lane & (32 / kLps - 1)) == 0 && lp <= last) a.obj[k + lp] = acc[0];
     }
 }
 
@@ -336,10 +375,14 @@ cudaError_t launch_hyperbox(const double* L, const double* lo, const double* hi,
     a.num_lps = num_lps;
     a.dim = dim;
     if (dim > kTileMaxDim) {
+        // 8 LPs per warp (4 with a box each: registers) from 16 warps per SM on; below
+        // that one each, for latency (10,000 of dim 100: 10 us either way)
+        const int per_warp = num_lps >= (int64_t)sms * 128 ? (box_per_lp ? 4 : 8) : 1;
         const int threads = 256;
-        const int64_t blocks = std::min<int64_t>((num_lps + 7) / 8, (int64_t)sms * 8);
-        if (box_per_lp) hyperbox_warp_kernel<true><<<(unsigned)blocks, threads, 0, stream>>>(a);
-        else hyperbox_warp_kernel<false><<<(unsigned)blocks, threads, 0, stream>>>(a);
+        const int64_t blocks = std::min<int64_t>((num_lps + 8 * per_warp - 1) / (8 * per_warp), (int64_t)sms * 8);
+        auto kernel = per_warp > 1 ? (box_per_lp ? hyperbox_warp_kernel<true, 4> : hyperbox_warp_kernel<false, 8>)
+                                   : (box_per_lp ? hyperbox_warp_kernel<true, 1> : hyperbox_warp_kernel<false, 1>);
+        kernel<<<(unsigned)blocks, threads, 0, stream>>>(a);
         return cudaGetLastError();
     }
     const int arrays = box_per_lp ? 3 : 1;

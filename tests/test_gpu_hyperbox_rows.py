@@ -1,6 +1,7 @@
 """Hyperbox LPs at the row lengths where the tile kernel changes its form: 1, 2
 or 4 coordinates per step, each bank-swap rule (dim a multiple of 4, 8, 16), the
-line between tiles of 128 and of 32, and numbers of LPs around a tile.  Integer
+line between tiles of 128 and of 32, and numbers of LPs around a tile; and above
+64 coordinates several LPs per warp with a last warp of every fill.  Integer
 data: every sum is exact, so objectives match the oracle bit for bit in any order
 of the FMAs, and a coordinate paired with another's bound shows."""
 import numpy as np
@@ -35,3 +36,9 @@ def _check(num, dim, per_lp):
 def test_row_forms_match_the_oracle(dim, per_lp):
     for num in (1, 31, 33, 128, 397):
         _check(num, dim, per_lp)
+
+
+@pytest.mark.parametrize("per_lp", [False, True])
+@pytest.mark.parametrize("num", range(20000, 20008))
+def test_several_lps_per_warp_match_the_oracle(num, per_lp):
+    _check(num, 65 + num % 8 * 13, per_lp)
