@@ -42,8 +42,14 @@ namespace {
 // instruction cache (the support function's 32 one-warp CTAs per SM stalled 40%
 // of the time on instructions).  Batches of 2 and loops unrolled by 2 instead of
 // 4 and 4: support function 3.23 -> 2.91 ms per 1e5, 20 x 20 LPs 0.73 -> 0.66, 50 x
-// 50 the same.  Unrolled by 1: 50 x 50 13.2 against 12.6 ms.
-constexpr int kPivotBatch = 2;
+// 50 the same.  Unrolled by 1: 50 x 50 13.2 against 12.6 ms.  The kernels whose
+// tableau may lie in a global workspace slot wait for its loads instead and keep 4
+// (lp_mixed_streamed.cu).
+#ifndef LPB_MIXED_UNROLL
+#define LPB_MIXED_UNROLL 2
+#endif
+constexpr int kPivotBatch = LPB_MIXED_UNROLL;
+constexpr int kCertUnroll = LPB_MIXED_UNROLL;
 
 // Thread layout of the pivot update over quads of 4 columns: thread tid takes
 // quads q0, q0 + qstep, ... and rows r0, r0 + rg, ...  It depends only on the
@@ -549,7 +555,7 @@ __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const To
                 else r = (rhs_var < n) ? -A[(size_t)c * n + rhs_var] : ((rhs_var - n == c) ? -1.0 : 0.0);
                 float mag = f64_abs_to_f32_trunc(r);  // b, A or 1: range-checked
                 const double* Ac = A + (size_t)c * n;
-#pragma unroll 2
+#pragma unroll kCertUnroll
                 for (int t = 0; t < s; ++t) {
                     const int i = slist[t];
                     const double a = Ac[row_var[i]];
@@ -571,7 +577,7 @@ __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const To
             for (int i = tid; i < m; i += nt) {
                 float acc = 0.0f;
                 const float* Ti = whole ? T + i * LD : df.slack + i;
-#pragma unroll 2
+#pragma unroll kCertUnroll
                 for (int u = 0; u < nnb; ++u) {
                     const int pc = nbl[u];
                     acc = __fmaf_rn(whole ? Ti[(unsigned)pc >> 16] : Ti[u * m], rf[pc & 0xffff], acc);
@@ -661,7 +667,7 @@ __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const To
                 if (act) {
                     const float* Tp = whole ? T + ((unsigned)pc >> 16) : df.slack + (size_t)u * m;
                     const int step = whole ? LD : 1;
-#pragma unroll 2
+#pragma unroll kCertUnroll
                     for (int i = sq; i < m; i += P) acc = __fmaf_rn(rf[i], Tp[i * step], acc);
                 }
                 acc = group_sum(acc, P);
@@ -696,7 +702,7 @@ __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const To
             float d32 = (act && sq == 0) ? -f64_to_f32_trunc(cv[v]) : 0.0f;
             float mag = fabs32(d32);
             if (act) {
-#pragma unroll 2
+#pragma unroll kCertUnroll
                 for (int c = sq; c < m; c += P) {
                     const float a = f64_to_f32_trunc(A[(size_t)c * n + v]);
                     const float yc = zf[c];
@@ -714,7 +720,7 @@ __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const To
             if (__any_sync(kFull, undecided)) {
                 double d = (undecided && sq == 0) ? -cv[v] : 0.0;
                 if (undecided) {
-#pragma unroll 2
+#pragma unroll kCertUnroll
                     for (int c = sq; c < m; c += P) d = __fma_rn(yv[c], A[(size_t)c * n + v], d);
                 }
                 d = group_sum(d, P);
@@ -803,7 +809,7 @@ __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const To
                     const int v = act ? row_var[slist[t]] : 0;
                     double r = 0.0;
                     if (act) {
-#pragma unroll 2
+#pragma unroll kCertUnroll
                         for (int c = sq; c < m; c += P) r = __fma_rn(-yv[c], A[(size_t)c * n + v], r);
                     }
                     r = group_sum(r, P);
@@ -831,7 +837,7 @@ __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const To
                     if (act) {
                         const float* Tp = whole ? T + ((unsigned)pc >> 16) : df.slack + (size_t)u * m;
                     const int step = whole ? LD : 1;
-#pragma unroll 2
+#pragma unroll kCertUnroll
                         for (int i = sq; i < m; i += P) acc = __fmaf_rn(rf[i], Tp[i * step], acc);
                     }
                     acc = group_sum(acc, P);
@@ -855,7 +861,7 @@ __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const To
             g.count_min(bad, 0u, bad, dummy);
             for (int j = tid; j < n; j += nt) {
                 double gj = 0.0, sc = 0.0;
-#pragma unroll 2
+#pragma unroll kCertUnroll
                 for (int c = 0; c < m; ++c) {
                     const double a = A[(size_t)c * n + j];
                     gj = __fma_rn(yv[c], a, gj);

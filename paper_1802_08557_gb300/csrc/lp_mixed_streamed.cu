@@ -8,11 +8,15 @@
 // tableau lives or on the number of threads, so the results are bit-identical
 // to the shared-memory kernels' (tested).
 //
-// Compiled with -dlcm=cg (global loads cached in L2 only), like the FP64
-// streamed kernel: the tableau is rewritten every pivot and gets no reuse
+// Compiled with -dlcm=cg (global loads cached in L2 only): the tableau is rewritten every pivot and gets no reuse
 // from L1.  Two CTAs per SM (64 registers): the kernel waits on L2 latency,
 // and twice the warps in flight measured 9% faster than one CTA with 128.
 
+// These kernels wait for loads from L2, not for instructions: 4 rows' loads in
+// flight against the 2 of the shared-memory kernels, 20,000 uneven LPs 5.51 -> 5.13
+// ms (12.40 -> 11.49 in one launch), 2000 of them 1.49 -> 1.41, 600 of 300 x 250
+// 1.48 -> 1.33.
+#define LPB_MIXED_UNROLL 4
 #include "lp_mixed_solve.cuh"
 
 namespace lpb {
