@@ -49,7 +49,8 @@ def _sources():
 
 
 def _deps():
-    return _sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(INCLUDE, "*.h")) + [__file__]
+    headers = [p for pat in ("*.h", "*.cuh") for p in glob.glob(os.path.join(CSRC, pat))]
+    return _sources() + headers + glob.glob(os.path.join(INCLUDE, "*.h")) + [__file__]
 
 
 def up_to_date() -> bool:
