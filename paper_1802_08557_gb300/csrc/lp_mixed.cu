@@ -17,7 +17,7 @@ mixed_kernel(const DeviceBatch B, const Tolerances tol, const MixedParams mp, co
     extern __shared__ __align__(16) unsigned char smem[];
     BlockGroup g(reinterpret_cast<long long*>(smem + SmallLayout::red64),
                  reinterpret_cast<unsigned*>(smem + SmallLayout::red32));
-    mixed_solve_lp(g, B, tol, mp, order[blockIdx.x], smem + SmallLayout::total, fq, diag);
+    mixed_solve_lp<4>(g, B, tol, mp, order[blockIdx.x], smem + SmallLayout::total, fq, diag);
 }
 
 // Persistent CTAs over a list: LP order[idx] for idx taken from an atomic
@@ -38,7 +38,7 @@ mixed_queue_kernel(const DeviceBatch B, const Tolerances tol, const MixedParams 
         if (idx >= n_items) break;
         BlockGroup g(reinterpret_cast<long long*>(smem + SmallLayout::red64),
                      reinterpret_cast<unsigned*>(smem + SmallLayout::red32));
-        mixed_solve_lp(g, B, tol, mp, order[idx], smem + SmallLayout::total, fq, diag);
+        mixed_solve_lp<4>(g, B, tol, mp, order[idx], smem + SmallLayout::total, fq, diag);
         __syncthreads();
     }
 }
@@ -51,8 +51,27 @@ mixed_warp_kernel(const DeviceBatch B, const Tolerances tol, const MixedParams m
 {
     extern __shared__ __align__(16) unsigned char smem[];
     WarpGroup g;
-    mixed_solve_lp(g, B, tol, mp, order[blockIdx.x], smem, fq, diag);
+    mixed_solve_lp<4>(g, B, tol, mp, order[blockIdx.x], smem, fq, diag);
 }
+
+// The same with half the unrolling, where 16 or more such CTAs share an SM and
+// stall on instructions (40% of the time for 32 of them).
+__global__ void __launch_bounds__(32, 32)
+mixed_warp_small_kernel(const DeviceBatch B, const Tolerances tol, const MixedParams mp,
+                        const int32_t* __restrict__ order, const FallbackQueues fq, int32_t* __restrict__ diag)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    WarpGroup g;
+    mixed_solve_lp<2>(g, B, tol, mp, order[blockIdx.x], smem, fq, diag);
+}
+
+// The line between the two.  Unrolling of 2 against 4, signed / packing /
+// phase-I LPs, time relative to 4: 20 x 20 (3 KB) 0.91 / 0.94 / 0.91, 40 x 40 (10 KB)
+// 0.92 / 0.95 / 0.96, 30 x 80 (13 KB) 0.97 / 0.95 / 0.99, 50 x 50 (13.5 KB) 1.01 / 0.97,
+// with phase I (14.6 KB) 1.04; 60 x 60 (19 KB) 1.03 / 1.01 / 1.06, 70 x 70 (24 KB) 1.11 /
+// 1.02 / 1.13, 88 x 88 1.14 / 1.04; and in CTAs of 128 and 256 threads 100 x 100 1.06 /
+// 1.04 / 1.06, 170 x 170 1.18 / 1.18 / 1.06.
+constexpr size_t kSmallWarpBytes = 14 * 1024;
 
 }  // namespace
 
@@ -63,6 +82,9 @@ cudaError_t mixed_kernel_prepare() {
     err = cudaFuncSetAttribute(mixed_queue_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)(kMaxSmemPerBlock - 1024));
     if (err != cudaSuccess) return err;
+    err = cudaFuncSetAttribute(mixed_warp_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)(kMaxSmemPerBlock - 1024));
+    if (err != cudaSuccess) return err;
     return cudaFuncSetAttribute(mixed_warp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)(kMaxSmemPerBlock - 1024));
 }
@@ -71,7 +93,9 @@ cudaError_t launch_mixed(const DeviceBatch& B, const Tolerances& tol, const Mixe
                          const int32_t* order, int32_t count, int threads, size_t smem,
                          const FallbackQueues& fq, int32_t* diag, cudaStream_t stream) {
     if (count <= 0) return cudaSuccess;
-    if (threads == 32)
+    if (threads == 32 && smem <= kSmallWarpBytes)
+        mixed_warp_small_kernel<<<count, 32, smem, stream>>>(B, tol, mp, order, fq, diag);
+    else if (threads == 32)
         mixed_warp_kernel<<<count, 32, smem, stream>>>(B, tol, mp, order, fq, diag);
     else
         mixed_kernel<<<count, threads, smem, stream>>>(B, tol, mp, order, fq, diag);

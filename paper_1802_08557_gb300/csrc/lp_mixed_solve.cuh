@@ -36,20 +36,12 @@
 namespace lpb {
 namespace {
 
-// Rows per batch of the pivot update (all loads of a batch issued before its
-// stores), and the unrolling of the certificate's loops: small, because the
-// warps of an SM are in different phases of this code and share its
-// instruction cache (the support function's 32 one-warp CTAs per SM stalled 40%
-// of the time on instructions).  Batches of 2 and loops unrolled by 2 instead of
-// 4 and 4: support function 3.23 -> 2.91 ms per 1e5, 20 x 20 LPs 0.73 -> 0.66, 50 x
-// 50 the same.  Unrolled by 1: 50 x 50 13.2 against 12.6 ms.  The kernels whose
-// tableau may lie in a global workspace slot wait for its loads instead and keep 4
-// (lp_mixed_streamed.cu).
-#ifndef LPB_MIXED_UNROLL
-#define LPB_MIXED_UNROLL 2
-#endif
-constexpr int kPivotBatch = LPB_MIXED_UNROLL;
-constexpr int kCertUnroll = LPB_MIXED_UNROLL;
+// kUnroll (of pivot32 and mixed_solve): the rows per batch of the pivot update
+// (all loads of a batch issued before its stores) and the unrolling of the
+// certificate's loops.  4 hides more latency; 2 is less code, which counts
+// where the warps of an SM are in different phases of it and share its
+// instruction cache (mixed_warp_small_kernel, lp_mixed.cu, with both sides
+// measured).  The same operations in the same order either way.
 
 // Thread layout of the pivot update over quads of 4 columns: thread tid takes
 // quads q0, q0 + qstep, ... and rows r0, r0 + rg, ...  It depends only on the
@@ -81,11 +73,11 @@ __device__ __forceinline__ QuadMap quad_map(int tid, int nt, int Cact) {
 //           gives fma(-t_ie, 1/PE, 0) = -t_ie/PE there (the leaving variable's
 //           column);
 //  phase B: t_rj = fma(-t_re, r_j, t_rj) for r != l over quads of 4 columns
-//           (16-byte loads and stores; LD is a multiple of 4), kPivotBatch
+//           (16-byte loads and stores; LD is a multiple of 4), kUnroll
 //           rows per batch with every load of a batch issued before its
 //           stores.
 //  Columns of the last quad beyond Cact are padding: updated, never read.
-template <class G>
+template <int kUnroll, class G>
 __device__ __forceinline__ int pivot32(G& g, Tab32& tb, int Ract, int Cact, int l, int e, const QuadMap& qm) {
     const int tid = g.tid, nt = g.nt;
     const int LD = tb.LD;
@@ -105,7 +97,7 @@ __device__ __forceinline__ int pivot32(G& g, Tab32& tb, int Ract, int Cact, int 
     const int left = tb.col_var[e];
     const int nq = (Cact + 3) >> 2;
     const int qstep = qm.qstep, r0 = qm.r0, rg = qm.rg;
-    constexpr int kB = kPivotBatch;
+    constexpr int kB = kUnroll;
     for (int q = qm.q0; q < nq; q += qstep) {
         const float4 p = *reinterpret_cast<const float4*>(Tl + 4 * q);
         float* base = T + 4 * q;
@@ -174,20 +166,20 @@ __device__ __forceinline__ float group_sum(float v, int P) {
     return v;
 }
 
-template <class G, bool kSplit, bool kDefer = false>
+template <int kUnroll, class G, bool kSplit, bool kDefer = false>
 __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const Tolerances& tol, const MixedParams& mp,
                                             const int lp, unsigned char* big, const FallbackQueues& fq,
                                             int32_t* diag, size_t big_bytes = 0, unsigned char* slot = nullptr);
 
 // mixed_solve with the split chosen from the LP's m (the same in every form).
-template <class G>
+template <int kUnroll, class G>
 __device__ __forceinline__ void mixed_solve_lp(G& g, const DeviceBatch& B, const Tolerances& tol,
                                                const MixedParams& mp, const int lp, unsigned char* big,
                                                const FallbackQueues& fq, int32_t* diag) {
     if (split_width(B.m[lp]) > 1)
-        mixed_solve<G, true>(g, B, tol, mp, lp, big, fq, diag);
+        mixed_solve<kUnroll, G, true>(g, B, tol, mp, lp, big, fq, diag);
     else
-        mixed_solve<G, false>(g, B, tol, mp, lp, big, fq, diag);
+        mixed_solve<kUnroll, G, false>(g, B, tol, mp, lp, big, fq, diag);
 }
 
 // max |v| over the group (FP64), as a double.
@@ -204,7 +196,7 @@ __device__ __forceinline__ double block_absmax(G& g, double v) {
 // shared memory (mixed_deferred_layout), `slot` the LP's workspace
 // (mixed_deferred_slot); the same FP32 operations on every element, so the
 // same results.
-template <class G, bool kSplit, bool kDefer>
+template <int kUnroll, class G, bool kSplit, bool kDefer>
 __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const Tolerances& tol, const MixedParams& mp,
                                             const int lp, unsigned char* big, const FallbackQueues& fq,
                                             int32_t* diag, size_t big_bytes, unsigned char* slot)
@@ -417,7 +409,7 @@ __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const To
                 if (!isfinite(tb.colE[l])) { status = kNumerical; break; }
                 if (iters >= max_iters) { status = kIterLimit; break; }
                 if (qm.cact != Cvar + 1) qm = quad_map(tid, nt, Cvar + 1);
-                const int left = pivot32(g, tb, Ract, Cvar + 1, l, e, qm);
+                const int left = pivot32<kUnroll>(g, tb, Ract, Cvar + 1, l, e, qm);
                 ++iters;
                 if (left >= nm) retire_column32(g, tb, Ract, e, Cvar);
             }
@@ -444,7 +436,7 @@ __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const To
                 for (int r = tid; r < m + 1; r += nt) tb.colE[r] = T[r * LD + e];
                 g.sync();
                 if (qm.cact != Cvar + 1) qm = quad_map(tid, nt, Cvar + 1);
-                const int left = pivot32(g, tb, m + 1, Cvar + 1, i, e, qm);
+                const int left = pivot32<kUnroll>(g, tb, m + 1, Cvar + 1, i, e, qm);
                 ++iters;
                 if (left >= nm) retire_column32(g, tb, m + 1, e, Cvar);
             }
@@ -555,7 +547,7 @@ __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const To
                 else r = (rhs_var < n) ? -A[(size_t)c * n + rhs_var] : ((rhs_var - n == c) ? -1.0 : 0.0);
                 float mag = f64_abs_to_f32_trunc(r);  // b, A or 1: range-checked
                 const double* Ac = A + (size_t)c * n;
-#pragma unroll kCertUnroll
+#pragma unroll kUnroll
                 for (int t = 0; t < s; ++t) {
                     const int i = slist[t];
                     const double a = Ac[row_var[i]];
@@ -577,7 +569,7 @@ __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const To
             for (int i = tid; i < m; i += nt) {
                 float acc = 0.0f;
                 const float* Ti = whole ? T + i * LD : df.slack + i;
-#pragma unroll kCertUnroll
+#pragma unroll kUnroll
                 for (int u = 0; u < nnb; ++u) {
                     const int pc = nbl[u];
                     acc = __fmaf_rn(whole ? Ti[(unsigned)pc >> 16] : Ti[u * m], rf[pc & 0xffff], acc);
@@ -667,7 +659,7 @@ __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const To
                 if (act) {
                     const float* Tp = whole ? T + ((unsigned)pc >> 16) : df.slack + (size_t)u * m;
                     const int step = whole ? LD : 1;
-#pragma unroll kCertUnroll
+#pragma unroll kUnroll
                     for (int i = sq; i < m; i += P) acc = __fmaf_rn(rf[i], Tp[i * step], acc);
                 }
                 acc = group_sum(acc, P);
@@ -702,7 +694,7 @@ __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const To
             float d32 = (act && sq == 0) ? -f64_to_f32_trunc(cv[v]) : 0.0f;
             float mag = fabs32(d32);
             if (act) {
-#pragma unroll kCertUnroll
+#pragma unroll kUnroll
                 for (int c = sq; c < m; c += P) {
                     const float a = f64_to_f32_trunc(A[(size_t)c * n + v]);
                     const float yc = zf[c];
@@ -720,7 +712,7 @@ __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const To
             if (__any_sync(kFull, undecided)) {
                 double d = (undecided && sq == 0) ? -cv[v] : 0.0;
                 if (undecided) {
-#pragma unroll kCertUnroll
+#pragma unroll kUnroll
                     for (int c = sq; c < m; c += P) d = __fma_rn(yv[c], A[(size_t)c * n + v], d);
                 }
                 d = group_sum(d, P);
@@ -809,7 +801,7 @@ __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const To
                     const int v = act ? row_var[slist[t]] : 0;
                     double r = 0.0;
                     if (act) {
-#pragma unroll kCertUnroll
+#pragma unroll kUnroll
                         for (int c = sq; c < m; c += P) r = __fma_rn(-yv[c], A[(size_t)c * n + v], r);
                     }
                     r = group_sum(r, P);
@@ -837,7 +829,7 @@ __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const To
                     if (act) {
                         const float* Tp = whole ? T + ((unsigned)pc >> 16) : df.slack + (size_t)u * m;
                     const int step = whole ? LD : 1;
-#pragma unroll kCertUnroll
+#pragma unroll kUnroll
                         for (int i = sq; i < m; i += P) acc = __fmaf_rn(rf[i], Tp[i * step], acc);
                     }
                     acc = group_sum(acc, P);
@@ -861,7 +853,7 @@ __device__ __forceinline__ void mixed_solve(G& g, const DeviceBatch& B, const To
             g.count_min(bad, 0u, bad, dummy);
             for (int j = tid; j < n; j += nt) {
                 double gj = 0.0, sc = 0.0;
-#pragma unroll kCertUnroll
+#pragma unroll kUnroll
                 for (int c = 0; c < m; ++c) {
                     const double a = A[(size_t)c * n + j];
                     gj = __fma_rn(yv[c], a, gj);

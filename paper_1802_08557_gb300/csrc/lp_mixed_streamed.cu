@@ -12,15 +12,15 @@
 // from L1.  Two CTAs per SM (64 registers): the kernel waits on L2 latency,
 // and twice the warps in flight measured 9% faster than one CTA with 128.
 
-// These kernels wait for loads from L2, not for instructions: 4 rows' loads in
-// flight against the 2 of the shared-memory kernels, 20,000 uneven LPs 5.51 -> 5.13
-// ms (12.40 -> 11.49 in one launch), 2000 of them 1.49 -> 1.41, 600 of 300 x 250
-// 1.48 -> 1.33.
-#define LPB_MIXED_UNROLL 4
 #include "lp_mixed_solve.cuh"
 
 namespace lpb {
 namespace {
+
+// These kernels wait for loads from L2, not for instructions: 4 rows' loads in
+// flight against 2, 20,000 uneven LPs 5.51 -> 5.13 ms (12.40 -> 11.49 in one
+// launch), 2000 of them 1.49 -> 1.41, 600 of 300 x 250 1.48 -> 1.33.
+constexpr int kUnroll = 4;
 
 __global__ void __launch_bounds__(kMixedStreamedThreads, 2)
 mixed_streamed_kernel(const DeviceBatch B, const Tolerances tol, const MixedParams mp,
@@ -39,7 +39,7 @@ mixed_streamed_kernel(const DeviceBatch B, const Tolerances tol, const MixedPara
         if (idx >= count) break;
         BlockGroup g(reinterpret_cast<long long*>(small + SmallLayout::red64),
                      reinterpret_cast<unsigned*>(small + SmallLayout::red32));
-        mixed_solve_lp(g, B, tol, mp, order[idx], big, fq, diag);
+        mixed_solve_lp<kUnroll>(g, B, tol, mp, order[idx], big, fq, diag);
         __syncthreads();
     }
 }
@@ -67,9 +67,9 @@ mixed_deferred_kernel(const DeviceBatch B, const Tolerances tol, const MixedPara
         BlockGroup g(reinterpret_cast<long long*>(smem + SmallLayout::red64),
                      reinterpret_cast<unsigned*>(smem + SmallLayout::red32));
         if (split_width(B.m[lp]) > 1)
-            mixed_solve<BlockGroup, true, true>(g, B, tol, mp, lp, area, fq, diag, bytes, slot);
+            mixed_solve<kUnroll, BlockGroup, true, true>(g, B, tol, mp, lp, area, fq, diag, bytes, slot);
         else
-            mixed_solve<BlockGroup, false, true>(g, B, tol, mp, lp, area, fq, diag, bytes, slot);
+            mixed_solve<kUnroll, BlockGroup, false, true>(g, B, tol, mp, lp, area, fq, diag, bytes, slot);
         __syncthreads();
     }
 }
@@ -109,9 +109,9 @@ mixed_single_kernel(const DeviceBatch B, const Tolerances tol, const MixedParams
         BlockGroup g(reinterpret_cast<long long*>(smem + SmallLayout::red64),
                      reinterpret_cast<unsigned*>(smem + SmallLayout::red32));
         if (resident[lp])
-            mixed_solve_lp(g, B, tol, mp, lp, smem + SmallLayout::total, fq, diag);
+            mixed_solve_lp<kUnroll>(g, B, tol, mp, lp, smem + SmallLayout::total, fq, diag);
         else if (slot)
-            mixed_solve_lp(g, B, tol, mp, lp, slot, fq, diag);
+            mixed_solve_lp<kUnroll>(g, B, tol, mp, lp, slot, fq, diag);
         else if (threadIdx.x == 0)
             record_internal_error(diag, 7, lp);  // a plan without a slot for a streamed LP
         __syncthreads();
@@ -124,7 +124,7 @@ mixed_single_kernel(const DeviceBatch B, const Tolerances tol, const MixedParams
     while (idx < count) {
         const int nxt = leader ? atomicAdd(counter, 1) : 0;
         WarpGroup g;
-        mixed_solve_lp(g, B, tol, mp, order[idx], area, fq, diag);
+        mixed_solve_lp<kUnroll>(g, B, tol, mp, order[idx], area, fq, diag);
         idx = __shfl_sync(0xffffffffu, nxt, 0);
     }
 }
