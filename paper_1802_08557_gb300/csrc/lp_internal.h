@@ -212,9 +212,12 @@ __host__ __device__ inline size_t mixed_smem_bytes(int m, int n, int k) {
 // The mixed path with deferred updates (lp_mixed_deferred.cuh): the k-independent
 // arrays of MixedLayout (up to its T), then the FP32 vectors, then (from
 // `hist`) the first pending pivots.
-// pending pivots before the whole tableau is formed (24: 2000 uneven LPs 2.7 ms,
-// 32 to 64: 1.3)
-constexpr int kMixedFirst = 48;
+// pending pivots before the whole tableau is formed.  Packing LPs of A in [0, 1],
+// 2000 uneven ones (8 pivots on average): 24 2.7 ms, 32 to 96 1.3.  Of A in [1, 10]
+// (twice the pivots), 48 / 64 / 96: 250 of 150 x 150 0.50 / 0.32 / 0.32 ms, 500 of 200 x
+// 200 0.92 / 0.96 / 0.64, 2500 of 300 x 300 9.5 / 7.6 / 7.0, 4000 uneven ones of 10 to 500
+// rows and columns 4.4 / 4.4 / 2.2; in the whole-tableau form 0.29, 0.76, 15.8 and 7.2.
+constexpr int kMixedFirst = 96;
 struct MixedDeferredLayout {
     size_t beta, rf, row_last, negidx, obj, aux, col_var, col_last, hist;
 };

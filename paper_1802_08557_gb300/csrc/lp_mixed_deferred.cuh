@@ -175,12 +175,17 @@ struct Deferred32 {
     }
     // The whole tableau after every pending pivot into T, in the whole-tableau
     // form's layout (retired columns 0: their labels keep them out): an LP of
-    // many pivots goes on there.  A thread takes a few columns and runs down the
-    // rows with several pivots' entries of them in registers, so that an
-    // element's step is an FMA and a share of a broadcast load.
+    // many pivots goes on there.  A warp takes 64 columns and kRows rows at a
+    // time, with kPivots pivots' entries of the columns in registers and those
+    // of the rows one per lane, so that a step waits for one round of loads per
+    // 8 x 4 x 64 FMAs.  Bound by that latency: in the tail of a batch an LP's CTA is
+    // alone on its SM.  One row at a time against this (packing LPs of A in [1, 10], 48
+    // pending pivots, one LP in a hundred handed over): 250 of 150 x 150 0.60 -> 0.50
+    // ms, 2500 of 300 x 300 11.1 -> 9.5.
     template <class G>
     __device__ void hand_over(G& g) {
-        constexpr int kCols = 2, kPivots = 8;
+        constexpr int kCols = 2, kPivots = 8, kRows = 4;
+        static_assert(kPivots * kRows == 32, "one lane per row and pivot");
         g.sync();  // row_last and col_last as settled
         const int nm = n + m;
         const int strips = (W + 32 * kCols - 1) / (32 * kCols);
@@ -203,31 +208,43 @@ struct Deferred32 {
                 for (int u = 0; u < kPivots; ++u)
 #pragma unroll
                     for (int q = 0; q < kCols; ++q) r[u][q] = on[q] && p0 + u < t ? r_at(p0 + u)[j[q]] : 0.0f;
-                for (int i = part; i < m; i += groups) {
-                    const int sr = row_last[i];
-                    float v[kCols];
+                for (int i0 = part * kRows; i0 < m; i0 += groups * kRows) {
+                    const int ls = p0 + g.lane / kRows, li = i0 + g.lane % kRows;
+                    const float c = ls < t && li < m ? -c_at(ls)[li] : 0.0f;
+                    int sr[kRows];
+                    float v[kRows][kCols];
 #pragma unroll
-                    for (int q = 0; q < kCols; ++q) {
-                        v[q] = 0.0f;
-                        if (p0 > 0 && on[q]) v[q] = T[(size_t)i * LD + j[q]];
-                        else if (on[q] && sr < 0 && sc[q] < 0) v[q] = source(i, j[q]);
+                    for (int a = 0; a < kRows; ++a) {
+                        const int i = min(i0 + a, m - 1);  // past the last row: that row again, not stored
+                        sr[a] = row_last[i];
+#pragma unroll
+                        for (int q = 0; q < kCols; ++q) {
+                            v[a][q] = 0.0f;
+                            if (p0 > 0 && on[q]) v[a][q] = T[(size_t)i * LD + j[q]];
+                            else if (on[q] && sr[a] < 0 && sc[q] < 0) v[a][q] = source(i, j[q]);
+                        }
                     }
 #pragma unroll
                     for (int u = 0; u < kPivots; ++u) {
                         const int s = p0 + u;
                         if (s < t) {
-                            const float b = -c_at(s)[i];
 #pragma unroll
-                            for (int q = 0; q < kCols; ++q) {
-                                const int last = max(sr, sc[q]);
-                                if (s == last) v[q] = (sr >= sc[q]) ? r[u][q] : __fmaf_rn(b, r[u][q], 0.0f);
-                                else if (s > last) v[q] = __fmaf_rn(b, r[u][q], v[q]);
+                            for (int a = 0; a < kRows; ++a) {
+                                const float b = __shfl_sync(kFull, c, u * kRows + a);
+#pragma unroll
+                                for (int q = 0; q < kCols; ++q) {
+                                    const int last = max(sr[a], sc[q]);
+                                    if (s == last) v[a][q] = (sr[a] >= sc[q]) ? r[u][q] : __fmaf_rn(b, r[u][q], 0.0f);
+                                    else if (s > last) v[a][q] = __fmaf_rn(b, r[u][q], v[a][q]);
+                                }
                             }
                         }
                     }
 #pragma unroll
-                    for (int q = 0; q < kCols; ++q)
-                        if (in[q]) T[(size_t)i * LD + j[q]] = v[q];
+                    for (int a = 0; a < kRows; ++a)
+#pragma unroll
+                        for (int q = 0; q < kCols; ++q)
+                            if (in[q] && i0 + a < m) T[(size_t)(i0 + a) * LD + j[q]] = v[a][q];
                 }
             }
         }
