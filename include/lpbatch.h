@@ -81,9 +81,12 @@ typedef struct {
     double eps_piv;      /* default 1e-9                                          */
     double eps_feas;     /* default 1e-9                                          */
     double tau;          /* relative tie window, default 1e-12                    */
-    int32_t block_threads; /* threads per LP (one CTA per LP); 0 = from the LP size;
-                              with LP_PREC_FP32_REFINE, 32 = one warp per LP       */
-    int32_t schedule;    /* LPB_SCHED_AUTO or LPB_SCHED_STREAMED                   */
+    int32_t block_threads; /* threads per LP (one CTA per LP) of the LPs whose tableau
+                              fits in one CTA's shared memory: > 0 also keeps all of
+                              them there; 0 = from the LP size; with
+                              LP_PREC_FP32_REFINE, 32 = one warp per LP.  Not used by
+                              the other LPs, LPB_SCHED_STREAMED and LPB_SCHED_SINGLE */
+    int32_t schedule;    /* LPB_SCHED_AUTO, _STREAMED, _CLUSTER or _SINGLE          */
 } lp_batch_opts;
 
 /* Kernel choice.  AUTO: shared-memory-resident tableau when it fits in one
@@ -255,7 +258,9 @@ lpb_err lp_batch_solve_graph(lp_batch *h, void *stream);
  * 32, 64, 128, 256) in both forms -- one CTA per LP, or persistent CTAs over an atomic
  * work queue with the LPs in descending order of work (groups that need the
  * whole 227 KB of a CTA's shared memory: one CTA per LP only) -- `rounds` times each,
- * and keep the fastest.  No counterpart in the paper.  Results of a solve do
+ * and keep the fastest; for a group with deferred updates all of whose LPs fit in
+ * shared memory, the fastest of these and of its own form.  Groups that do not fit
+ * keep their form.  No counterpart in the paper.  Results of a solve do
  * not depend on these choices.  The trial launches overwrite the outputs, so
  * call lp_batch_solve again before lp_batch_results.  Waits for the GPU. */
 lpb_err lp_batch_autotune(lp_batch *h, int32_t rounds, void *stream);
@@ -278,7 +283,9 @@ lpb_err lp_batch_group_info(lp_batch *h, int32_t index, lp_batch_group *out);
 /* Set a group's form by hand (threads a multiple of 32, at most 512; for a
  * mixed-precision group 32 without persistent selects one warp per LP;
  * persistent 0 or 1, and 0 for groups that need more than 226 KB of shared
- * memory).  Streamed groups are fixed. */
+ * memory).  A group with deferred updates (kind 2 or 4) all of whose LPs fit in
+ * shared memory moves there (kind 1 or 0); the other groups in a workspace, and
+ * those of LPB_SCHED_STREAMED, are fixed. */
 lpb_err lp_batch_set_group_form(lp_batch *h, int32_t index, int32_t threads, int32_t persistent);
 
 /* Device timing of the stages of lp_batch_solve, off by default.  enable != 0

@@ -211,7 +211,9 @@ struct lp_batch {
     int32_t num_phase1 = 0;
     size_t max_smem = 0;
     // FP64 LPs with deferred updates and a global workspace slot, one group per
-    // size class: order[offset ...), persistent CTAs over slots
+    // size class: order[offset ...), persistent CTAs over slots.  `whole`: the same
+    // LPs with their tableaux in shared memory, where all of them fit (fits), run
+    // instead when the caller or the tuner chose it (use_whole).
     struct DeferredGroup {
         lpb::DeferredForm form;
         int64_t offset;
@@ -219,6 +221,8 @@ struct lp_batch {
         size_t slot_bytes;
         unsigned char* workspace;
         int32_t* counter;
+        Group whole;
+        bool fits, use_whole;
     };
     std::vector<DeferredGroup> deferred_groups;
     // mixed precision with deferred updates, one group per size class
@@ -229,6 +233,8 @@ struct lp_batch {
         size_t slot_bytes;
         unsigned char* workspace;
         int32_t* counter;
+        Group whole;
+        bool fits, use_whole;
     };
     std::vector<MixedDeferredGroup> mdeferred_groups;
     int32_t num_mdeferred = 0;
@@ -378,6 +384,16 @@ cudaError_t launch_group(lp_batch* h, int kind, const Group& g, cudaStream_t ls)
     return lpb::launch_fp64_resident(h->d, h->tol, order, g.count, g.threads, g.smem, h->diag, ls);
 }
 
+// A group with deferred updates on stream ls.
+cudaError_t launch_deferred(lp_batch* h, const lp_batch::DeferredGroup& g, cudaStream_t ls) {
+    return lpb::launch_fp64_deferred(h->d, h->tol, h->d_order + g.offset, g.count, g.form, g.slots, g.workspace,
+                                     g.slot_bytes, g.counter, h->diag, ls);
+}
+cudaError_t launch_deferred(lp_batch* h, const lp_batch::MixedDeferredGroup& g, cudaStream_t ls) {
+    return lpb::launch_mixed_deferred(h->d, h->tol, h->mp, h->d_order + g.offset, g.count, g.form, g.slots, g.workspace,
+                                      g.slot_bytes, g.counter, fallback_queues(h), h->diag, ls);
+}
+
 // Everything a solve enqueues on stream s: counters reset, launch groups forked
 // onto the internal streams (largest first, round robin) and joined back, the
 // FP64 re-solve of uncertified LPs; with `timing`, the stage events.
@@ -433,12 +449,10 @@ lpb_err enqueue_solve(lp_batch* h, cudaStream_t s, bool timing) {
                                           h->single_counter, h->diag, ls);
         } else if (j.kind == 2) {
             const auto& dg = *reinterpret_cast<const lp_batch::DeferredGroup*>(j.g);
-            err = lpb::launch_fp64_deferred(h->d, h->tol, h->d_order + dg.offset, dg.count, dg.form, dg.slots,
-                                            dg.workspace, dg.slot_bytes, dg.counter, h->diag, ls);
+            err = dg.use_whole ? launch_group(h, 1, dg.whole, ls) : launch_deferred(h, dg, ls);
         } else if (j.kind == 6) {
             const auto& mg = *reinterpret_cast<const lp_batch::MixedDeferredGroup*>(j.g);
-            err = lpb::launch_mixed_deferred(h->d, h->tol, h->mp, h->d_order + mg.offset, mg.count, mg.form, mg.slots,
-                                             mg.workspace, mg.slot_bytes, mg.counter, fallback_queues(h), h->diag, ls);
+            err = mg.use_whole ? launch_group(h, 0, mg.whole, ls) : launch_deferred(h, mg, ls);
         } else if (j.kind == 4) {
             err = lpb::launch_mixed_streamed(h->d, h->tol, h->mp, h->d_order + h->mstream_offset, h->num_mstream,
                                              h->mstream_slots, h->mworkspace, h->mslot_bytes, h->mcounter,
@@ -727,7 +741,9 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
                 }
                 continue;
             }
-            if (o.schedule == LPB_SCHED_AUTO && lpb::mixed_defer_updates(hm[k], hn[k], hk[k], nonneg[k], h->uniform_m < 0)) {
+            // (a requested thread count keeps the LPs that fit in shared memory there)
+            if (o.schedule == LPB_SCHED_AUTO && (o.block_threads <= 0 || mneed > queue_smem_cap) &&
+                lpb::mixed_defer_updates(hm[k], hn[k], hk[k], nonneg[k], h->uniform_m < 0)) {
                 mdeferred[lpb::mixed_deferred_form(hm[k], hn[k]).cls].push_back(k);
                 continue;
             }
@@ -775,7 +791,8 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
                 continue;
             }
         }
-        if (o.schedule == LPB_SCHED_STREAMED || lpb::defer_updates(hm[k], hn[k], hk[k], nonneg[k])) {
+        if (o.schedule == LPB_SCHED_STREAMED || need > lpb::kMaxSmemPerBlock ||
+            (o.block_threads <= 0 && lpb::defer_updates(hm[k], hn[k], hk[k], nonneg[k]))) {
             defer(k);
             continue;
         }
@@ -825,17 +842,6 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
         h->mixed_groups.push_back(g);
         h->num_mixed += g.count;
     }
-    {
-        // per-group device counters of the persistent form
-        std::vector<int32_t> lens;
-        for (Group& g : h->groups) { g.gi = (int32_t)lens.size(); lens.push_back(g.count); }
-        for (Group& g : h->mixed_groups) { g.gi = (int32_t)lens.size(); lens.push_back(g.count); }
-        if (!lens.empty()) {
-            if ((err = alloc(h, &h->group_len, lens.size(), s)) || (err = alloc(h, &h->group_counter, lens.size(), s)) ||
-                (err = cudaMemcpyAsync(h->group_len, lens.data(), lens.size() * 4, cudaMemcpyHostToDevice, s)))
-                return bail_cuda(err, "group counters");
-        }
-    }
     // cluster groups (a cluster shape that cannot be placed gets deferred updates)
     for (auto& kv : cluster_buckets) {
         const int C = kv.first;
@@ -871,7 +877,16 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
         g.form = lpb::mixed_deferred_form(hm[v[0]], hn[v[0]]);
         g.offset = (int64_t)order.size();
         g.count = (int32_t)v.size();
-        for (int32_t k : v) g.slot_bytes = std::max(g.slot_bytes, lpb::mixed_deferred_slot(hm[k], hn[k], hk[k]).total);
+        g.whole.offset = g.offset;
+        g.whole.count = g.count;
+        for (int32_t k : v) {
+            g.slot_bytes = std::max(g.slot_bytes, lpb::mixed_deferred_slot(hm[k], hn[k], hk[k]).total);
+            g.whole.threads = std::max(g.whole.threads, mixed_threads(hm[k], hn[k], hk[k], 0));
+            g.whole.smem = std::max(g.whole.smem, (lpb::mixed_smem_bytes(hm[k], hn[k], hk[k]) + 1023) / 1024 * 1024);
+            g.whole.smem_warp =
+                std::max(g.whole.smem_warp, (lpb::mixed_layout(hm[k], hn[k], hk[k]).total + 127) / 128 * 128);
+        }
+        g.fits = g.whole.smem <= queue_smem_cap;
         order.insert(order.end(), v.begin(), v.end());
         h->mdeferred_groups.push_back(g);
         h->num_mdeferred += g.count;
@@ -909,10 +924,33 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
         g.form = lpb::deferred_form(hm[v[0]], hn[v[0]], hk[v[0]], nonneg[v[0]]);
         g.offset = (int64_t)order.size();
         g.count = (int32_t)v.size();
-        for (int32_t k : v) g.slot_bytes = std::max(g.slot_bytes, lpb::deferred_slot(hm[k], hn[k], hk[k]).total);
+        g.whole.offset = g.offset;
+        g.whole.count = g.count;
+        size_t need = 0;
+        for (int32_t k : v) {
+            g.slot_bytes = std::max(g.slot_bytes, lpb::deferred_slot(hm[k], hn[k], hk[k]).total);
+            g.whole.threads = std::max(g.whole.threads, pick_threads(hm[k], hn[k], hk[k], 0));
+            need = std::max(need, lpb::resident_smem_bytes(hm[k], hn[k], hk[k]));
+        }
+        g.whole.smem = std::min(lpb::kMaxSmemPerBlock, (need + 4095) / 4096 * 4096);
+        // (LPB_SCHED_STREAMED asks for the workspace)
+        g.fits = o.schedule != LPB_SCHED_STREAMED && need <= lpb::kMaxSmemPerBlock;
         order.insert(order.end(), v.begin(), v.end());
         h->deferred_groups.push_back(g);
         h->num_streamed += g.count;
+    }
+    {
+        // per-group device counters of the persistent form
+        std::vector<int32_t> lens;
+        for (Group& g : h->groups) { g.gi = (int32_t)lens.size(); lens.push_back(g.count); }
+        for (Group& g : h->mixed_groups) { g.gi = (int32_t)lens.size(); lens.push_back(g.count); }
+        for (auto& g : h->deferred_groups) { g.whole.gi = (int32_t)lens.size(); lens.push_back(g.count); }
+        for (auto& g : h->mdeferred_groups) { g.whole.gi = (int32_t)lens.size(); lens.push_back(g.count); }
+        if (!lens.empty()) {
+            if ((err = alloc(h, &h->group_len, lens.size(), s)) || (err = alloc(h, &h->group_counter, lens.size(), s)) ||
+                (err = cudaMemcpyAsync(h->group_len, lens.data(), lens.size() * 4, cudaMemcpyHostToDevice, s)))
+                return bail_cuda(err, "group counters");
+        }
     }
     // the last upload from pageable host memory, ahead of every memset and
     // kernel of this function: such a copy may wait for the stream, and
@@ -1117,48 +1155,62 @@ lpb_err lp_batch_autotune(lp_batch* h, int32_t rounds, void* stream) {
     if ((err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device))) return cuda_fail(err, "device query");
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if ((err = cudaEventCreate(&e0)) || (err = cudaEventCreate(&e1))) return cuda_fail(err, "tuning events");
-    auto time_group = [&](int kind, Group& g, float& best) -> cudaError_t {
-        float t_min = 1e30f;
+    // best of `rounds` launches by `launch`
+    auto time_form = [&](int kind, float& best, auto launch) -> cudaError_t {
+        best = 1e30f;
         for (int r = 0; r < rounds; ++r) {
             cudaError_t e;
             if ((e = cudaMemsetAsync(h->diag, 0, 32, s))) return e;
             if (kind == 0 && ((e = cudaMemsetAsync(h->fb_len, 0, 4, s)) || (e = cudaMemsetAsync(h->fbig_len, 0, 4, s))))
                 return e;
-            if ((e = cudaEventRecord(e0, s)) || (e = launch_group(h, kind, g, s)) || (e = cudaEventRecord(e1, s)) ||
+            if ((e = cudaEventRecord(e0, s)) || (e = launch()) || (e = cudaEventRecord(e1, s)) ||
                 (e = cudaEventSynchronize(e1)))
                 return e;
             float ms = 0.0f;
             if ((e = cudaEventElapsedTime(&ms, e0, e1))) return e;
-            t_min = std::min(t_min, ms);
-        }
-        best = t_min;
-        return cudaSuccess;
-    };
-    auto tune = [&](int kind, std::vector<Group>& gs, std::initializer_list<int> cand) -> cudaError_t {
-        for (Group& g : gs) {
-            Group best_g = g;
-            float best = 1e30f;
-            // the queue kernels keep a word of static shared memory: the
-            // largest groups run one CTA per LP only
-            const int max_form = g.smem <= lpb::kMaxSmemPerBlock - 1024 ? 1 : 0;
-            for (int persistent = 0; persistent <= max_form; ++persistent)
-                for (int threads : cand) {
-                    Group t = g;
-                    t.threads = threads;
-                    t.persistent = persistent;
-                    if (persistent) size_persistent(t, kind, sms);
-                    float ms = 0.0f;
-                    cudaError_t e = time_group(kind, t, ms);
-                    if (e != cudaSuccess) return e;
-                    if (ms < best) { best = ms; best_g = t; }
-                }
-            best_g.tuned_ms = best;
-            g = best_g;
+            best = std::min(best, ms);
         }
         return cudaSuccess;
     };
-    err = tune(1, h->groups, {32, 64, 128, 256, 512});
-    if (!err) err = tune(0, h->mixed_groups, {32, 64, 128, 256});
+    auto tune = [&](int kind, Group& g) -> cudaError_t {
+        Group best_g = g;
+        float best = 1e30f;
+        // the queue kernels keep a word of static shared memory: the
+        // largest groups run one CTA per LP only
+        const int max_form = g.smem <= lpb::kMaxSmemPerBlock - 1024 ? 1 : 0;
+        for (int persistent = 0; persistent <= max_form; ++persistent)
+            for (int threads = 32; threads <= (kind == 1 ? 512 : 256); threads *= 2) {
+                Group t = g;
+                t.threads = threads;
+                t.persistent = persistent;
+                if (persistent) size_persistent(t, kind, sms);
+                float ms = 0.0f;
+                cudaError_t e = time_form(kind, ms, [&] { return launch_group(h, kind, t, s); });
+                if (e != cudaSuccess) return e;
+                if (ms < best) { best = ms; best_g = t; }
+            }
+        best_g.tuned_ms = best;
+        g = best_g;
+        return cudaSuccess;
+    };
+    // groups with deferred updates: those against the shared-memory forms, where all their LPs fit
+    auto tune_deferred = [&](int kind, auto& groups) -> cudaError_t {
+        for (auto& g : groups) {
+            if (!g.fits) continue;
+            float ms = 0.0f;
+            cudaError_t e = time_form(kind, ms, [&] { return launch_deferred(h, g, s); });
+            if (e != cudaSuccess || (e = tune(kind, g.whole)) != cudaSuccess) return e;
+            g.use_whole = g.whole.tuned_ms < ms;
+            if (!g.use_whole) g.whole.tuned_ms = ms;
+        }
+        return cudaSuccess;
+    };
+    for (Group& g : h->groups)
+        if (!err) err = tune(1, g);
+    for (Group& g : h->mixed_groups)
+        if (!err) err = tune(0, g);
+    if (!err) err = tune_deferred(1, h->deferred_groups);
+    if (!err) err = tune_deferred(0, h->mdeferred_groups);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (err) return cuda_fail(err, "autotune");
@@ -1174,13 +1226,19 @@ lpb_err lp_batch_set_group_form(lp_batch* h, int32_t index, int32_t threads, int
     g_last_error.clear();
     if (!h) return fail(LPB_EINVAL, "handle is NULL");
     const int32_t nr = (int32_t)h->groups.size(), nm = (int32_t)h->mixed_groups.size();
-    if (index < 0 || index >= nr + nm) return fail(LPB_EINVAL, "group index out of range (or a streamed group)");
-    const int kind = index < nr ? 1 : 0;
+    const int32_t d0 = nr + nm + (int32_t)h->cluster_groups.size();  // groups with deferred updates
+    const int32_t ns = (int32_t)h->deferred_groups.size(), nmd = (int32_t)h->mdeferred_groups.size();
+    lp_batch::DeferredGroup* dg = index >= d0 && index < d0 + ns ? &h->deferred_groups[index - d0] : nullptr;
+    lp_batch::MixedDeferredGroup* mg =
+        index >= d0 + ns && index < d0 + ns + nmd ? &h->mdeferred_groups[index - d0 - ns] : nullptr;
+    const bool fits = dg ? dg->fits : (mg ? mg->fits : index >= 0 && index < nr + nm);
+    if (!fits) return fail(LPB_EINVAL, "group index out of range (or a group that is not in shared memory)");
+    const int kind = dg || (!mg && index < nr) ? 1 : 0;
     if (threads < 32 || threads > lpb::kMaxThreads || threads % 32)
         return fail(LPB_EINVAL, "threads must be a multiple of 32 within the kernel's range");
     if (persistent != 0 && persistent != 1) return fail(LPB_EINVAL, "persistent must be 0 or 1");
     DeviceGuard guard(h->device);
-    Group& g = index < nr ? h->groups[index] : h->mixed_groups[index - nr];
+    Group& g = dg ? dg->whole : (mg ? mg->whole : (index < nr ? h->groups[index] : h->mixed_groups[index - nr]));
     if (persistent && g.smem > lpb::kMaxSmemPerBlock - 1024)
         return fail(LPB_EINVAL, "this group's shared memory leaves no room for the persistent form");
     g.threads = threads;
@@ -1192,6 +1250,8 @@ lpb_err lp_batch_set_group_form(lp_batch* h, int32_t index, int32_t threads, int
         if (err) return cuda_fail(err, "device query");
         size_persistent(g, kind, sms);
     }
+    if (dg) dg->use_whole = true;
+    if (mg) mg->use_whole = true;
     if (h->graph_exec) {
         cudaGraphExecDestroy(h->graph_exec);
         h->graph_exec = nullptr;
@@ -1229,30 +1289,35 @@ lpb_err lp_batch_group_info(lp_batch* h, int32_t index, lp_batch_group* out) {
         out->cluster_ctas = g.C;
         return LPB_OK;
     }
-    if (index < nr + nm) {
-        const Group& g = index < nr ? h->groups[index] : h->mixed_groups[index - nr];
-        out->kind = index < nr ? 1 : 0;
+    // a shared-memory form
+    auto whole = [&](int kind, const Group& g) {
+        out->kind = kind;
         out->count = g.count;
         out->threads = g.threads;
         out->persistent = g.persistent;
-        out->smem_bytes = (int64_t)(index >= nr && g.threads == 32 && !g.persistent ? g.smem_warp : g.smem);
+        out->smem_bytes = (int64_t)(kind == 0 && g.threads == 32 && !g.persistent ? g.smem_warp : g.smem);
         out->tuned_ms = g.tuned_ms;
+    };
+    auto deferred = [&](int kind, const auto& g) {
+        out->kind = kind;
+        out->count = g.count;
+        out->threads = g.form.threads;
+        out->persistent = 1;
+        out->smem_bytes = (int64_t)g.form.smem;
+        out->tuned_ms = g.whole.tuned_ms;
+    };
+    if (index < nr) {
+        whole(1, h->groups[index]);
+    } else if (index < nr + nm) {
+        whole(0, h->mixed_groups[index - nr]);
     } else if (index < nr + nm + nc + ns) {
         const lp_batch::DeferredGroup& g = h->deferred_groups[index - nr - nm - nc];
-        out->kind = 2;
-        out->count = g.count;
-        out->threads = g.form.threads;
-        out->persistent = 1;
-        out->smem_bytes = (int64_t)g.form.smem;
-        out->tuned_ms = -1.0f;
+        if (g.use_whole) whole(1, g.whole);
+        else deferred(2, g);
     } else if (index < nr + nm + nc + ns + nmd) {
         const lp_batch::MixedDeferredGroup& g = h->mdeferred_groups[index - nr - nm - nc - ns];
-        out->kind = 4;
-        out->count = g.count;
-        out->threads = g.form.threads;
-        out->persistent = 1;
-        out->smem_bytes = (int64_t)g.form.smem;
-        out->tuned_ms = -1.0f;
+        if (g.use_whole) whole(0, g.whole);
+        else deferred(4, g);
     } else {
         out->kind = 4;
         out->count = h->num_mstream;
@@ -1487,7 +1552,18 @@ lpb_err lp_batch_plan_info(lp_batch* h, lp_batch_plan* plan) {
     plan->num_groups = (int32_t)(h->groups.size() + h->mixed_groups.size() + h->cluster_groups.size()) +
                        (int32_t)(h->deferred_groups.size() + h->mdeferred_groups.size()) + (h->num_mstream > 0 ? 1 : 0) + (h->num_fsmall > 0 ? 1 : 0) +
                        (h->num_fbig > 0 ? 1 : 0) + (h->num_single > 0 ? 1 : 0);
-    plan->num_resident = h->num_lps - h->num_streamed - h->num_mstream - h->num_mdeferred - h->num_cluster - h->num_single_streamed;
+    int32_t in_workspace = h->num_streamed + h->num_mstream + h->num_mdeferred + h->num_single_streamed;
+    size_t max_smem = h->max_smem;
+    auto not_whole = [&](const auto& groups) {
+        for (const auto& g : groups)
+            if (g.use_whole) {
+                in_workspace -= g.count;
+                max_smem = std::max(max_smem, g.whole.smem);
+            }
+    };
+    not_whole(h->deferred_groups);
+    not_whole(h->mdeferred_groups);
+    plan->num_resident = h->num_lps - in_workspace - h->num_cluster;
     plan->num_cluster = h->num_cluster;
     plan->num_mixed = h->num_mixed;
     plan->num_fallback = 0;
@@ -1519,9 +1595,9 @@ lpb_err lp_batch_plan_info(lp_batch* h, lp_batch_plan* plan) {
         plan->internal_error_lp = dg[0] ? dg[2] : -1;
         for (int i = 0; i < 5; ++i) plan->internal_error_detail[i] = dg[0] ? dg[3 + i] : 0;
     }
-    plan->num_streamed = h->num_streamed + h->num_mstream + h->num_mdeferred + h->num_single_streamed;
+    plan->num_streamed = in_workspace;
     plan->num_phase1 = h->num_phase1;
-    plan->max_smem_bytes = (int64_t)h->max_smem;
+    plan->max_smem_bytes = (int64_t)max_smem;
     plan->workspace_bytes = (int64_t)h->mstream_slots * (int64_t)h->mslot_bytes +
                             (int64_t)h->fbig_slots * (int64_t)h->fbig_slot_bytes +
                             (h->single_workspace ? (int64_t)h->single_ctas * (int64_t)h->single_slot_bytes : 0);
