@@ -85,7 +85,7 @@ typedef struct {
                               fits in one CTA's shared memory: > 0 also keeps all of
                               them there; 0 = from the LP size; with
                               LP_PREC_FP32_REFINE, 32 = one warp per LP.  Not used by
-                              the other LPs, LPB_SCHED_STREAMED and LPB_SCHED_SINGLE */
+                              the other LPs and LPB_SCHED_STREAMED                 */
     int32_t schedule;    /* LPB_SCHED_AUTO, _STREAMED, _CLUSTER or _SINGLE          */
 } lp_batch_opts;
 

@@ -163,8 +163,28 @@ int lanes_for(size_t groups) { return (int)std::min<size_t>(groups, std::min<siz
 // Solves whose stage times lp_batch_stage_times can average.
 constexpr int kTimingRing = 64;
 
-// Cap of the streamed kernel's global workspace (slots x largest tableau).
+// Cap of a solve's global workspace: of the slots of all its groups together, and
+// of the FP64 re-solve's.
 constexpr int64_t kMaxWorkspaceBytes = int64_t(16) << 30;
+
+// Workspace slots of groups that run at the same time: what each can use, and
+// where that is more than kMaxWorkspaceBytes in total, one each and the same
+// share of the rest for all.
+struct SlotWant {
+    int64_t want, bytes;  // slots the group can use (>= 1), bytes per slot
+};
+std::vector<int32_t> share_slots(const std::vector<SlotWant>& w) {
+    double all = 0, one = 0;
+    for (const SlotWant& g : w) {
+        all += (double)g.want * (double)g.bytes;
+        one += (double)g.bytes;
+    }
+    const double cap = (double)kMaxWorkspaceBytes;
+    const double share = all <= cap ? 1.0 : (all > one ? std::max(0.0, cap - one) / (all - one) : 0.0);
+    std::vector<int32_t> slots;
+    for (const SlotWant& g : w) slots.push_back((int32_t)(1 + (int64_t)((double)(g.want - 1) * share)));
+    return slots;
+}
 
 // LPB_SCHED_SINGLE: the largest tableau kept in shared memory (two 512-thread
 // CTAs per SM); larger ones go to the CTA's global workspace slot.
@@ -897,17 +917,6 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
     h->num_mstream = (int32_t)mstream.size();
     h->num_mixed += h->num_mstream;
     order.insert(order.end(), mstream.begin(), mstream.end());
-    if (h->num_mstream > 0) {
-        int sms = 0;
-        if ((err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device)))
-            return bail_cuda(err, "device query");
-        int64_t slots = (int64_t)sms * lpb::mixed_streamed_ctas_per_sm();
-        const int64_t cap = std::max<int64_t>(1, kMaxWorkspaceBytes / (int64_t)h->mslot_bytes);
-        slots = std::min<int64_t>({slots, (int64_t)h->num_mstream, cap});
-        h->mstream_slots = (int32_t)slots;
-        if ((err = alloc(h, &h->mworkspace, (size_t)slots * h->mslot_bytes, s)) || (err = alloc(h, &h->mcounter, 1, s)))
-            return bail_cuda(err, "mixed streamed workspace allocation");
-    }
     lpt(single);
     lpt(single_warp);
     h->single_warp_from = (int32_t)single.size();
@@ -986,27 +995,37 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
         h->max_smem = std::max(h->max_smem, h->single_smem);
         if ((err = alloc(h, &h->single_counter, 1, s))) return bail_cuda(err, "single-launch counter");
     }
-    for (lp_batch::MixedDeferredGroup& g : h->mdeferred_groups) {
+    if (!h->mdeferred_groups.empty() || !h->deferred_groups.empty() || h->num_mstream > 0) {
         int sms = 0;
         if ((err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device)))
             return bail_cuda(err, "device query");
-        int64_t slots = (int64_t)sms * lpb::mixed_deferred_ctas_per_sm(g.form);
-        const int64_t cap = std::max<int64_t>(1, kMaxWorkspaceBytes / (int64_t)g.slot_bytes);
-        slots = std::min<int64_t>({slots, (int64_t)g.count, cap});
-        g.slots = (int32_t)slots;
-        if ((err = alloc(h, &g.workspace, (size_t)slots * g.slot_bytes, s)) || (err = alloc(h, &g.counter, 1, s)))
-            return bail_cuda(err, "workspace allocation");
-    }
-    for (lp_batch::DeferredGroup& g : h->deferred_groups) {
-        int sms = 0;
-        if ((err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device)))
-            return bail_cuda(err, "device query");
-        int64_t slots = (int64_t)sms * lpb::fp64_deferred_ctas_per_sm(g.form);
-        const int64_t cap = std::max<int64_t>(1, kMaxWorkspaceBytes / (int64_t)g.slot_bytes);
-        slots = std::min<int64_t>({slots, (int64_t)g.count, cap});
-        g.slots = (int32_t)slots;
-        if ((err = alloc(h, &g.workspace, (size_t)slots * g.slot_bytes, s)) || (err = alloc(h, &g.counter, 1, s)))
-            return bail_cuda(err, "workspace allocation");
+        auto want = [&](int ctas_per_sm, int32_t count, size_t bytes) {
+            return SlotWant{std::min<int64_t>((int64_t)sms * ctas_per_sm, count), (int64_t)bytes};
+        };
+        std::vector<SlotWant> wants;
+        for (const auto& g : h->mdeferred_groups)
+            wants.push_back(want(lpb::mixed_deferred_ctas_per_sm(g.form), g.count, g.slot_bytes));
+        for (const auto& g : h->deferred_groups)
+            wants.push_back(want(lpb::fp64_deferred_ctas_per_sm(g.form), g.count, g.slot_bytes));
+        if (h->num_mstream > 0) wants.push_back(want(lpb::mixed_streamed_ctas_per_sm(), h->num_mstream, h->mslot_bytes));
+        const std::vector<int32_t> slots = share_slots(wants);
+        size_t at = 0;
+        auto place = [&](auto& g) {
+            g.slots = slots[at++];
+            err = alloc(h, &g.workspace, (size_t)g.slots * g.slot_bytes, s);
+            if (!err) err = alloc(h, &g.counter, 1, s);
+            return err == cudaSuccess;
+        };
+        for (auto& g : h->mdeferred_groups)
+            if (!place(g)) return bail_cuda(err, "workspace allocation");
+        for (auto& g : h->deferred_groups)
+            if (!place(g)) return bail_cuda(err, "workspace allocation");
+        if (h->num_mstream > 0) {
+            h->mstream_slots = slots[at];
+            if ((err = alloc(h, &h->mworkspace, (size_t)h->mstream_slots * h->mslot_bytes, s)) ||
+                (err = alloc(h, &h->mcounter, 1, s)))
+                return bail_cuda(err, "mixed streamed workspace allocation");
+        }
     }
     if (h->num_mixed > 0) {
         h->mp.eps_opt32 = 1e-6f;
