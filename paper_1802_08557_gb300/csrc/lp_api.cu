@@ -206,6 +206,12 @@ int32_t count_negative(const double* b, int32_t m) {
     return cnt;
 }
 
+// How the plan looks for the sign of A under these options.
+lpb::SignLook sign_look(const lp_batch_opts& o) {
+    if (o.schedule != LPB_SCHED_AUTO) return lpb::kLookNot;
+    return o.precision == LP_PREC_FP32_REFINE ? lpb::kLookLeading : lpb::kLookSpread;
+}
+
 int mixed_threads(int m, int n, int k, int requested) {
     if (requested > 0) return pick_threads(m, n, k, requested);
     const int64_t e = (int64_t)(m + 1 + (k > 0)) * (n + k + 1);
@@ -662,10 +668,10 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
 
     h->d = lpb::DeviceBatch{dm, dn, da, db, dc, dx_off, dy_off, dA, dbv, dcv, dstatus, diters, dobj, dx, dy};
     h->d_order = dorder;
+    const lpb::SignLook look = sign_look(o);
     if (ptr_kind == LPB_DEVICE &&
         ((err = lpb::launch_input_check(dA, a_len, dbv, b_len, dcv, c_len, dbad, s)) ||
-         (err = lpb::launch_plan_info(
-              h->d, num_lps, o.schedule == LPB_SCHED_AUTO, dk, s))))
+         (err = lpb::launch_plan_info(h->d, num_lps, look, dk, s))))
         return bail_cuda(err, "input check kernel");
     std::vector<int32_t> hk(num_lps);
     std::vector<uint8_t> nonneg(num_lps, 0);  // no negative entry seen in A (device inputs only)

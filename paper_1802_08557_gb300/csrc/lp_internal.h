@@ -315,6 +315,20 @@ constexpr int64_t kDeferNonneg = 2000;  // least tableau entries of such an LP's
 __host__ __device__ inline bool sign_matters(int m, int n) {
     return (int64_t)(m + 1) * (n + 1) > kDeferNonneg && m >= 32 && n >= 32;
 }
+// Where the plan looks for a negative entry in an LP's A.  kLookSpread (FP64): 256
+// entries, 4 in a row at 64 places evenly over the whole of A, so that rows of one
+// sign ahead of others of mixed sign (budgets, capacities) are not taken for all
+// of them; a signed LP taken for a packing LP costs time: 1000 of 70 x 70 0.27
+// against 0.34 ms, 300 of 300 x 300 29.5 against 31.4.  kLookLeading (mixed
+// precision): the first 1024 entries; there such a guess costs nothing measured
+// (1000 LPs of 100 to 300 rows and columns 9.1 ms whole, 8.7 deferred).
+enum SignLook { kLookNot = 0, kLookLeading = 1, kLookSpread = 2 };
+__host__ __device__ inline int sign_samples(SignLook look) { return look == kLookLeading ? 1024 : 256; }
+// Entry of sample i (< sign_samples) in an A of len entries; len or more: none.
+__host__ __device__ inline int64_t sign_sample_at(SignLook look, int64_t len, int i) {
+    if (look == kLookLeading || len <= 256) return i;
+    return (int64_t)(i / 4) * (len - 4) / 63 + i % 4;
+}
 int resident_threads(int m, int n, int k);
 int fp64_deferred_ctas_per_sm(const DeferredForm& f);
 // Persistent CTAs (grid = slots) take LPs of `order` from the atomic `counter`
@@ -474,9 +488,9 @@ cudaError_t launch_input_check(double* A, int64_t a_len, double* b, int64_t b_le
 // info[lp] = the number of rows of LP lp with b_i < 0 (rows that get an
 // artificial), plus kPlanSigned unless a sample of A has no negative entry,
 // plus kPlanSameA if A is the previous LP's (kPlanSigned is then that LP's).
-// The sign is looked for with want_sign, and only where sign_matters.
+// The sign is looked for as `look` says, and only where sign_matters.
 constexpr int32_t kPlanSigned = 1 << 30, kPlanSameA = 1 << 29;
-cudaError_t launch_plan_info(const DeviceBatch& B, int32_t num_lps, bool want_sign, int32_t* info,
+cudaError_t launch_plan_info(const DeviceBatch& B, int32_t num_lps, SignLook look, int32_t* info,
                              cudaStream_t stream);
 
 // Up to five arrays copied device to device in one launch (lp_batch_results);

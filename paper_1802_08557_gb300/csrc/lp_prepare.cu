@@ -29,9 +29,9 @@ __global__ void check_finite_kernel(double* __restrict__ v, int64_t len, unsigne
 // One warp per LP: number of rows with b_i < 0 (rows that get an artificial),
 // with kPlanSigned added unless A was seen to have no negative entry, and
 // kPlanSameA when A is the previous LP's (its sign is then not looked for).  A
-// sample of A is read, its first 1024 entries, and only where its sign matters
-// to the plan: a wrong guess costs time, not results.
-__global__ void plan_info_kernel(const DeviceBatch B, int32_t num_lps, bool want_sign, int32_t* __restrict__ info) {
+// sample of A is read (SignLook), and only where its sign matters to the plan: a
+// wrong guess costs time, not results.
+__global__ void plan_info_kernel(const DeviceBatch B, int32_t num_lps, SignLook look, int32_t* __restrict__ info) {
     const int lane = threadIdx.x & 31;
     const int lp = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     if (lp >= num_lps) return;
@@ -41,18 +41,18 @@ __global__ void plan_info_kernel(const DeviceBatch B, int32_t num_lps, bool want
     for (int i = lane; i < m; i += 32) cnt += (bv[i] < 0.0) ? 1 : 0;
     cnt = __reduce_add_sync(0xffffffffu, cnt);
     int flags = kPlanSigned;  // where it was not looked for
-    if (want_sign && sign_matters(m, n)) {
+    if (look != kLookNot && sign_matters(m, n)) {
         if (lp > 0 && B.a_off[lp] == B.a_off[lp - 1] && m == B.m[lp - 1] && n == B.n[lp - 1]) {
             flags = kPlanSameA;
         } else {
             flags = 0;
             const double* A = B.A + B.a_off[lp];
-            const int64_t len = min((int64_t)m * n, (int64_t)1024);
-            for (int64_t i = 0; i < len && !flags; i += 512) {
+            const int64_t len = (int64_t)m * n;
+            for (int i = 0; i < sign_samples(look) && !flags; i += 256) {
                 bool negative = false;
 #pragma unroll
-                for (int q = 0; q < 16; ++q) {
-                    const int64_t at = i + q * 32 + lane;
+                for (int q = 0; q < 8; ++q) {
+                    const int64_t at = sign_sample_at(look, len, i + q * 32 + lane);
                     negative |= at < len && A[at] < 0.0;
                 }
                 if (__any_sync(0xffffffffu, negative)) flags = kPlanSigned;
@@ -103,11 +103,11 @@ cudaError_t launch_input_check(double* A, int64_t a_len, double* b, int64_t b_le
     return cudaGetLastError();
 }
 
-cudaError_t launch_plan_info(const DeviceBatch& B, int32_t num_lps, bool want_sign, int32_t* info,
+cudaError_t launch_plan_info(const DeviceBatch& B, int32_t num_lps, SignLook look, int32_t* info,
                              cudaStream_t stream) {
     const int t = 256;
     const int64_t threads = (int64_t)num_lps * 32;
-    plan_info_kernel<<<(unsigned)((threads + t - 1) / t), t, 0, stream>>>(B, num_lps, want_sign, info);
+    plan_info_kernel<<<(unsigned)((threads + t - 1) / t), t, 0, stream>>>(B, num_lps, look, info);
     return cudaGetLastError();
 }
 
