@@ -208,8 +208,26 @@ int32_t count_negative(const double* b, int32_t m) {
 
 // How the plan looks for the sign of A under these options.
 lpb::SignLook sign_look(const lp_batch_opts& o) {
-    if (o.schedule != LPB_SCHED_AUTO) return lpb::kLookNot;
-    return o.precision == LP_PREC_FP32_REFINE ? lpb::kLookLeading : lpb::kLookSpread;
+    const bool mixed = o.precision == LP_PREC_FP32_REFINE;
+    if (o.schedule == LPB_SCHED_AUTO && mixed) return lpb::kLookLeading;
+    if (o.schedule == LPB_SCHED_AUTO || (o.schedule == LPB_SCHED_CLUSTER && !mixed)) return lpb::kLookSpread;
+    return lpb::kLookNot;
+}
+
+// What launch_plan_info finds on the device, for an LP in host memory: its rows
+// with b_i < 0, plus kPlanSigned unless a sample of A has no negative entry.  The
+// sample costs the host some 0.5 us, so it is taken only of LPs whose copy takes
+// longer; a smaller packing LP from host memory keeps its tableau in shared memory.
+int32_t host_plan_info(const double* A, const double* b, int32_t m, int32_t n, lpb::SignLook look) {
+    const int32_t k = count_negative(b, m);
+    const int64_t least = look == lpb::kLookLeading ? lpb::kMixedDeferEntries : lpb::kDeferEntries;
+    if (look == lpb::kLookNot || (int64_t)(m + 1) * (n + k + 1) <= least) return k | lpb::kPlanSigned;
+    const int64_t len = (int64_t)m * n;
+    for (int i = 0; i < lpb::sign_samples(look); ++i) {
+        const int64_t at = lpb::sign_sample_at(look, len, i);
+        if (at < len && A[at] < 0.0) return k | lpb::kPlanSigned;
+    }
+    return k;
 }
 
 int mixed_threads(int m, int n, int k, int requested) {
@@ -560,14 +578,14 @@ const char* lpb_last_error(void) { return g_last_error.c_str(); }
 // the stream, leaving the count of non-finite inputs in h->d_bad for the
 // caller to read after its solve (the check zeroes every such entry, so the
 // solve sees finite data).  Without it the call waits for the check and fails
-// on a non-finite entry.  `phase1_rows` (host inputs only, optional): every
-// LP's count of rows with b_i < 0, already counted by the caller.
+// on a non-finite entry.  `plan_info` (host inputs only, optional): every LP's
+// host_plan_info, already found by the caller.
 static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, const int32_t* n,
                             const int64_t* a_off, const double* A, int64_t a_len,
                             const int64_t* b_off, const double* b, int64_t b_len,
                             const int64_t* c_off, const double* c, int64_t c_len,
                             int32_t ptr_kind, const lp_batch_opts* opts, void* stream, cudaEvent_t copied,
-                            bool defer_check, const int32_t* phase1_rows = nullptr) {
+                            bool defer_check, const int32_t* plan_info = nullptr) {
     g_last_error.clear();
     if (!out) return fail(LPB_EINVAL, "out is NULL");
     if (defer_check && ptr_kind != LPB_HOST) return fail(LPB_EINVAL, "a deferred input check needs host inputs");
@@ -674,18 +692,18 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
          (err = lpb::launch_plan_info(h->d, num_lps, look, dk, s))))
         return bail_cuda(err, "input check kernel");
     std::vector<int32_t> hk(num_lps);
-    std::vector<uint8_t> nonneg(num_lps, 0);  // no negative entry seen in A (device inputs only)
+    std::vector<uint8_t> nonneg(num_lps, 0);  // no negative entry seen in A
     unsigned long long bad = 0;
     if (ptr_kind == LPB_HOST) {
-        // phase-I rows counted here while the copies run (the plan below
+        // phase-I rows and signs found here while the copies run (the plan below
         // overlaps them too); the input check is launched after the last
         // upload of the plan, so that no host call of this function waits for
         // a kernel (a kernel queued behind another stream's large grid can
         // wait for most of that grid)
-        if (phase1_rows) {
-            std::copy(phase1_rows, phase1_rows + num_lps, hk.begin());
+        if (plan_info) {
+            std::copy(plan_info, plan_info + num_lps, hk.begin());
         } else {
-            for (int32_t k = 0; k < num_lps; ++k) hk[k] = count_negative(b + hb[k], hm[k]);
+            for (int32_t k = 0; k < num_lps; ++k) hk[k] = host_plan_info(A + ha[k], b + hb[k], hm[k], hn[k], look);
         }
     } else {
         if ((err = cudaMemcpyAsync(hk.data(), dk, nl * 4, cudaMemcpyDeviceToHost, s)) ||
@@ -693,10 +711,10 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
             (err = cudaStreamSynchronize(s)))
             return bail_cuda(err, "input check");
         if (bad) return bail(LPB_EINVAL, std::to_string(bad) + " non-finite entries in A, b or c");
-        for (int32_t k = 0; k < num_lps; ++k) {
-            nonneg[k] = (hk[k] & lpb::kPlanSameA) ? nonneg[k - 1] : !(hk[k] & lpb::kPlanSigned);
-            hk[k] &= ~(lpb::kPlanSigned | lpb::kPlanSameA);
-        }
+    }
+    for (int32_t k = 0; k < num_lps; ++k) {
+        nonneg[k] = (hk[k] & lpb::kPlanSameA) ? nonneg[k - 1] : !(hk[k] & lpb::kPlanSigned);
+        hk[k] &= ~(lpb::kPlanSigned | lpb::kPlanSameA);
     }
 
     // Plan: LPs whose tableau fits in one CTA's shared memory are grouped by
@@ -1743,11 +1761,15 @@ lpb_err lp_solve_host(int32_t num_lps, const int32_t* m, const int32_t* n,
     lpb_err e = LPB_OK;
     int64_t px = 0, py = 0;
     for (int32_t i = 0; i <= chunks; ++i) k0s[i] = (int32_t)((int64_t)num_lps * i / chunks);
-    // The phase-I row counts of ranges 1.. are taken by a helper thread while
-    // range 0 is created: each create would otherwise read its range's b on
+    // The phase-I row counts and signs of ranges 1.. are taken by a helper thread
+    // while range 0 is created: each create would otherwise read its range's b on
     // the host path that issues the copies (~0.3 ms per 12,500 LPs of 50 rows
     // on the GPU machine's host).
-    std::vector<int32_t> phase1(chunks > 1 ? (size_t)num_lps : 0);
+    lp_batch_opts o;
+    lpb_default_opts(&o);
+    if (opts) o = *opts;
+    const lpb::SignLook look = sign_look(o);
+    std::vector<int32_t> info(chunks > 1 ? (size_t)num_lps : 0);
     std::atomic<int32_t> counted{0};  // ranges 1 .. counted-1 are done
     std::thread counter;
     bool helper = false;
@@ -1756,7 +1778,8 @@ lpb_err lp_solve_host(int32_t num_lps, const int32_t* m, const int32_t* n,
         try {
             counter = std::thread([&] {
                 for (int32_t i = 1; i < chunks; ++i) {
-                    for (int32_t k = k0s[i]; k < k0s[i + 1]; ++k) phase1[k] = count_negative(b + hb[k], m[k]);
+                    for (int32_t k = k0s[i]; k < k0s[i + 1]; ++k)
+                        info[k] = host_plan_info(A + ha[k], b + hb[k], m[k], n[k], look);
                     counted.store(i + 1, std::memory_order_release);
                 }
             });
@@ -1799,7 +1822,7 @@ lpb_err lp_solve_host(int32_t num_lps, const int32_t* m, const int32_t* n,
             while (counted.load(std::memory_order_acquire) <= i) std::this_thread::yield();
         e = create_batch(&hs[i], k1 - k0, m + k0, n + k0, sa.data(), A + alo, ahi - alo, sb.data(), b + blo,
                          bhi - blo, sc.data(), c + clo, chi - clo, LPB_HOST, opts, streams[i], copied[i], true,
-                         helper && i > 0 ? phase1.data() + k0 : nullptr);
+                         helper && i > 0 ? info.data() + k0 : nullptr);
         if (e == LPB_OK) e = lp_batch_solve(hs[i], streams[i]);
     }
     if (helper) counter.join();

@@ -608,18 +608,32 @@ cudaError_t launch_fp64_resident_queue(const DeviceBatch& B, const Tolerances& t
 }
 
 // Deferred updates for every tableau above one CTA's shared memory, and below
-// that by size.  The number of pivots decides, and is not known beforehand; a
-// packing LP (no negative entry in A) takes few.  Measured, positive LPs,
-// deferred against resident, ms: 45 x 45 0.38 / 0.44, 40 x 60 0.41 / 0.53, 130 x 60
-// 0.99 / 1.19, 130 x 130 1.04 / 2.02, but 30 x 70 0.54 / 0.50, 16 x 130 0.97 / 0.56
-// (few elements per pivot row or column: the pivot's fixed cost counts) and
-// 20 x 20 0.22 / 0.20.  Other LPs, mixed signs: 130 x 130 (326 pivots) 34.7 / 37.5,
-// 100 x 100 (200 pivots) 20.3 / 18.5, 70 x 70 11.5 / 8.1.
+// that by size, shape and sign.  They save FMAs while few pivots are pending, and
+// spread a pivot's work over fewer threads; an LP that has to flush makes them
+// all after all.  The number of pivots decides, and is not known beforehand.
+// Measured on 1000 LPs, deferred / resident, ms:
+//  - packing LPs (no negative entry in A: few pivots) of both sides >= 32: 45 x 45
+//    (20,000) 0.47 / 0.74, 80 x 80 (2400) 0.28 / 0.39, 130 x 130 0.19 / 0.67, but 30 x 70
+//    0.54 / 0.50 and 16 x 130 0.97 / 0.56 (the pivot's fixed cost counts);
+//  - packing LPs of a shorter side, above 14,000 entries: 16 x 900 0.95 / 1.07, 24 x 600
+//    0.77 / 0.90, 750 x 20 0.24 / 0.61, 1600 x 8 0.31 / 0.72; with rows of more than 1024
+//    entries, which only one CTA per SM has room for, 8 x 1600 1.65 / 1.22, 12 x 1200
+//    1.42 / 1.15, 20 x 1100 1.67 / 1.44;
+//  - others, above 14,000 entries: rows longer than columns by half, 16 x 900 0.51 /
+//    0.67, 24 x 1000 1.12 / 1.32, 64 x 225 2.3 / 2.5, 90 x 250 4.9 / 5.4, 120 x 180 9.7 /
+//    9.9; a thread per row and column within 128, 125 x 125 12.9 / 13.8; fewer than 12
+//    columns (no more pivots than are kept pending), 1450 x 10 0.84 / 1.02, 2000 x 6 0.66 /
+//    0.86; but 130 x 130 17.0 / 15.5, 110 x 160 8.7 / 8.0, 250 x 90 17.7 / 14.1, 225 x 64
+//    8.1 / 5.6, 700 x 32 4.8 / 3.2, 1100 x 12 1.14 / 0.98, 16 x 1400 0.95 / 0.95 (with phase
+//    I 1.77 / 1.61).
 bool defer_updates(int m, int n, int k, bool nonneg) {
     if (resident_smem_bytes(m, n, k) > kMaxSmemPerBlock) return true;
-    const int64_t e = (int64_t)(m + 1) * (n + k + 1);
+    const int w = n + k + 1, d = m > w ? m : w;
+    const int64_t e = (int64_t)(m + 1) * w;
     if (nonneg && e > kDeferNonneg && m >= 32 && n >= 32) return true;
-    return e > 14000;
+    if (e <= kDeferEntries) return false;
+    if (d > 1024) return m > w && (nonneg || n < 12);
+    return nonneg || d <= 128 || 2 * w >= 3 * m;
 }
 
 int resident_threads(int m, int n, int k) {
@@ -643,7 +657,7 @@ DeferredForm deferred_form(int m, int n, int k, bool nonneg) {
     const int d = m > n + k + 1 ? m : n + k + 1;
     for (int c = 0; c < 4; ++c)
         if (d <= (32 << c)) return {c, 32 << c, (size_t)(9 << 10) << c};
-    if (d <= 1024) return nonneg ? DeferredForm{4, 256, 74 << 10} : DeferredForm{5, 512, 100 << 10};
+    if (d <= 1024) return nonneg && m >= 32 && n >= 32 ? DeferredForm{4, 256, 74 << 10} : DeferredForm{5, 512, 100 << 10};
     return {6, kMaxThreads, kMaxSmemPerBlock - 1024};
 }
 

@@ -307,13 +307,18 @@ struct DeferredForm {
 };
 constexpr int kDeferredClasses = 7;
 DeferredForm deferred_form(int m, int n, int k, bool nonneg);
-// Whether an LP gets deferred updates by default, and the threads per CTA of
-// the resident kernel for the others.  nonneg: no negative entry was seen in A;
-// a packing LP takes few pivots.
+// Whether deferred updates suit an LP better than its tableau in shared memory
+// (always, where that does not fit), and the threads per CTA of the resident
+// kernel for the others.  nonneg: no negative entry was seen in A; a packing LP
+// takes few pivots.
 bool defer_updates(int m, int n, int k, bool nonneg);
 constexpr int64_t kDeferNonneg = 2000;  // least tableau entries of such an LP's deferred updates
+constexpr int64_t kDeferEntries = 14000;  // ... of an LP of either sign, or of short rows or columns
+constexpr int64_t kMixedDeferEntries = 12000;
+// Whether the sign of an LP's A matters to the plan, for some number of artificials.
 __host__ __device__ inline bool sign_matters(int m, int n) {
-    return (int64_t)(m + 1) * (n + 1) > kDeferNonneg && m >= 32 && n >= 32;
+    return ((int64_t)(m + 1) * (n + 1) > kDeferNonneg && m >= 32 && n >= 32) ||
+           (int64_t)(m + 1) * (n + m + 1) > kDeferEntries;
 }
 // Where the plan looks for a negative entry in an LP's A.  kLookSpread (FP64): 256
 // entries, 4 in a row at 64 places evenly over the whole of A, so that rows of one

@@ -175,7 +175,7 @@ MixedDeferredForm mixed_deferred_form(int m, int n) {
 // whole-tableau forms keep them: an FP32 update is cheap, and positive LPs of
 // 200 x 200 (28 pivots) take 0.90 against 1.22 ms, 300 x 300 2.4 against 3.0.
 bool mixed_defer_updates(int m, int n, int k, bool nonneg, bool uneven) {
-    return uneven && nonneg && (int64_t)(m + 1) * (n + k + 1) > 12000 && m >= 32 && n >= 32 &&
+    return uneven && nonneg && (int64_t)(m + 1) * (n + k + 1) > kMixedDeferEntries && m >= 32 && n >= 32 &&
            SmallLayout::total + mixed_deferred_layout(m, n, k).hist <= mixed_deferred_form(m, n).smem;
 }
 
