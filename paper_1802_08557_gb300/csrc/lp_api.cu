@@ -686,6 +686,9 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
 
     h->d = lpb::DeviceBatch{dm, dn, da, db, dc, dx_off, dy_off, dA, dbv, dcv, dstatus, diters, dobj, dx, dy};
     h->d_order = dorder;
+    int sms = 0;
+    if ((err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device)))
+        return bail_cuda(err, "device query");
     const lpb::SignLook look = sign_look(o);
     if (ptr_kind == LPB_DEVICE &&
         ((err = lpb::launch_input_check(dA, a_len, dbv, b_len, dcv, c_len, dbad, s)) ||
@@ -949,12 +952,16 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
     h->num_single = (int32_t)single.size();
     if (o.precision == LP_PREC_FP32_REFINE) h->num_mixed += h->num_single;
     order.insert(order.end(), single.begin(), single.end());
+    if ((int64_t)deferred[4].size() < (int64_t)lpb::kDeferClass4PerSm * sms) {
+        deferred[5].insert(deferred[5].end(), deferred[4].begin(), deferred[4].end());
+        deferred[4].clear();
+    }
     for (int c = 0; c < lpb::kDeferredClasses; ++c) {
         std::vector<int32_t>& v = deferred[c];
         if (v.empty()) continue;
         lpt(v);
         lp_batch::DeferredGroup g{};
-        g.form = lpb::deferred_form(hm[v[0]], hn[v[0]], hk[v[0]], nonneg[v[0]]);
+        g.form = lpb::deferred_class(c);
         g.offset = (int64_t)order.size();
         g.count = (int32_t)v.size();
         g.whole.offset = g.offset;
@@ -995,7 +1002,6 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
         if ((err = alloc(h, &h->d_resident, (size_t)num_lps, s)) ||
             (err = cudaMemcpyAsync(h->d_resident, single_resident.data(), (size_t)num_lps, cudaMemcpyHostToDevice, s)))
             return bail_cuda(err, "plan upload");
-        int sms = 0;
         const bool mixed = o.precision == LP_PREC_FP32_REFINE;
         // (each LP's footprint above includes the reduction scratch its area follows)
         h->single_smem = std::max(h->single_smem, lpb::SmallLayout::total);
@@ -1003,8 +1009,7 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
         if (!mixed && h->num_single_streamed > 0)
             h->single_smem = std::max(h->single_smem, lpb::SmallLayout::total + lpb::kSingleDeferredBytes);
         h->single_smem = (h->single_smem + 1023) / 1024 * 1024;
-        if ((err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device)) ||
-            (err = mixed ? lpb::mixed_single_prepare(h->single_smem) : lpb::fp64_single_prepare(h->single_smem)))
+        if ((err = mixed ? lpb::mixed_single_prepare(h->single_smem) : lpb::fp64_single_prepare(h->single_smem)))
             return bail_cuda(err, "single launch set-up");
         const int per_sm = std::max(1, mixed ? lpb::mixed_single_ctas_per_sm(h->single_smem)
                                              : lpb::fp64_single_ctas_per_sm(h->single_smem));
@@ -1020,9 +1025,6 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
         if ((err = alloc(h, &h->single_counter, 1, s))) return bail_cuda(err, "single-launch counter");
     }
     if (!h->mdeferred_groups.empty() || !h->deferred_groups.empty() || h->num_mstream > 0) {
-        int sms = 0;
-        if ((err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device)))
-            return bail_cuda(err, "device query");
         auto want = [&](int ctas_per_sm, int32_t count, size_t bytes) {
             return SlotWant{std::min<int64_t>((int64_t)sms * ctas_per_sm, count), (int64_t)bytes};
         };
@@ -1070,9 +1072,7 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
             (err = alloc(h, &h->fbig_queue, (size_t)h->num_fbig, s)) || (err = alloc(h, &h->fbig_len, 1, s)) ||
             (err = alloc(h, &h->fbig_counter, 1, s)) || (err = cudaMemsetAsync(h->fbig_len, 0, 4, s)))
             return bail_cuda(err, "fallback queue allocation");
-        int sms = 0;
-        if ((err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device)) ||
-            (err = lpb::fp64_kernels_prepare()) || (err = lpb::mixed_kernel_prepare()))
+        if ((err = lpb::fp64_kernels_prepare()) || (err = lpb::mixed_kernel_prepare()))
             return bail_cuda(err, "device query");
         if (h->num_fsmall > 0)
             h->fb_ctas = sms * lpb::fp64_resident_queue_ctas_per_sm(h->fb_threads, h->fb_smem);

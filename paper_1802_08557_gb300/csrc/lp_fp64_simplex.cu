@@ -649,16 +649,27 @@ int resident_threads(int m, int n, int k) {
 // Size classes by the longer of a row and a column, d: a thread for each up to
 // 256 (a warp's FP64 instruction holds its quarter of the SM's FP64 pipe for 64
 // clocks, so one LP needs its elements spread over warps), 9 KB of shared memory
-// per warp, 24 warps per SM at 80 registers.  Above, several per thread: 256
-// threads and three CTAs per SM suit short runs of pivots (20,000 uneven packing
-// LPs 2.7 against 3.2 ms with 512), 512 threads the flushes of long ones (300
-// mixed-sign 300 x 300 LPs 179 against 238 ms).
+// per warp, 24 warps per SM at 80 registers.  Above, several per thread: 512
+// threads; 256 and three CTAs per SM (class 4) only for packing LPs by the
+// thousand (kDeferClass4PerSm), where throughput counts and not one LP's time.
+// Class 4 / 5, ms: uneven packing LPs, 20,000 (4200 of class 4) 2.66 / 2.95, 10,000
+// 1.73 / 1.71, 1000 0.92 / 0.75; 10,000 of 300 x 300 4.5 / 4.8, 2400 1.29 / 1.26, 200 0.35 /
+// 0.25; with A in [1, 10] (43 pivots) 200 6.3 / 4.4 (5.1 with the whole tableau
+// rewritten in the workspace at every pivot), 2400 9.3 / 7.4; 300 mixed-sign 300 x 300
+// LPs 238 / 179.
+DeferredForm deferred_class(int cls) {
+    if (cls < 4) return {cls, 32 << cls, (size_t)(9 << 10) << cls};
+    if (cls == 4) return {4, 256, 74 << 10};
+    if (cls == 5) return {5, 512, 100 << 10};
+    return {6, kMaxThreads, kMaxSmemPerBlock - 1024};
+}
+
 DeferredForm deferred_form(int m, int n, int k, bool nonneg) {
     const int d = m > n + k + 1 ? m : n + k + 1;
     for (int c = 0; c < 4; ++c)
-        if (d <= (32 << c)) return {c, 32 << c, (size_t)(9 << 10) << c};
-    if (d <= 1024) return nonneg && m >= 32 && n >= 32 ? DeferredForm{4, 256, 74 << 10} : DeferredForm{5, 512, 100 << 10};
-    return {6, kMaxThreads, kMaxSmemPerBlock - 1024};
+        if (d <= (32 << c)) return deferred_class(c);
+    if (d <= 1024) return deferred_class(nonneg && m >= 32 && n >= 32 ? 4 : 5);
+    return deferred_class(6);
 }
 
 namespace {

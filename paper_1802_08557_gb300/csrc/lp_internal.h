@@ -306,6 +306,8 @@ struct DeferredForm {
     size_t smem;
 };
 constexpr int kDeferredClasses = 7;
+constexpr int kDeferClass4PerSm = 16;  // least class-4 LPs per SM of a batch; fewer go to class 5
+DeferredForm deferred_class(int cls);
 DeferredForm deferred_form(int m, int n, int k, bool nonneg);
 // Whether deferred updates suit an LP better than its tableau in shared memory
 // (always, where that does not fit), and the threads per CTA of the resident
