@@ -14,6 +14,7 @@
 #include <cstdio>
 #include <cstring>
 #include <map>
+#include <set>
 #include <mutex>
 #include <string>
 #include <thread>
@@ -228,6 +229,25 @@ int32_t host_plan_info(const double* A, const double* b, int32_t m, int32_t n, l
         if (at < len && A[at] < 0.0) return k | lpb::kPlanSigned;
     }
     return k;
+}
+
+// Deferred updates of LPs that fit in shared memory: `count` LPs that they suit, of
+// `entries` tableau entries in total, in what would otherwise be `groups` launch
+// groups.  Where the GPU is full they save work, but one LP by itself takes longer
+// (its work is spread over fewer threads, and from the first flush on none of it is
+// saved); and one queue per size class saves the launches and tails of many small
+// groups.  Deferred / shared memory, ms:
+//  - FP64, one size, packing LPs of A in [1, 10]: 60 x 60 600 LPs 0.16 / 0.14, 2400 0.21 /
+//    0.27; 100 x 100 200 0.33 / 0.20, 800 0.52 / 0.42, 1200 0.44 / 0.59; 150 x 150 50 0.61 /
+//    0.37, 200 0.64 / 0.48, 600 0.72 / 0.99; signed 125 x 125 LPs 50 5.6 / 2.9, 200 6.3 / 4.3,
+//    600 8.1 / 8.7: some 56,000 entries per SM are the line;
+//  - mixed precision, the same: 120 x 120 250 LPs 0.31 / 0.19, 1000 0.38 / 0.37, 2500 0.67 /
+//    0.76; 200 x 200 100 0.34 / 0.25, 250 0.42 / 0.42, 1000 1.5 / 1.9; 300 x 300 (beyond
+//    shared memory) 100 2.7 / 1.5, 250 1.2 / 1.7: also three LPs per two SMs;
+//  - sizes all over 30 to 170 rows and columns, 100 LPs: FP64 0.36 / 0.59, mixed precision
+//    (100 to 220) 0.36 / 1.0; four sizes, 100 LPs 0.38 / 0.24 and 0.32 / 0.30: eight groups.
+bool enough_to_defer(int64_t count, int64_t entries, size_t groups, int sms) {
+    return groups >= 8 || (entries >= (int64_t)56000 * sms && 2 * count >= 3 * (int64_t)sms);
 }
 
 int mixed_threads(int m, int n, int k, int requested) {
@@ -738,6 +758,51 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
     h->uniform_n = hn[0];
     for (int32_t k = 1; k < num_lps; ++k)
         if (hm[k] != hm[0] || hn[k] != hn[0]) h->uniform_m = h->uniform_n = -1;
+    // launch group of an LP in shared memory: threads and rounded footprint.
+    // FP64: 4 KiB steps, coarser above 24 KiB when sizes differ (20,000 uneven LPs
+    // 2.98 -> 2.90 ms, 2000 of them 0.86 -> 0.78 ms)
+    auto resident_group = [&](int32_t k) {
+        const size_t need = lpb::resident_smem_bytes(hm[k], hn[k], hk[k]);
+        const size_t step = h->uniform_m > 0 || need <= 24 * 1024 ? 4096 : (need <= 48 * 1024 ? 8192 : 16384);
+        return std::make_pair(pick_threads(hm[k], hn[k], hk[k], o.block_threads),
+                              std::min(lpb::kMaxSmemPerBlock, (need + step - 1) / step * step));
+    };
+    // Mixed precision: 1 KiB for the one-warp form (it sets how many LPs share an
+    // SM), 8 KiB otherwise: fewer, larger launches (uneven workload: 1 KiB 280 groups
+    // 17.3 ms, 4 KiB 123 groups 11.6 ms, 8 KiB 97 groups 11.2 ms, 16 KiB 84 groups
+    // 11.4 ms).  One-warp LPs of uneven sizes to 4 KiB: 2000 uneven LPs 2.0 -> 1.35 ms,
+    // 20,000 6.3 -> 5.9.  Beyond shared memory {0, 0}.
+    auto mixed_group = [&](int32_t k) {
+        const size_t need = lpb::mixed_smem_bytes(hm[k], hn[k], hk[k]);
+        if (need > queue_smem_cap) return std::make_pair(0, size_t(0));
+        const int threads = mixed_threads(hm[k], hn[k], hk[k], o.block_threads);
+        const size_t gran = threads == 32 ? (h->uniform_m < 0 ? 4096 : 1024) : 8192;
+        return std::make_pair(threads, std::min(queue_smem_cap, (need + gran - 1) / gran * gran));
+    };
+    // LPs that deferred updates suit (a requested thread count keeps those that
+    // fit in shared memory there), and whether they are enough
+    const bool mixed = o.precision == LP_PREC_FP32_REFINE;
+    std::vector<uint8_t> suits(num_lps, 0);
+    bool defer_suited = false;
+    if (o.schedule == LPB_SCHED_AUTO || (o.schedule == LPB_SCHED_CLUSTER && !mixed)) {
+        std::set<std::pair<int, size_t>> groups;
+        int64_t count = 0, entries = 0;
+        for (int32_t k = 0; k < num_lps; ++k) {
+            if (mixed ? !lpb::mixed_defer_updates(hm[k], hn[k], hk[k], nonneg[k])
+                      : !lpb::defer_updates(hm[k], hn[k], hk[k], nonneg[k]) ||
+                            lpb::resident_smem_bytes(hm[k], hn[k], hk[k]) > lpb::kMaxSmemPerBlock)
+                continue;  // (FP64 beyond shared memory: deferred in any case)
+            const auto g = mixed ? mixed_group(k) : resident_group(k);
+            if (o.block_threads > 0 && g.first > 0) continue;
+            suits[k] = 1;
+            groups.insert(g);
+            ++count;
+            entries += (int64_t)(hm[k] + 1) * (hn[k] + hk[k] + 1);
+        }
+        defer_suited = enough_to_defer(count, entries, groups.size(), sms);
+        // mixed precision, few LPs a group: launches of a handful of LPs otherwise
+        if (mixed && groups.size() >= 2 && count < 4 * (int64_t)groups.size()) defer_suited = true;
+    }
     for (int32_t k = 0; k < num_lps; ++k) {
         const size_t need = lpb::resident_smem_bytes(hm[k], hn[k], hk[k]);
         h->num_phase1 += hk[k] > 0;
@@ -788,22 +853,12 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
                 }
                 continue;
             }
-            // (a requested thread count keeps the LPs that fit in shared memory there)
-            if (o.schedule == LPB_SCHED_AUTO && (o.block_threads <= 0 || mneed > queue_smem_cap) &&
-                lpb::mixed_defer_updates(hm[k], hn[k], hk[k], nonneg[k], h->uniform_m < 0)) {
+            if (defer_suited && suits[k]) {
                 mdeferred[lpb::mixed_deferred_form(hm[k], hn[k]).cls].push_back(k);
                 continue;
             }
             if (o.schedule != LPB_SCHED_STREAMED && mneed <= queue_smem_cap) {
-                const int threads = mixed_threads(hm[k], hn[k], hk[k], o.block_threads);
-                // shared memory rounded to 1 KiB for the one-warp form (it sets
-                // how many LPs share an SM), to 8 KiB otherwise: fewer, larger
-                // launches (uneven workload: 1 KiB 280 groups 17.3 ms, 4 KiB
-                // 123 groups 11.6 ms, 8 KiB 97 groups 11.2 ms, 16 KiB 84 groups
-                // 11.4 ms).  One-warp LPs of uneven sizes to 4 KiB: 2000 uneven
-                // LPs 2.0 -> 1.35 ms, 20,000 6.3 -> 5.9
-                const size_t gran = threads == 32 ? (h->uniform_m < 0 ? 4096 : 1024) : 8192;
-                mixed_buckets[{threads, std::min(queue_smem_cap, (mneed + gran - 1) / gran * gran)}].push_back(k);
+                mixed_buckets[mixed_group(k)].push_back(k);
             } else {
                 mstream.push_back(k);
                 h->mslot_bytes = std::max(h->mslot_bytes, (lpb::mixed_layout(hm[k], hn[k], hk[k]).total + 255) &
@@ -838,18 +893,13 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
                 continue;
             }
         }
-        if (o.schedule == LPB_SCHED_STREAMED || need > lpb::kMaxSmemPerBlock ||
-            (o.block_threads <= 0 && lpb::defer_updates(hm[k], hn[k], hk[k], nonneg[k]))) {
+        if (o.schedule == LPB_SCHED_STREAMED || need > lpb::kMaxSmemPerBlock || (defer_suited && suits[k])) {
             defer(k);
             continue;
         }
-        // one launch per footprint step: 4 KiB, coarser above 24 KiB when sizes
-        // differ (20,000 uneven LPs 2.98 -> 2.90 ms, 2000 of them 0.86 -> 0.78 ms)
-        const size_t step = h->uniform_m > 0 || need <= 24 * 1024 ? 4096 : (need <= 48 * 1024 ? 8192 : 16384);
-        const size_t smem = std::min(lpb::kMaxSmemPerBlock, (need + step - 1) / step * step);
-        const int threads = pick_threads(hm[k], hn[k], hk[k], o.block_threads);
-        buckets[{threads, smem}].push_back(k);
-        h->max_smem = std::max(h->max_smem, smem);
+        const auto group = resident_group(k);
+        buckets[group].push_back(k);
+        h->max_smem = std::max(h->max_smem, group.second);
     }
     // Longest work first within every list (LPT): the tail of a launch is
     // made of small LPs.  Work estimate: (m+1)(n+k+1) per pivot, O(m+n) pivots.
@@ -1002,7 +1052,6 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
         if ((err = alloc(h, &h->d_resident, (size_t)num_lps, s)) ||
             (err = cudaMemcpyAsync(h->d_resident, single_resident.data(), (size_t)num_lps, cudaMemcpyHostToDevice, s)))
             return bail_cuda(err, "plan upload");
-        const bool mixed = o.precision == LP_PREC_FP32_REFINE;
         // (each LP's footprint above includes the reduction scratch its area follows)
         h->single_smem = std::max(h->single_smem, lpb::SmallLayout::total);
         // FP64 LPs with deferred updates keep their first pending pivots in the CTA's shared memory

@@ -452,9 +452,8 @@ struct MixedDeferredForm {
 };
 constexpr int kMixedDeferredClasses = 3;
 MixedDeferredForm mixed_deferred_form(int m, int n);
-// Whether an LP gets deferred updates by default (nonneg as for defer_updates;
-// uneven: the batch's LPs differ in size).
-bool mixed_defer_updates(int m, int n, int k, bool nonneg, bool uneven);
+// Whether deferred updates suit an LP (nonneg as for defer_updates).
+bool mixed_defer_updates(int m, int n, int k, bool nonneg);
 int mixed_deferred_ctas_per_sm(const MixedDeferredForm& f);
 cudaError_t launch_mixed_deferred(const DeviceBatch& B, const Tolerances& tol, const MixedParams& mp,
                                   const int32_t* order, int32_t count, const MixedDeferredForm& f, int slots,

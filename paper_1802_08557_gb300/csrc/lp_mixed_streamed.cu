@@ -168,14 +168,11 @@ MixedDeferredForm mixed_deferred_form(int m, int n) {
     return {2, 256, 76 << 10};
 }
 
-// In a batch of uneven sizes, packing LPs of more than 12,000 entries: one queue
-// per class instead of a launch per footprint step, no FP32 copy of A, few
-// pivots (20,000 LPs of 10-500 rows and columns 10.4 -> 4.9 ms, 2000 of them 2.1 ->
-// 1.3; from 2000 entries on 5.5, from 30,000 5.2).  In a batch of one size the
-// whole-tableau forms keep them: an FP32 update is cheap, and positive LPs of
-// 200 x 200 (28 pivots) take 0.90 against 1.22 ms, 300 x 300 2.4 against 3.0.
-bool mixed_defer_updates(int m, int n, int k, bool nonneg, bool uneven) {
-    return uneven && nonneg && (int64_t)(m + 1) * (n + k + 1) > kMixedDeferEntries && m >= 32 && n >= 32 &&
+// Packing LPs of more than 12,000 entries: no FP32 copy of A, few pivots.  20,000
+// uneven ones of 10-500 rows and columns 10.4 -> 4.9 ms; from 2000 entries on 5.5, from
+// 30,000 5.2.
+bool mixed_defer_updates(int m, int n, int k, bool nonneg) {
+    return nonneg && (int64_t)(m + 1) * (n + k + 1) > kMixedDeferEntries && m >= 32 && n >= 32 &&
            SmallLayout::total + mixed_deferred_layout(m, n, k).hist <= mixed_deferred_form(m, n).smem;
 }
 
