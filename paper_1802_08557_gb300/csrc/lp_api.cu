@@ -788,6 +788,8 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
         std::set<std::pair<int, size_t>> groups;
         int64_t count = 0, entries = 0;
         for (int32_t k = 0; k < num_lps; ++k) {
+            const int64_t e = (int64_t)(hm[k] + 1) * (hn[k] + hk[k] + 1);
+            if (e <= lpb::kDeferNonneg) continue;
             if (mixed ? !lpb::mixed_defer_updates(hm[k], hn[k], hk[k], nonneg[k])
                       : !lpb::defer_updates(hm[k], hn[k], hk[k], nonneg[k]) ||
                             lpb::resident_smem_bytes(hm[k], hn[k], hk[k]) > lpb::kMaxSmemPerBlock)
@@ -797,7 +799,7 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
             suits[k] = 1;
             groups.insert(g);
             ++count;
-            entries += (int64_t)(hm[k] + 1) * (hn[k] + hk[k] + 1);
+            entries += e;
         }
         defer_suited = enough_to_defer(count, entries, groups.size(), sms);
         // mixed precision, few LPs a group: launches of a handful of LPs otherwise

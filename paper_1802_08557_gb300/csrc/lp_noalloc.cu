@@ -124,11 +124,13 @@ extern "C" lpb_err lp_solve_uniform_noalloc(int32_t num_lps, int32_t m, int32_t 
 
     // Room: the counter, the descriptors, and, for LPs with deferred updates,
     // at least one workspace slot; sized for the widest phase-I tableau (every
-    // row with b_i < 0: the right-hand sides are on the device).  The form is
-    // chosen by the rule of lp_batch_create; measured, 1500 LPs of 50 x 50:
-    // 0.94 ms with the tableau in shared memory, 3.0 ms with deferred updates,
-    // 3.5 ms with the whole tableau updated in the slot.
-    const bool deferred = defer_updates(m, n, m, false);
+    // row with b_i < 0: the right-hand sides are on the device), which also
+    // bounds how many tableaux in shared memory share an SM: so deferred updates
+    // above 14,000 entries of that tableau, whatever its shape.  Measured, 1500 LPs
+    // of 50 x 50: 0.94 ms with the tableau in shared memory, 3.0 ms with deferred
+    // updates, 3.5 ms with the whole tableau updated in the slot.
+    const bool deferred = (int64_t)(m + 1) * ((int64_t)n + m + 1) > kDeferEntries ||
+                          resident_smem_bytes(m, n, m) > kMaxSmemPerBlock - 1024;
     const size_t slot_bytes = deferred_slot(m, n, m).total;
     const DeferredForm form = deferred_form(m, n, m, false);
     const size_t desc_bytes = descriptor_bytes(num_lps);
