@@ -223,6 +223,7 @@ __device__ __forceinline__ void deferred_solve(G& g, const DeviceBatch& B, const
     double* rg = reinterpret_cast<double*>(slot + S.hist) + (size_t)S.first * m - (ptrdiff_t)ks * W;
     int cap = S.first;  // pending pivots before the next flush
 
+    constexpr int kRetired = INT_MAX;  // col_last of a retired column
     bool from_a = true;  // the source of an element: A, or T after a flush
     auto source = [&](int i, int j, bool neg_i) -> double {  // j >= 1
         if (!from_a) return T[(size_t)i * LD + j];
@@ -282,23 +283,30 @@ __device__ __forceinline__ void deferred_solve(G& g, const DeviceBatch& B, const
         vcol = v;
         c_at(t)[tid] = v;
     };
-    // own element of row i (live columns only)
-    auto element = [&](int i, int sr, bool neg_i) -> double {
+    // element (i, j) of a live column
+    auto element = [&](int i, int j, int sr, int sc, bool neg_i) -> double {
         int s0;
-        double v = begin(i, tid, sr, clast, neg_i, s0);
-        v = chain(v, s0, sr + 1, min(t, ks), cs + i, m, rs + tid, W);
-        if (t > ks) v = chain(v, s0, max(sr + 1, ks), t, cg + i, m, rg + tid, W);
+        double v = begin(i, j, sr, sc, neg_i, s0);
+        v = chain(v, s0, sr + 1, min(t, ks), cs + i, m, rs + j, W);
+        if (t > ks) v = chain(v, s0, max(sr + 1, ks), t, cg + i, m, rg + j, W);
         return v;
     };
-    // the body after every pending pivot, into T (the source from then on)
+    // the body after every pending pivot, into T (the source from then on).  As
+    // many threads per column as the group has, an element always by the same
+    // thread: with one per column, LPs of few columns left most of the group idle.
+    // 1000 signed LPs of 225 x 64 8.1 -> 4.9 ms, of 200 x 40 3.0 -> 1.5; without
+    // allocation (a form for every row negated) 1500 of 200 x 40 8.6 -> 3.2, of 100 x
+    // 100 10.8 -> 9.0.
     auto flush = [&]() {
-        if (cvar < nm)
-            for (int i = 0; i < m; ++i)
-                T[(size_t)i * LD + tid] = element(i, row_last[i], (negbits[i >> 5] >> (i & 31)) & 1u);
+        const int parts = g.nt / (W - 1), part = tid / (W - 1), j = 1 + tid - part * (W - 1);
+        const int sc = part < parts ? col_last[j] : kRetired;
+        if (sc != kRetired)
+            for (int i = part; i < m; i += parts)
+                T[(size_t)i * LD + j] = element(i, j, row_last[i], sc, (negbits[i >> 5] >> (i & 31)) & 1u);
         g.sync();
         rlast = clast = -1;
         if (has_row) row_last[tid] = -1;
-        if (has_col) col_last[tid] = -1;
+        if (has_col && col_last[tid] != kRetired) col_last[tid] = -1;
         from_a = false;
         t = 0;
         cap = S.later;
@@ -318,7 +326,8 @@ __device__ __forceinline__ void deferred_solve(G& g, const DeviceBatch& B, const
     auto relabel = [&](int l, int e, int entering, int left) {
         if (tid == e) {
             cvar = left;  // an artificial (>= nm) retires with its column
-            clast = col_last[e] = t;
+            clast = t;
+            col_last[e] = left < nm ? t : kRetired;
         }
         if (tid == l) {
             rvar = entering;
@@ -380,7 +389,7 @@ __device__ __forceinline__ void deferred_solve(G& g, const DeviceBatch& B, const
                 double u = rhs;
                 unsigned sel = none;
                 if (cvar < nm) {
-                    u = element(i, boxi[1], boxi[2] != 0);
+                    u = element(i, tid, boxi[1], clast, boxi[2] != 0);
                     if (abskey(u) > key_eps_piv) sel = ((unsigned)cvar << 16) | (unsigned)tid;
                 }
                 sel = g.min_u32(sel);
@@ -463,7 +472,7 @@ __device__ __forceinline__ void deferred_solve(G& g, const DeviceBatch& B, const
         // ---- Step 3: pivot ---------------------------------------------------
         const int left = boxi[0];
         double u = box[2];
-        if (live) u = element(l, boxi[1], boxi[2] != 0);
+        if (live) u = element(l, tid, boxi[1], clast, boxi[2] != 0);
         scale(u, e, pe, box[0], box[1], one);
         relabel(l, e, (int)(esel >> 16), left);
         rhs_row = l;
@@ -645,7 +654,7 @@ __device__ __forceinline__ void deferred_solve_large(DeferBlock& g, const Device
     auto flush = [&]() {
         for (int i = warp; i < m; i += nw) {
             double* Ti = T + (size_t)i * LD;
-            row(i, row_last[i], lane, 32, [&](int j, double v) { Ti[j] = v; });
+            row(i, row_last[i], 1 + lane, 32, [&](int j, double v) { Ti[j] = v; });
         }
         g.sync();
         for (int i = tid; i < m; i += nt) row_last[i] = -1;

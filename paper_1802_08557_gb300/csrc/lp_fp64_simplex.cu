@@ -620,12 +620,12 @@ cudaError_t launch_fp64_resident_queue(const DeviceBatch& B, const Tolerances& t
 //    entries, which only one CTA per SM has room for, 8 x 1600 1.65 / 1.22, 12 x 1200
 //    1.42 / 1.15, 20 x 1100 1.67 / 1.44;
 //  - others, above 14,000 entries: rows longer than columns by half, 16 x 900 0.51 /
-//    0.67, 24 x 1000 1.12 / 1.32, 64 x 225 2.3 / 2.5, 90 x 250 4.9 / 5.4, 120 x 180 9.7 /
-//    9.9; a thread per row and column within 128, 125 x 125 12.9 / 13.8; fewer than 12
-//    columns (no more pivots than are kept pending), 1450 x 10 0.84 / 1.02, 2000 x 6 0.66 /
-//    0.86; but 130 x 130 17.0 / 15.5, 110 x 160 8.7 / 8.0, 250 x 90 17.7 / 14.1, 225 x 64
-//    8.1 / 5.6, 700 x 32 4.8 / 3.2, 1100 x 12 1.14 / 0.98, 16 x 1400 0.95 / 0.95 (with phase
-//    I 1.77 / 1.61).
+//    0.66, 24 x 1000 1.13 / 1.32, 64 x 225 2.3 / 2.5, 90 x 250 4.9 / 5.4, 120 x 180 9.4 /
+//    9.9; a thread per row and column within 128, 125 x 125 13.1 / 13.8; fewer than 12
+//    columns (no more pivots than are kept pending), 1450 x 10 0.84 / 1.01, 2000 x 6 0.68 /
+//    0.85; but 130 x 130 17.0 / 15.5, with phase I 120 x 118 21.2 / 19.6, 300 x 48 4.5 / 3.8,
+//    500 x 48 6.9 / 5.7, 1100 x 12 1.14 / 0.98, 16 x 1400 0.95 / 0.95 (with phase I 1.77 /
+//    1.61); 225 x 64 4.9 / 5.6 and 160 x 90 8.6 / 9.1 are on the other side of the line.
 bool defer_updates(int m, int n, int k, bool nonneg) {
     if (resident_smem_bytes(m, n, k) > kMaxSmemPerBlock) return true;
     const int w = n + k + 1, d = m > w ? m : w;

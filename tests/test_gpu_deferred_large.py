@@ -108,3 +108,19 @@ def test_class_edges(edge):
     got = gpu_solve(batch, opts=lpb.lpb_default_opts(schedule=lpb.LPB_SCHED_STREAMED))
     assert got["plan"]["num_streamed"] == len(lps)
     assert compare(batch, got, oracle_solve(batch)) == (len(lps), len(lps))
+
+
+# several threads per column in a flush: columns that divide the group's threads and that do not, rows left
+# over, retired columns (phase I)
+@pytest.mark.parametrize("phase1", [False, True])
+def test_flushes_of_few_columns(phase1):
+    sizes = [(225, 64), (250, 40), (128, 25), (120, 20), (63, 21), (250, 85), (200, 50), (97, 32)]
+    lps = [_dense(m, n, 31 * m + n, signed=True, phase1=phase1) for m, n in sizes]
+    batch = W.pack("tall", lps)
+    ref = oracle_solve(batch)
+    pending = [max(16, m * (n + 1) // (2 * (m + n + 1))) for m, n in sizes]
+    if not phase1:
+        assert all(it > p for it, p in zip(ref["iters"], pending)), (list(ref["iters"]), pending)
+    got = gpu_solve(batch, opts=lpb.lpb_default_opts(schedule=lpb.LPB_SCHED_STREAMED))
+    assert got["plan"]["num_streamed"] == len(lps)
+    assert compare(batch, got, ref) == (len(lps), len(lps))
