@@ -217,8 +217,11 @@ lpb::SignLook sign_look(const lp_batch_opts& o) {
 
 // What launch_plan_info finds on the device, for an LP in host memory: its rows
 // with b_i < 0, plus kPlanSigned unless a sample of A has no negative entry.  The
-// sample costs the host some 0.5 us, so it is taken only of LPs whose copy takes
-// longer; a smaller packing LP from host memory keeps its tableau in shared memory.
+// host's time is on the path of a call from host memory, so the sample is taken
+// only where the kind of updates depends on it, and FP64 reads a quarter of the
+// device's places (4000 uneven LPs, one call: all places of every LP above 14,000
+// entries 2.5 ms, this 2.2).  Smaller packing LPs from host memory keep their
+// tableaux in shared memory.
 int32_t host_plan_info(const double* A, const double* b, int32_t m, int32_t n, lpb::SignLook look) {
     const int32_t k = count_negative(b, m);
     const int64_t least = look == lpb::kLookLeading ? lpb::kMixedDeferEntries : lpb::kDeferEntries;
@@ -308,6 +311,7 @@ struct lp_batch {
     int32_t num_mixed = 0;
     lpb::MixedParams mp{};
     int32_t* fb_queue = nullptr;
+    bool mixed_small_code = true;  // of the one-warp kernel
     int32_t* fb_len = nullptr;
     int32_t* fb_counter = nullptr;
     int32_t* diag = nullptr;  // 8 int32: internal-consistency failures of the last solve
@@ -440,7 +444,7 @@ cudaError_t launch_group(lp_batch* h, int kind, const Group& g, cudaStream_t ls)
             return lpb::launch_mixed_queue(h->d, h->tol, h->mp, order, h->group_len + g.gi, h->group_counter + g.gi,
                                            g.ctas, g.threads, g.smem, fallback_queues(h), h->diag, ls);
         return lpb::launch_mixed(h->d, h->tol, h->mp, order, g.count, g.threads, g.threads == 32 ? g.smem_warp : g.smem,
-                                 fallback_queues(h), h->diag, ls);
+                                 h->mixed_small_code, fallback_queues(h), h->diag, ls);
     }
     if (g.persistent)
         return lpb::launch_fp64_resident_queue(h->d, h->tol, order, h->group_len + g.gi, g.count, h->num_lps,
@@ -932,6 +936,7 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
         g.offset = (int64_t)order.size();
         g.count = (int32_t)kv.second.size();
         g.threads = kv.first.first;
+    int64_t small_lps = 0, large_lps = 0;  // of the one-warp form
         g.smem = kv.first.second;
         // the one-warp form at its exact size (128-byte units): 13.5 KB, not
         // 14 KB, is what lets 16 CTAs of 50 x 50 LPs share an SM
@@ -945,7 +950,9 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
     for (auto& kv : cluster_buckets) {
         const int C = kv.first;
         lpt(kv.second);
+        if (g.threads == 32) (g.smem_warp <= lpb::kSmallWarpBytes ? small_lps : large_lps) += g.count;
         size_t smem = 0;
+    h->mixed_small_code = lpb::mixed_small_code(small_lps, large_lps);
         for (int32_t k : kv.second) smem = std::max(smem, lpb::cluster_smem_bytes(hm[k], hn[k], hk[k], C));
         smem = (smem + 1023) / 1024 * 1024;
         int active = 0;

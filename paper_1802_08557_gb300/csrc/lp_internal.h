@@ -282,12 +282,17 @@ struct FallbackQueues {
 };
 
 cudaError_t mixed_kernel_prepare();
+// Which of the one-warp kernel's two codes a batch takes (small_code of
+// launch_mixed), from its numbers of one-warp LPs of up to and above
+// kSmallWarpBytes.
+constexpr size_t kSmallWarpBytes = 14 * 1024;
+bool mixed_small_code(int64_t small_lps, int64_t large_lps);
 // One CTA per LP of order[0..count) (one warp per LP when threads == 32):
 // FP32 simplex in shared memory, FP64 certificate; uncertified LPs to fq.
 // diag: 3 int32 (count, first code, first LP) of internal-consistency
 // failures (see record_internal_error); may be null.
 cudaError_t launch_mixed(const DeviceBatch& B, const Tolerances& tol, const MixedParams& mp,
-                         const int32_t* order, int32_t count, int threads, size_t smem,
+                         const int32_t* order, int32_t count, int threads, size_t smem, bool small_code,
                          const FallbackQueues& fq, int32_t* diag, cudaStream_t stream);
 
 // Launchers (lp_fp64_simplex.cu).

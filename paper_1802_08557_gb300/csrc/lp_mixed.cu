@@ -54,8 +54,7 @@ mixed_warp_kernel(const DeviceBatch B, const Tolerances tol, const MixedParams m
     mixed_solve_lp<4>(g, B, tol, mp, order[blockIdx.x], smem, fq, diag);
 }
 
-// The same with half the unrolling, where 16 or more such CTAs share an SM and
-// stall on instructions (40% of the time for 32 of them).
+// The same with half the unrolling (mixed_small_code).
 __global__ void __launch_bounds__(32, 32)
 mixed_warp_small_kernel(const DeviceBatch B, const Tolerances tol, const MixedParams mp,
                         const int32_t* __restrict__ order, const FallbackQueues fq, int32_t* __restrict__ diag)
@@ -64,14 +63,6 @@ mixed_warp_small_kernel(const DeviceBatch B, const Tolerances tol, const MixedPa
     WarpGroup g;
     mixed_solve_lp<2>(g, B, tol, mp, order[blockIdx.x], smem, fq, diag);
 }
-
-// The line between the two.  Unrolling of 2 against 4, signed / packing /
-// phase-I LPs, time relative to 4: 20 x 20 (3 KB) 0.91 / 0.94 / 0.91, 40 x 40 (10 KB)
-// 0.92 / 0.95 / 0.96, 30 x 80 (13 KB) 0.97 / 0.95 / 0.99, 50 x 50 (13.5 KB) 1.01 / 0.97,
-// with phase I (14.6 KB) 1.04; 60 x 60 (19 KB) 1.03 / 1.01 / 1.06, 70 x 70 (24 KB) 1.11 /
-// 1.02 / 1.13, 88 x 88 1.14 / 1.04; and in CTAs of 128 and 256 threads 100 x 100 1.06 /
-// 1.04 / 1.06, 170 x 170 1.18 / 1.18 / 1.06.
-constexpr size_t kSmallWarpBytes = 14 * 1024;
 
 }  // namespace
 
@@ -89,11 +80,23 @@ cudaError_t mixed_kernel_prepare() {
                                 (int)(kMaxSmemPerBlock - 1024));
 }
 
+// Where 16 or more one-warp CTAs share an SM, in different phases of the code,
+// they stall on instructions (40% of the time for 32 of them), and half the
+// unrolling is faster: time relative to the full one, signed / packing / phase-I
+// LPs, 20 x 20 (3 KB) 0.91 / 0.94 / 0.91, 40 x 40 (10 KB) 0.92 / 0.95 / 0.96, 30 x 80 (13
+// KB) 0.97 / 0.95 / 0.99, 50 x 50 (13.5 KB) 1.01 / 0.97, with phase I (to 18 KB) 1.04; 60 x
+// 60 (19 KB) 1.03 / 1.01 / 1.06, 70 x 70 (24 KB) 1.11 / 1.02 / 1.13, 88 x 88 1.14 / 1.04;
+// and in CTAs of 128 and 256 threads 100 x 100 1.06 / 1.04 / 1.06, 170 x 170 1.18 / 1.18 /
+// 1.06.  One choice for all groups of a batch, by the majority of its one-warp LPs:
+// both codes at a time share the instruction cache (100,000 LPs of 50 x 50, a fifth
+// with phase I, from host arrays in 8 ranges: 17.2 ms, 16.5 with either alone).
+bool mixed_small_code(int64_t small_lps, int64_t large_lps) { return small_lps >= large_lps; }
+
 cudaError_t launch_mixed(const DeviceBatch& B, const Tolerances& tol, const MixedParams& mp,
-                         const int32_t* order, int32_t count, int threads, size_t smem,
+                         const int32_t* order, int32_t count, int threads, size_t smem, bool small_code,
                          const FallbackQueues& fq, int32_t* diag, cudaStream_t stream) {
     if (count <= 0) return cudaSuccess;
-    if (threads == 32 && smem <= kSmallWarpBytes)
+    if (threads == 32 && small_code)
         mixed_warp_small_kernel<<<count, 32, smem, stream>>>(B, tol, mp, order, fq, diag);
     else if (threads == 32)
         mixed_warp_kernel<<<count, 32, smem, stream>>>(B, tol, mp, order, fq, diag);

@@ -1,6 +1,6 @@
-"""One-warp mixed-precision groups on both sides of the shared-memory line at
-which the kernel's unrolling changes (14 KB): the same outputs, bit for bit, as
-the form with the tableau in a global workspace."""
+"""The one-warp mixed-precision kernel's two codes, chosen by the majority of a
+batch's LPs on one side of a shared-memory line (14 KB): the same outputs, bit
+for bit, as the form with the tableau in a global workspace."""
 import numpy as np
 import pytest
 
@@ -22,6 +22,20 @@ def _built():
 @pytest.mark.parametrize("m,n", [(1, 1), (3, 2), (50, 50), (51, 51), (30, 86), (86, 30), (62, 40), (89, 90)])
 def test_both_unrollings_match_the_workspace_form(m, n):
     batch = W.mixed_sign_dense(60, m, n, start=17 * m + n, p_phase1=0.4)
+    got = gpu_solve(batch, opts=lpb.lpb_default_opts(precision=lpb.LP_PREC_FP32_REFINE))
+    want = gpu_solve(batch, opts=lpb.lpb_default_opts(precision=lpb.LP_PREC_FP32_REFINE,
+                                                      schedule=lpb.LPB_SCHED_STREAMED))
+    for key in ("status", "iters", "obj", "x", "y"):
+        np.testing.assert_array_equal(got[key], want[key], err_msg=key)
+
+
+@pytest.mark.parametrize("most", ["small", "large"])
+def test_every_size_in_either_code(most):
+    """The largest one-warp LPs in a batch of small ones and the other way round."""
+    counts = (60, 9) if most == "small" else (9, 60)
+    lps = [W.mixed_sign_dense(counts[0], 20, 30, start=3).lp(k) for k in range(counts[0])]
+    lps += [W.mixed_sign_dense(counts[1], 80, 86, start=4, p_phase1=0.0).lp(k) for k in range(counts[1])]
+    batch = W.pack(most, lps)
     got = gpu_solve(batch, opts=lpb.lpb_default_opts(precision=lpb.LP_PREC_FP32_REFINE))
     want = gpu_solve(batch, opts=lpb.lpb_default_opts(precision=lpb.LP_PREC_FP32_REFINE,
                                                       schedule=lpb.LPB_SCHED_STREAMED))
