@@ -224,10 +224,13 @@ lpb::SignLook sign_look(const lp_batch_opts& o) {
 // tableaux in shared memory.
 int32_t host_plan_info(const double* A, const double* b, int32_t m, int32_t n, lpb::SignLook look) {
     const int32_t k = count_negative(b, m);
-    const int64_t least = look == lpb::kLookLeading ? lpb::kMixedDeferEntries : lpb::kDeferEntries;
-    if (look == lpb::kLookNot || (int64_t)(m + 1) * (n + k + 1) <= least) return k | lpb::kPlanSigned;
+    const int64_t e = (int64_t)(m + 1) * (n + k + 1);
+    if (look == lpb::kLookNot || e <= (look == lpb::kLookLeading ? lpb::kMixedDeferEntries : lpb::kDeferEntries) ||
+        (look == lpb::kLookSpread && lpb::defer_updates(m, n, k, false)))
+        return k | lpb::kPlanSigned;
     const int64_t len = (int64_t)m * n;
     for (int i = 0; i < lpb::sign_samples(look); ++i) {
+        if (look == lpb::kLookSpread && (i / 4) % 4 != 3) continue;  // (the last place among them)
         const int64_t at = lpb::sign_sample_at(look, len, i);
         if (at < len && A[at] < 0.0) return k | lpb::kPlanSigned;
     }
@@ -308,10 +311,10 @@ struct lp_batch {
     int32_t num_streamed = 0;
     // mixed precision: groups of the FP32 + certificate kernel, fallback queue
     std::vector<Group> mixed_groups;
+    bool mixed_small_code = true;  // of the one-warp kernel
     int32_t num_mixed = 0;
     lpb::MixedParams mp{};
     int32_t* fb_queue = nullptr;
-    bool mixed_small_code = true;  // of the one-warp kernel
     int32_t* fb_len = nullptr;
     int32_t* fb_counter = nullptr;
     int32_t* diag = nullptr;  // 8 int32: internal-consistency failures of the last solve
@@ -739,8 +742,10 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
             return bail_cuda(err, "input check");
         if (bad) return bail(LPB_EINVAL, std::to_string(bad) + " non-finite entries in A, b or c");
     }
+    bool any_nonneg = false;
     for (int32_t k = 0; k < num_lps; ++k) {
         nonneg[k] = (hk[k] & lpb::kPlanSameA) ? nonneg[k - 1] : !(hk[k] & lpb::kPlanSigned);
+        any_nonneg |= nonneg[k] != 0;
         hk[k] &= ~(lpb::kPlanSigned | lpb::kPlanSameA);
     }
 
@@ -765,8 +770,7 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
     // launch group of an LP in shared memory: threads and rounded footprint.
     // FP64: 4 KiB steps, coarser above 24 KiB when sizes differ (20,000 uneven LPs
     // 2.98 -> 2.90 ms, 2000 of them 0.86 -> 0.78 ms)
-    auto resident_group = [&](int32_t k) {
-        const size_t need = lpb::resident_smem_bytes(hm[k], hn[k], hk[k]);
+    auto resident_group = [&](int32_t k, size_t need) {
         const size_t step = h->uniform_m > 0 || need <= 24 * 1024 ? 4096 : (need <= 48 * 1024 ? 8192 : 16384);
         return std::make_pair(pick_threads(hm[k], hn[k], hk[k], o.block_threads),
                               std::min(lpb::kMaxSmemPerBlock, (need + step - 1) / step * step));
@@ -776,8 +780,7 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
     // 17.3 ms, 4 KiB 123 groups 11.6 ms, 8 KiB 97 groups 11.2 ms, 16 KiB 84 groups
     // 11.4 ms).  One-warp LPs of uneven sizes to 4 KiB: 2000 uneven LPs 2.0 -> 1.35 ms,
     // 20,000 6.3 -> 5.9.  Beyond shared memory {0, 0}.
-    auto mixed_group = [&](int32_t k) {
-        const size_t need = lpb::mixed_smem_bytes(hm[k], hn[k], hk[k]);
+    auto mixed_group = [&](int32_t k, size_t need) {
         if (need > queue_smem_cap) return std::make_pair(0, size_t(0));
         const int threads = mixed_threads(hm[k], hn[k], hk[k], o.block_threads);
         const size_t gran = threads == 32 ? (h->uniform_m < 0 ? 4096 : 1024) : 8192;
@@ -788,17 +791,19 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
     const bool mixed = o.precision == LP_PREC_FP32_REFINE;
     std::vector<uint8_t> suits(num_lps, 0);
     bool defer_suited = false;
-    if (o.schedule == LPB_SCHED_AUTO || (o.schedule == LPB_SCHED_CLUSTER && !mixed)) {
+    if (look != lpb::kLookNot && (any_nonneg || !mixed)) {
         std::set<std::pair<int, size_t>> groups;
         int64_t count = 0, entries = 0;
         for (int32_t k = 0; k < num_lps; ++k) {
             const int64_t e = (int64_t)(hm[k] + 1) * (hn[k] + hk[k] + 1);
-            if (e <= lpb::kDeferNonneg) continue;
+            if (e <= (nonneg[k] ? lpb::kDeferNonneg : lpb::kDeferEntries) || (mixed && !nonneg[k])) continue;
             if (mixed ? !lpb::mixed_defer_updates(hm[k], hn[k], hk[k], nonneg[k])
-                      : !lpb::defer_updates(hm[k], hn[k], hk[k], nonneg[k]) ||
-                            lpb::resident_smem_bytes(hm[k], hn[k], hk[k]) > lpb::kMaxSmemPerBlock)
-                continue;  // (FP64 beyond shared memory: deferred in any case)
-            const auto g = mixed ? mixed_group(k) : resident_group(k);
+                      : !lpb::defer_updates(hm[k], hn[k], hk[k], nonneg[k]))
+                continue;
+            const size_t need = mixed ? lpb::mixed_smem_bytes(hm[k], hn[k], hk[k])
+                                      : lpb::resident_smem_bytes(hm[k], hn[k], hk[k]);
+            if (!mixed && need > lpb::kMaxSmemPerBlock) continue;  // deferred in any case
+            const auto g = mixed ? mixed_group(k, need) : resident_group(k, need);
             if (o.block_threads > 0 && g.first > 0) continue;
             suits[k] = 1;
             groups.insert(g);
@@ -864,7 +869,7 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
                 continue;
             }
             if (o.schedule != LPB_SCHED_STREAMED && mneed <= queue_smem_cap) {
-                mixed_buckets[mixed_group(k)].push_back(k);
+                mixed_buckets[mixed_group(k, mneed)].push_back(k);
             } else {
                 mstream.push_back(k);
                 h->mslot_bytes = std::max(h->mslot_bytes, (lpb::mixed_layout(hm[k], hn[k], hk[k]).total + 255) &
@@ -903,7 +908,7 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
             defer(k);
             continue;
         }
-        const auto group = resident_group(k);
+        const auto group = resident_group(k, need);
         buckets[group].push_back(k);
         h->max_smem = std::max(h->max_smem, group.second);
     }
@@ -931,12 +936,12 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
         order.insert(order.end(), kv.second.begin(), kv.second.end());
         h->groups.push_back(g);
     }
+    int64_t small_lps = 0, large_lps = 0;  // of the one-warp form
     for (auto& kv : mixed_buckets) {
         Group g;
         g.offset = (int64_t)order.size();
         g.count = (int32_t)kv.second.size();
         g.threads = kv.first.first;
-    int64_t small_lps = 0, large_lps = 0;  // of the one-warp form
         g.smem = kv.first.second;
         // the one-warp form at its exact size (128-byte units): 13.5 KB, not
         // 14 KB, is what lets 16 CTAs of 50 x 50 LPs share an SM
@@ -945,14 +950,14 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
         order.insert(order.end(), kv.second.begin(), kv.second.end());
         h->mixed_groups.push_back(g);
         h->num_mixed += g.count;
+        if (g.threads == 32) (g.smem_warp <= lpb::kSmallWarpBytes ? small_lps : large_lps) += g.count;
     }
+    h->mixed_small_code = lpb::mixed_small_code(small_lps, large_lps);
     // cluster groups (a cluster shape that cannot be placed gets deferred updates)
     for (auto& kv : cluster_buckets) {
         const int C = kv.first;
         lpt(kv.second);
-        if (g.threads == 32) (g.smem_warp <= lpb::kSmallWarpBytes ? small_lps : large_lps) += g.count;
         size_t smem = 0;
-    h->mixed_small_code = lpb::mixed_small_code(small_lps, large_lps);
         for (int32_t k : kv.second) smem = std::max(smem, lpb::cluster_smem_bytes(hm[k], hn[k], hk[k], C));
         smem = (smem + 1023) / 1024 * 1024;
         int active = 0;
