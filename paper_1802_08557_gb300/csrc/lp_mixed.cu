@@ -44,24 +44,15 @@ mixed_queue_kernel(const DeviceBatch B, const Tolerances tol, const MixedParams 
 }
 
 // One warp per LP (blockDim = 32): for small tableaux, where a whole CTA per
-// LP mostly waits at barriers.
+// LP mostly waits at barriers.  kUnroll 2: the smaller code (mixed_small_code).
+template <int kUnroll>
 __global__ void __launch_bounds__(32, 32)
 mixed_warp_kernel(const DeviceBatch B, const Tolerances tol, const MixedParams mp, const int32_t* __restrict__ order,
                   const FallbackQueues fq, int32_t* __restrict__ diag)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     WarpGroup g;
-    mixed_solve_lp<4>(g, B, tol, mp, order[blockIdx.x], smem, fq, diag);
-}
-
-// The same with half the unrolling (mixed_small_code).
-__global__ void __launch_bounds__(32, 32)
-mixed_warp_small_kernel(const DeviceBatch B, const Tolerances tol, const MixedParams mp,
-                        const int32_t* __restrict__ order, const FallbackQueues fq, int32_t* __restrict__ diag)
-{
-    extern __shared__ __align__(16) unsigned char smem[];
-    WarpGroup g;
-    mixed_solve_lp<2>(g, B, tol, mp, order[blockIdx.x], smem, fq, diag);
+    mixed_solve_lp<kUnroll>(g, B, tol, mp, order[blockIdx.x], smem, fq, diag);
 }
 
 }  // namespace
@@ -73,10 +64,10 @@ cudaError_t mixed_kernel_prepare() {
     err = cudaFuncSetAttribute(mixed_queue_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)(kMaxSmemPerBlock - 1024));
     if (err != cudaSuccess) return err;
-    err = cudaFuncSetAttribute(mixed_warp_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    err = cudaFuncSetAttribute(mixed_warp_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)(kMaxSmemPerBlock - 1024));
     if (err != cudaSuccess) return err;
-    return cudaFuncSetAttribute(mixed_warp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    return cudaFuncSetAttribute(mixed_warp_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)(kMaxSmemPerBlock - 1024));
 }
 
@@ -97,9 +88,9 @@ cudaError_t launch_mixed(const DeviceBatch& B, const Tolerances& tol, const Mixe
                          const FallbackQueues& fq, int32_t* diag, cudaStream_t stream) {
     if (count <= 0) return cudaSuccess;
     if (threads == 32 && small_code)
-        mixed_warp_small_kernel<<<count, 32, smem, stream>>>(B, tol, mp, order, fq, diag);
+        mixed_warp_kernel<2><<<count, 32, smem, stream>>>(B, tol, mp, order, fq, diag);
     else if (threads == 32)
-        mixed_warp_kernel<<<count, 32, smem, stream>>>(B, tol, mp, order, fq, diag);
+        mixed_warp_kernel<4><<<count, 32, smem, stream>>>(B, tol, mp, order, fq, diag);
     else
         mixed_kernel<<<count, threads, smem, stream>>>(B, tol, mp, order, fq, diag);
     return cudaGetLastError();

@@ -40,7 +40,7 @@ namespace {
 // (all loads of a batch issued before its stores) and the unrolling of the
 // certificate's loops.  4 hides more latency; 2 is less code, which counts
 // where the warps of an SM are in different phases of it and share its
-// instruction cache (mixed_warp_small_kernel, lp_mixed.cu, with both sides
+// instruction cache (mixed_small_code, lp_mixed.cu, with both sides
 // measured).  The same operations in the same order either way.
 
 // Thread layout of the pivot update over quads of 4 columns: thread tid takes
