@@ -89,14 +89,21 @@ typedef struct {
     int32_t schedule;    /* LPB_SCHED_AUTO, _STREAMED, _CLUSTER or _SINGLE          */
 } lp_batch_opts;
 
-/* Kernel choice.  AUTO: shared-memory-resident tableau when it fits in one
- * CTA, else a global workspace slot per LP (persistent CTAs, many LPs at
- * once).  With LP_PREC_FP32_REFINE the FP32 tableau is in one CTA's shared
- * memory when it fits, else in a global workspace; the FP64 re-solve of an
- * uncertified LP runs in one CTA when its FP64 tableau fits, else on a
- * thread-block cluster (one LP's latency matters there).
- * STREAMED: global workspace for every LP (FP32_REFINE: the FP32 tableau of
- * every LP).  CLUSTER: as AUTO, but an FP64 tableau above one CTA is split by
+/* Kernel choice.  AUTO: an LP's tableau in one CTA's shared memory, or deferred
+ * updates (a tableau element is formed when a pivot reads it; persistent CTAs,
+ * a global workspace slot each, many LPs at once).  FP64 LPs that do not fit in
+ * shared memory get deferred updates, and so do, in batches with enough of them,
+ * LPs whose number of pivots, size and shape they suit: packing LPs (no negative
+ * entry seen in a sample of A) of more than 2,000 tableau entries, and some of more
+ * than 14,000.  With LP_PREC_FP32_REFINE they are used for packing LPs of more than
+ * 12,000 entries; otherwise the FP32 tableau is in one CTA's shared memory when
+ * it fits, else in a global workspace; the FP64 re-solve of an uncertified LP runs
+ * in one CTA when its FP64 tableau fits, else on a thread-block cluster (one
+ * LP's latency matters there).  Where A is in host memory its sign is looked for
+ * only in LPs of more than 14,000 (FP32_REFINE: 12,000) entries, so smaller
+ * packing LPs from there keep their tableaux in shared memory.
+ * STREAMED: workspace for every LP (FP64: deferred updates; FP32_REFINE: the FP32
+ * tableau of every LP).  CLUSTER: as AUTO, but an FP64 tableau above one CTA is split by
  * rows over the shared memory of a thread-block cluster of 2-16 CTAs (the
  * smallest that holds it; all CTAs take the same decisions).  SINGLE: the
  * whole batch in one persistent launch -- CTAs (512 threads for LP_PREC_FP64,
@@ -152,9 +159,10 @@ lpb_err lp_batch_create(lp_batch **out, int32_t num_lps,
  * Solve every LP of the batch on `stream` (cudaStream_t; NULL = legacy
  * default stream).  Asynchronous: returns after the kernels are enqueued.
  * Builds each tableau on the device from the uploaded A, b, c and runs
- * Steps 1-3 until every LP halts (Section 3.1).  Tableaux that fit in one
- * CTA's shared memory stay there for the whole solve; larger ones are kept
- * in a library-owned global workspace (allocated by lp_batch_create).  May be
+ * Steps 1-3 until every LP halts (Section 3.1), in shared memory or with a
+ * library-owned global workspace (allocated by lp_batch_create, at most 16 GiB,
+ * and as much again for the FP64 re-solve of LP_PREC_FP32_REFINE; at least one
+ * slot per launch group) as the plan says.  May be
  * called again (each call solves from scratch); calls on one handle must not
  * overlap on the GPU (they share the workspace).
  */
@@ -237,8 +245,8 @@ typedef struct {
                                   outgrew the first pass's 16 rows and went to the
                                   second pass (up to 32 rows)                     */
     int64_t max_smem_bytes;    /* largest shared-memory footprint of a launch        */
-    int64_t workspace_bytes;   /* global workspace of the streamed LPs (and of the
-                                  streamed FP64 re-solve of large mixed LPs)      */
+    int64_t workspace_bytes;   /* global workspace of the LPs not in shared memory (and
+                                  of the FP64 re-solve of large mixed LPs)        */
 } lp_batch_plan;
 
 /* Report the launch plan made by lp_batch_create (and, for num_fallback, the
@@ -268,9 +276,11 @@ lpb_err lp_batch_autotune(lp_batch *h, int32_t rounds, void *stream);
 /* One launch group of the plan: index 0 .. lp_batch_plan.num_groups-1 (the
  * FP64 re-solve launches of the mixed path are not listed). */
 typedef struct {
-    int32_t kind;        /* 0 mixed precision, 1 FP64 shared-memory resident, 2 FP64 streamed,
+    int32_t kind;        /* 0 mixed precision, 1 FP64 shared-memory resident, 2 FP64 with
+                            deferred updates,
                             3 FP64 on a thread-block cluster, 4 mixed precision
-                            with the FP32 tableau in a global workspace, 5 single
+                            with deferred updates (smem_bytes > 0) or the FP32
+                            tableau in a global workspace, 5 single
                             launch (LPB_SCHED_SINGLE, FP64 or mixed) */
     int32_t count;       /* LPs in the group                                  */
     int32_t threads;     /* threads per CTA                                   */

@@ -25,11 +25,11 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 COMMON = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall",
                  "-I", INCLUDE, "-I", CSRC]
 # FP64 kernels must not contract a*b+c: their arithmetic mirrors the oracle op by op.
-# Their global loads are cached in L2 only (-dlcm=cg): the streamed kernel's
-# tableau lives in global memory and is rewritten every pivot; with loads
-# cached in L1 it was observed to read stale tableau values (pivot sequences
-# differing from the shared-memory kernel's after another kernel had changed
-# the L1/shared-memory split), and L1 gives that data no reuse anyway.
+# The global loads of the kernels with a workspace slot are cached in L2 only
+# (-dlcm=cg): the slot (tableaux, and pending pivots beyond shared memory) is
+# written by some threads of a CTA and read by others while the LP is solved, and
+# L1 gives that data little reuse.  (An earlier kernel that rewrote its tableau
+# there at every pivot was observed to read stale values with loads cached in L1.)
 PER_FILE = {
     "lp_fp64_simplex.cu": ["--fmad=false", "-Xptxas", "-dlcm=cg"],
     "lp_cluster.cu": ["--fmad=false"],

@@ -823,7 +823,7 @@ static lpb_err create_batch(lp_batch** out, int32_t num_lps, const int32_t* m, c
             // FP32 tableau + FP64 certificate: in shared memory when the FP32
             // tableau fits one CTA (AUTO), else in a global workspace slot.
             // The FP64 re-solve of an uncertified LP runs in one CTA when its
-            // FP64 tableau fits, else streamed.
+            // FP64 tableau fits, else on a cluster or with deferred updates.
             if (need <= queue_smem_cap) {
                 ++h->num_fsmall;
                 h->fb_smem = std::max(h->fb_smem, need);

@@ -571,7 +571,7 @@ fp64_single_kernel(const DeviceBatch B, const Tolerances tol, const int32_t* __r
         } else if (slot) {
             deferred_large(B, tol, lp, smem, smem + SmallLayout::total, smem_bytes - SmallLayout::total, slot, diag);
         } else if (threadIdx.x == 0) {
-            record_internal_error(diag, 7, lp);  // a plan without a slot for a streamed LP
+            record_internal_error(diag, 7, lp);  // a plan without a slot for an LP that needs one
         }
         __syncthreads();
     }

@@ -268,8 +268,8 @@ struct MixedParams {
 
 // Where the mixed-precision kernels put the LPs they do not certify: an LP
 // whose FP64 tableau fits one CTA (resident_smem_bytes <= kMaxSmemPerBlock -
-// 1 KiB) is appended to q (length *len, capacity cap), any other to qbig (the
-// FP64 streamed re-solve).  The lengths are zeroed by the caller before the
+// 1 KiB) is appended to q (length *len, capacity cap), any other to qbig (re-
+// solved on a cluster or with deferred updates).  The lengths are zeroed by the caller before the
 // first mixed launch of a solve; a null queue or a full one records internal
 // error 4 and reports the LP LP_NUMERICAL.
 struct FallbackQueues {

@@ -72,8 +72,8 @@ cudaError_t mixed_kernel_prepare() {
 }
 
 // Where 16 or more one-warp CTAs share an SM, in different phases of the code,
-// they stall on instructions (40% of the time for 32 of them), and half the
-// unrolling is faster: time relative to the full one, signed / packing / phase-I
+// they wait for instructions (ncu, 32 of them, half the unrolling: 17% of a warp's
+// time), and half the unrolling is faster: time relative to the full one, signed / packing / phase-I
 // LPs, 20 x 20 (3 KB) 0.91 / 0.94 / 0.91, 40 x 40 (10 KB) 0.92 / 0.95 / 0.96, 30 x 80 (13
 // KB) 0.97 / 0.95 / 0.99, 50 x 50 (13.5 KB) 1.01 / 0.97, with phase I (to 18 KB) 1.04; 60 x
 // 60 (19 KB) 1.03 / 1.01 / 1.06, 70 x 70 (24 KB) 1.11 / 1.02 / 1.13, 88 x 88 1.14 / 1.04;

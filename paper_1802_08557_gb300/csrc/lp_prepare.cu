@@ -114,7 +114,7 @@ cudaError_t launch_plan_info(const DeviceBatch& B, int32_t num_lps, SignLook loo
 cudaError_t launch_copy_list(const CopyList& list, cudaStream_t stream) {
     size_t most = 0;
     for (int i = 0; i < list.count; ++i) most = list.bytes[i] > most ? list.bytes[i] : most;
-    // four 16-byte pieces per thread, at most two waves of CTAs
+    // four 16-byte pieces per thread, at most 8 CTAs per SM (of 152) for each array
     const size_t blocks = (most + 16383) / 16384;
     copy_list_kernel<<<dim3((unsigned)(blocks < 1 ? 1 : (blocks > 1216 ? 1216 : blocks)), list.count), 256, 0, stream>>>(
         list);
