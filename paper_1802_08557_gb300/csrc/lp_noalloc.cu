@@ -126,10 +126,12 @@ extern "C" lpb_err lp_solve_uniform_noalloc(int32_t num_lps, int32_t m, int32_t 
     // at least one workspace slot; sized for the widest phase-I tableau (every
     // row with b_i < 0: the right-hand sides are on the device), which also
     // bounds how many tableaux in shared memory share an SM: so deferred updates
-    // above 14,000 entries of that tableau, whatever its shape.  Measured, 1500 LPs
-    // of 50 x 50: 0.94 ms with the tableau in shared memory, 3.0 ms with deferred
-    // updates, 3.5 ms with the whole tableau updated in the slot.
-    const bool deferred = (int64_t)(m + 1) * ((int64_t)n + m + 1) > kDeferEntries ||
+    // above 14,000 entries of that tableau, whatever its shape, unless its rows are
+    // longer than 1024 entries (one CTA per SM either way).  Measured, 1500 LPs of 50
+    // x 50: 0.94 ms with the tableau in shared memory, 3.0 ms with deferred updates,
+    // 3.5 ms with the whole tableau updated in the slot; packing LPs of long rows, in
+    // shared memory / deferred, 1500 of 8 x 1600 1.65 / 2.13, 150 of 20 x 1100 0.47 / 0.58.
+    const bool deferred = ((int64_t)(m + 1) * ((int64_t)n + m + 1) > kDeferEntries && n + m + 1 <= 1024) ||
                           resident_smem_bytes(m, n, m) > kMaxSmemPerBlock - 1024;
     const size_t slot_bytes = deferred_slot(m, n, m).total;
     const DeferredForm form = deferred_form(m, n, m, false);
